@@ -397,7 +397,7 @@ int libraspec_accept_tree_bf16(const uint16_t* target_logits, const int32_t* dra
  * token_prob and row_stat are libraspec_confidence's conf and dstat. Logits
  * are binary32 accumulations of exact bf16 products; partials merge in
  * binary64. A token outside [-1, V) sets LIBRASPEC_ST_BAD_TOKEN (its
- * probability NaN). Reads W once per 128-row tile of H.
+ * probability NaN). Reads W once per 256-row tile of H.
  * Workspace: libraspec_lm_head_workspace_size(M, V) bytes (status word and
  * the per-tile partials).
  */

@@ -2,115 +2,180 @@
 // epilogue: logits x = H W^T (H [M, Dm] hidden states, W [V, Dm] the head,
 // bf16) are accumulated by the 5th-generation tensor cores in tensor memory
 // and reduced there to per-row (max, sum of exp, argmax, logit of one token)
-// partials per 128-column vocabulary tile, so the logits never reach HBM;
-// a second kernel merges each row's partials in binary64 (Assumption 1's
-// confidence q = softmax(x / T)[token], and the max / argmax / Z of the
-// acceptance rows, Sec. 3.1).
+// partials, so the logits never reach HBM; a second kernel merges each row's
+// partials in binary64 (Assumption 1's confidence q = softmax(x / T)[token],
+// and the max / argmax / Z of the acceptance rows, Sec. 3.1).
 //
-// Work: items = (row tile of 128, vocabulary tile of 128), vocabulary-major
-// so that CTAs running at the same time share the head's tile through L2;
-// CTA c of a grid of one CTA per SM takes items c, c + G, ... Roles (192
-// threads): warp 4 streams H and W k-slabs (64 columns, 128-byte swizzle)
-// by TMA into a ring of stages; warp 5 issues tcgen05.mma (M = 128, N =
-// 128, K = 16, fp32 accumulate) into one of two tensor-memory accumulators;
-// warps 0-3 (thread i <-> row i) read an accumulator, fold its 128 columns
-// into the row's partial and free it. Rows past M and columns past V come
-// from the TMA's zero fill and are left out of the statistics.
+// Work: CTA pairs (cta_group::2), one pair per two SMs. The vocabulary lies
+// on the MMA's M side (256 head rows over the pair, 128 per CTA) and the rows
+// of H on its N side (up to 256, split between the two CTAs), so a k-slab of
+// 64 brings 16 KB of W and N x 64 bytes of H into each CTA. At N = 256 that
+// is 64 bytes per cycle and SM at the tensor peak, which L2 sustains (1269 us
+// for 2112 rows over V = 128256, Dm = 4096: 1.75 PFLOP/s); single-CTA tiles of
+// 128 x 128 need twice the bytes and were bound by them (1920 us). The time
+// of a tile follows its operand bytes, 256 + N (N = 64: 96 us per row tile
+// of that head, 128: 103, 192: 119, 256: 141), so rows are cut into as few
+// tiles as 256 allows, of sizes that differ by 32 at most.
+//  * Several row tiles: items (vocabulary tile, row tile) with the row tile
+//    innermost, item i to pair i mod pairs: the pairs at work share the same
+//    few tiles of W through L2. One partial per (row, 128 vocabulary columns).
+//  * One row tile (M <= 256, decode: bound by the head's bytes): each pair
+//    walks its own contiguous V / pairs columns, whose last tile is cut short,
+//    so no pair streams more than its share (whole tiles of 256 leave 6.6
+//    tiles per pair, a loss of 6%); its rows' statistics stay in registers
+//    from tile to tile and leave one partial per (row, CTA).
 //
-// Decode batches have few rows (M <= 128: one row tile), and the head's
-// bytes set the time. There a stage holds only a_rows = M rounded up to 8
-// rows of H (the MMA still reads 128 rows: the rest is whatever follows in
-// shared memory, and only feeds accumulator rows that are never used), so
-// the ring has room for more stages and keeps more of W in flight per SM.
+// Roles (192 threads): warp 4 streams W and H k-slabs (128-byte swizzle) by
+// TMA into a ring of stages, each CTA its half, counted on the leader's
+// barrier; warp 5 of the leader issues tcgen05.mma into one of two
+// accumulators (lane = head column, column = row of H); warps 0-3 turn 32 x 32
+// blocks of an accumulator through shared memory, so that a thread holds one
+// row's 32 logits, reduce them, and combine the four warps' shares. Rows past
+// M and columns past V come from the TMA's zero fill (or are never loaded)
+// and are left out of the statistics.
 #include <cstdio>
 
 #include "tc.cuh"
 
 namespace libraspec {
 
-constexpr int kLmBM = 128, kLmBN = 128, kLmBK = 64, kLmMaxStages = 16;
+constexpr int kLmBK = 64, kLmMaxStages = 12;
 constexpr int kLmEpiWarps = 4, kLmProducer = 4, kLmMma = 5, kLmThreads = 6 * 32;
-constexpr uint32_t kLmATile = kLmBM * kLmBK * 2;  // 16 KB: a full H tile
-constexpr uint32_t kLmBTile = kLmBN * kLmBK * 2;  // 16 KB
+constexpr int kLmHalf = 128;                           // head rows per CTA and tile
+constexpr int kLmTile = 2 * kLmHalf;                   // head rows per tile
+constexpr int kLmRows = 256;                           // rows of H per row tile (at most)
+constexpr int kLmSub = 2;                              // k-slabs per stage (1 if Dm / 64 is odd)
+constexpr uint32_t kLmATile = kLmHalf * kLmBK * 2;     // 16 KB
 constexpr int kLmBarBytes = (2 * kLmMaxStages + 5) * 8 + 16;  // barriers and the tensor-memory slot
+constexpr int kLmTurn = kLmEpiWarps * 32 * 33 * 4;     // a padded 32 x 32 block per epilogue warp
+constexpr int kLmShares = kLmEpiWarps * kLmRows;       // the warps' (max, sum, argmax) per row
+constexpr int kLmFixed = 1024 + 1024 + kLmTurn + 3 * kLmShares * 4;  // shared memory besides the ring
 constexpr int kLmSmemMax = 227 * 1024;
-constexpr int kLmTmemCols = 2 * kLmBN;
-constexpr int kLmSub = 2;  // k-slabs per stage (fewer when Dm / 64 is not a multiple)
-constexpr uint32_t kLmIdesc = mma_idesc(kLmBM, kLmBN, 0);
-
-// Shared memory of a ring of `stages` stages of stage_bytes: barriers first,
-// then the ring at the next 1024-byte boundary, then the 16 KB the MMA may
-// read past the last stage's short H tile; plus room to align the base.
-__host__ __device__ constexpr int lm_ring_offset() { return (kLmBarBytes + 1023) / 1024 * 1024; }
-__host__ __device__ constexpr int lm_smem_bytes(int stages, int stage_bytes) {
-  return 1024 + lm_ring_offset() + stages * stage_bytes + (int)kLmATile;
-}
+static_assert(kLmBarBytes <= 1024, "barriers before the ring");
 
 struct LmPartial {
-  float m, z;  // max of the tile's logits, sum of 2^((x - m) c)
+  float m, z;  // max of the logits, sum of 2^((x - m) c)
   int arg;     // first column of the max
-  float xtok;  // the row's token logit if its column is in the tile, else NaN
+  float xtok;  // in a row's first partial: the logit of the row's token
 };
 
-__global__ void __launch_bounds__(kLmThreads, 1) lm_head_stats_kernel(
-    const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapW,
-    const float* __restrict__ temperature, int rows_per_seq, const int32_t* __restrict__ tokens, int M, int V,
-    int Dm, int m_tiles, int n_tiles, int a_rows, int stages, int sub, LmPartial* __restrict__ part,
+// How the work is cut. The vocabulary: ranges of `range` columns, each in
+// `tiles` tiles of which the last gives each CTA `tail` head rows (a multiple
+// of 8), the others 128. The rows of H: row_tiles tiles, the first n_big of
+// `big` rows (a multiple of 32, the MMA's N), the others of 32 fewer.
+struct LmCut {
+  int range, tiles, tail;
+  int row_tiles, n_big, big;
+};
+
+constexpr int kEpiBar = 1;  // named barrier of the epilogue warps
+__device__ __forceinline__ void epi_sync() {
+  asm volatile("bar.sync %0, %1;" ::"n"(kEpiBar), "n"(kLmEpiWarps * 32) : "memory");
+}
+
+// One item of a pair: head rows [v0, v0 + rows) of this CTA, rows [h0, h0 + nrow) of H, the partial's slot.
+struct LmItem {
+  int v0, rows, h0, nrow, slot;
+};
+
+__device__ __forceinline__ LmItem lm_item(int it, int pair, int pairs, int rank, const LmCut& cut) {
+  LmItem x;
+  if (cut.row_tiles == 1) {  // tile `it` of the pair's own range
+    x.rows = it == cut.tiles - 1 ? cut.tail : kLmHalf;
+    x.v0 = pair * cut.range + it * kLmTile + rank * x.rows;
+    x.h0 = 0;
+    x.nrow = cut.big;
+    x.slot = 2 * pair + rank;
+  } else {
+    const int i = pair + it * pairs, v = i / cut.row_tiles, n = i - v * cut.row_tiles;
+    x.rows = kLmHalf;
+    x.v0 = v * kLmTile + rank * kLmHalf;
+    x.h0 = n * cut.big - 32 * max(n - cut.n_big, 0);
+    x.nrow = n < cut.n_big ? cut.big : cut.big - 32;
+    x.slot = 2 * v + rank;
+  }
+  return x;
+}
+
+// mapH / mapHs: boxes of cut.big / 2 rows / 16 fewer; mapW / mapWt: boxes of 128 / cut.tail head rows.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_head_stats_kernel(
+    const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapHs,
+    const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapWt,
+    const float* __restrict__ temperature, int rows_per_seq, const int32_t* __restrict__ tokens, int M, int V, int Dm,
+    LmCut cut, int stages, int sub, int n_part, LmPartial* __restrict__ part,
     int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // a stage holds `sub` consecutive k-slabs (H slab, then W slab, each 1024-byte aligned), so every
-  // row of W is read `sub` * 128 contiguous bytes at a time
-  const uint32_t a_bytes = (uint32_t)a_rows * kLmBK * 2, slab_bytes = a_bytes + kLmBTile;
+  // a stage holds `sub` consecutive k-slabs (W slab, then H slab), so every row is read `sub` * 128 contiguous
+  // bytes at a time
+  const uint32_t slab_bytes = kLmATile + (uint32_t)cut.big * kLmBK;
   const uint32_t stage_bytes = sub * slab_bytes;
-  const uint32_t sbase = smem_u32(smem) + lm_ring_offset();
+  const uint32_t sbase = smem_u32(smem) + 1024;
   const uint32_t bFull = smem_u32(smem), bEmpty = bFull + 8 * kLmMaxStages;
   const uint32_t bAccFull = bEmpty + 8 * kLmMaxStages, bAccEmpty = bAccFull + 16, bDrain = bAccEmpty + 16;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + (2 * kLmMaxStages + 5) * 8);
+  float* turn = reinterpret_cast<float*>(smem + 1024 + stages * stage_bytes);
+  float* sh_m = turn + kLmEpiWarps * 32 * 33;
+  float* sh_z = sh_m + kLmShares;
+  int* sh_arg = reinterpret_cast<int*>(sh_z + kLmShares);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int items = m_tiles * n_tiles, nk = Dm / kLmBK / sub;  // stages per item
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  // items of this pair, stages per item
+  const int n_items = cut.row_tiles == 1 ? cut.tiles : (cut.row_tiles * cut.tiles - pair + pairs - 1) / pairs;
+  const int nk = Dm / kLmBK / sub;
+  auto item_at = [&](int it) { return lm_item(it, pair, pairs, (int)rank, cut); };
 
+  // the merge launch may start its CTAs (they wait for this grid's end)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
-      mbar_init(bFull + 8 * s, 1);   // the producer's expect_tx; bytes as transactions
-      mbar_init(bEmpty + 8 * s, 1);  // the MMA warp's commit
+      mbar_init(bFull + 8 * s, 1);   // (the leader's) its expect_tx; both CTAs' bytes as transactions
+      mbar_init(bEmpty + 8 * s, 1);  // the leader's commit
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(bAccFull + 8 * a, 1);
-      mbar_init(bAccEmpty + 8 * a, kLmEpiWarps);
+      mbar_init(bAccEmpty + 8 * a, 2 * kLmEpiWarps);  // (the leader's) both CTAs' epilogue warps
     }
     mbar_init(bDrain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kLmMma) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(const_cast<uint32_t*>(tmem_slot))),
-                 "n"(kLmTmemCols)
+                 "n"(2 * kLmRows)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // both CTAs' barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   bool ok = true;
 
   if (warp == kLmProducer) {
     if (lane == 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapH)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapW)) : "memory");
-      uint32_t it = 0;
-      for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
-        const int n = item / m_tiles, m = item - n * m_tiles;
-        for (int k = 0; k < nk; ++k, ++it) {
-          const uint32_t s = it % stages, ph = (it / stages) & 1;
+      uint32_t s = 0, ph = 0;
+      for (int it = 0; it < n_items && ok; ++it) {
+        const LmItem x = item_at(it);
+        const CUtensorMap* mh = x.nrow < cut.big ? &mapHs : &mapH;
+        const CUtensorMap* mw = x.rows < kLmHalf ? &mapWt : &mapW;
+        const int hrow = x.h0 + (int)rank * (x.nrow >> 1);
+        const uint32_t bytes = (uint32_t)(x.rows * 128 + x.nrow * kLmBK) * sub;  // this CTA's of a stage
+        for (int k = 0; k < nk; ++k) {
           if (!(ok = mbar_wait(bEmpty + 8 * s, ph ^ 1))) break;
           const uint32_t a = sbase + s * stage_bytes;
-          mbar_expect_tx(bFull + 8 * s, stage_bytes);
+          const uint32_t bar = map_rank(bFull + 8 * s, 0);
+          if (rank == 0) mbar_expect_tx(bFull + 8 * s, 2 * bytes);
           for (int j = 0; j < sub; ++j) {
             const int kc = (k * sub + j) * kLmBK;
-            tma_load_2d(a + j * slab_bytes, &mapH, bFull + 8 * s, kc, m * kLmBM);
-            tma_load_2d(a + j * slab_bytes + a_bytes, &mapW, bFull + 8 * s, kc, n * kLmBN);
+            tma_load_2d_pair(a + j * slab_bytes, mw, bar, kc, x.v0);
+            tma_load_2d_pair(a + j * slab_bytes + kLmATile, mh, bar, kc, hrow);
+          }
+          if (++s == (uint32_t)stages) {
+            s = 0;
+            ph ^= 1;
           }
         }
       }
@@ -119,126 +184,161 @@ __global__ void __launch_bounds__(kLmThreads, 1) lm_head_stats_kernel(
     __syncwarp();
   } else if (warp == kLmMma) {
     if (lane == 0) {
-      uint32_t it = 0, t = 0;
-      for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++t) {
-        const uint32_t ab = t & 1, aph = (t >> 1) & 1;
-        if (!(ok = mbar_wait(bAccEmpty + 8 * ab, aph ^ 1))) break;
-        tc_fence_after();
-        const uint32_t d = tmem + ab * kLmBN;
-        for (int k = 0; k < nk; ++k, ++it) {
-          const uint32_t s = it % stages, ph = (it / stages) & 1;
-          if (!(ok = mbar_wait(bFull + 8 * s, ph))) break;
+      if (rank == 0) {
+        uint32_t s = 0, ph = 0;
+        for (int it = 0; it < n_items && ok; ++it) {
+          const uint32_t ab = it & 1, aph = (it >> 1) & 1;
+          if (!(ok = mbar_wait(bAccEmpty + 8 * ab, aph ^ 1))) break;
           tc_fence_after();
-          for (int j = 0; j < sub; ++j) {
-            const uint32_t a = sbase + s * stage_bytes + j * slab_bytes;
+          const uint32_t idesc = mma_idesc(kLmTile, item_at(it).nrow, 0);
+          const uint32_t d = tmem + ab * kLmRows;
+          for (int k = 0; k < nk; ++k) {
+            if (!(ok = mbar_wait(bFull + 8 * s, ph))) break;
+            tc_fence_after();
+            for (int j = 0; j < sub; ++j) {
+              const uint32_t a = sbase + s * stage_bytes + j * slab_bytes;
 #pragma unroll
-            for (int kk = 0; kk < kLmBK / 16; ++kk)
-              mma_ss(d, smem_desc(a + kk * 32, 16, 1024), smem_desc(a + a_bytes + kk * 32, 16, 1024), kLmIdesc,
-                     (k | j | kk) != 0 ? 1u : 0u);
+              for (int kk = 0; kk < kLmBK / 16; ++kk)
+                mma_ss_pair(d, smem_desc(a + kk * 32, 16, 1024), smem_desc(a + kLmATile + kk * 32, 16, 1024), idesc,
+                            (k | j | kk) != 0 ? 1u : 0u);
+            }
+            mma_commit_pair(bEmpty + 8 * s);  // the stage is free, in both CTAs, once these MMAs have read it
+            if (++s == (uint32_t)stages) {
+              s = 0;
+              ph ^= 1;
+            }
           }
-          mma_commit(bEmpty + 8 * s);  // the stage is free once these MMAs have read it
+          if (ok) mma_commit_pair(bAccFull + 8 * ab);
         }
-        if (ok) mma_commit(bAccFull + 8 * ab);
+        if (!ok) raise_status(status, LIBRASPEC_ST_TIMEOUT);
+        mma_commit_pair(bDrain);
+      } else {  // item by item, so that each bounded wait covers one item
+        for (int it = 0; it < n_items && ok; ++it) ok = mbar_wait(bAccFull + 8 * (it & 1), (it >> 1) & 1);
       }
-      if (!ok) raise_status(status, LIBRASPEC_ST_TIMEOUT);
-      // every MMA issued has completed before the tensor memory is released
-      mma_commit(bDrain);
+      // every MMA has completed, and its signals have landed in both CTAs, before the tensor memory is released
       if (!mbar_wait(bDrain, 0)) raise_status(status, LIBRASPEC_ST_TIMEOUT);
     }
     __syncwarp();
   } else {
-    // ===== epilogue: thread i <-> accumulator lane i = row i of the tile =====
-    const int row = warp * 32 + lane;
+    // ===== epilogue: accumulator lane = head row v0 + warp * 32 + lane, column = row of H =====
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
-    uint32_t t = 0;
-    for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++t) {
-      const int n = item / m_tiles, m = item - n * m_tiles;
-      const uint32_t ab = t & 1, aph = (t >> 1) & 1;
+    float* tw = turn + warp * 32 * 33;
+    auto factor = [&](int grow) {  // log2(e) / T of row grow of H
+      float T = temperature ? temperature[grow / rows_per_seq] : 1.f;
+      return log2e_over(T > 0.f ? T : 1.f);
+    };
+    // one row tile: the statistics so far of rows threadIdx.x and threadIdx.x + 128
+    float run_m[2] = {-INFINITY, -INFINITY}, run_z[2] = {0.f, 0.f};
+    int run_arg[2] = {0x7fffffff, 0x7fffffff};
+    for (int it = 0; it < n_items; ++it) {
+      const LmItem x = item_at(it);
+      const uint32_t ab = it & 1, aph = (it >> 1) & 1;
+      const int vw = x.v0 + warp * 32;
+      int nvalid = min(min(32, x.rows - warp * 32), V - vw);
+      if (cut.row_tiles == 1) nvalid = min(nvalid, (pair + 1) * cut.range - vw);  // the next range's columns
       if (!(ok = warp_wait(bAccFull + 8 * ab, aph))) break;
       tc_fence_after();
-      const int grow = m * kLmBM + row;
-      const bool valid = grow < M;
-      float T = (valid && temperature) ? temperature[grow / rows_per_seq] : 1.f;
-      if (!(T > 0.f)) T = 1.f;
-      const float c = log2e_over(T);
-      const int tok = (valid && tokens) ? tokens[grow] : -1;
-      const int v0 = n * kLmBN;
-      float mrun = -INFINITY, z = 0.f, xt = __int_as_float(0x7fc00000);
-      int arg = 0x7fffffff;
 #pragma unroll 1
-      for (int ch = 0; ch < kLmBN / 32; ++ch) {
+      for (int ch = 0; ch < x.nrow / 32; ++ch) {
+        const int grow = x.h0 + ch * 32 + lane;  // this thread's row of H
+        const bool valid = grow < M;
+        const int tok = (valid && tokens) ? tokens[grow] : -1;
+        const float c = factor(valid ? grow : 0);
         uint32_t r[32];
-        tmem_ld32(tmem + lane_off + ab * kLmBN + ch * 32, r);
+        tmem_ld32(tmem + lane_off + ab * kLmRows + ch * 32, r);
         tmem_wait_ld();
-        const int vc = v0 + ch * 32, nvalid = min(32, V - vc);
+        __syncwarp();  // the last block has been read
+#pragma unroll
+        for (int i = 0; i < 32; ++i) tw[lane * 33 + i] = __uint_as_float(r[i]);
+        __syncwarp();
+        float y[32];
         float cm = -INFINITY;
         int ca = 0x7fffffff;
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
-          const float x = __uint_as_float(r[i]);
-          if (i < nvalid && x > cm) {
-            cm = x;
-            ca = vc + i;
+          y[i] = tw[i * 33 + lane];
+          if (i < nvalid && y[i] > cm) {
+            cm = y[i];
+            ca = vw + i;
           }
         }
-        if (cm > mrun) {
-          z = (mrun == -INFINITY) ? 0.f : z * ex2_approx((mrun - cm) * c);
-          mrun = cm;
-          arg = ca;
-        }
+        const float ref = cm == -INFINITY ? 0.f : cm;
         float zs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < 32; ++i)
-          if (i < nvalid) zs[i & 3] += ex2_approx((__uint_as_float(r[i]) - mrun) * c);
-        z += (zs[0] + zs[1]) + (zs[2] + zs[3]);
-        if ((unsigned)(tok - vc) < 32u) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if (i == tok - vc) xt = __uint_as_float(r[i]);
-        }
+          if (i < nvalid) zs[i & 3] += ex2_approx((y[i] - ref) * c);
+        const int at = warp * kLmRows + ch * 32 + lane;
+        sh_m[at] = cm;
+        sh_z[at] = (zs[0] + zs[1]) + (zs[2] + zs[3]);
+        sh_arg[at] = ca;
+        if (tok >= vw && tok - vw < nvalid) part[(size_t)grow * n_part].xtok = tw[(tok - vw) * 33 + lane];
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bAccEmpty + 8 * ab);
-      if (valid) {
-        LmPartial p;
-        p.m = mrun;
-        p.z = z;
-        p.arg = arg;
-        p.xtok = xt;
-        part[(size_t)grow * n_tiles + n] = p;
+      if (lane == 0) mbar_arrive_remote(map_rank(bAccEmpty + 8 * ab, 0));
+      epi_sync();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int j = threadIdx.x + h * kLmEpiWarps * 32, grow = x.h0 + j;
+        if (j >= x.nrow || grow >= M) continue;
+        const float c = factor(grow);
+        float m = run_m[h];
+        int arg = run_arg[h];
+#pragma unroll
+        for (int w = 0; w < kLmEpiWarps; ++w)  // (columns in ascending order: the first of equal maxima stays)
+          if (sh_m[w * kLmRows + j] > m) {
+            m = sh_m[w * kLmRows + j];
+            arg = sh_arg[w * kLmRows + j];
+          }
+        float z = run_m[h] == -INFINITY ? 0.f : run_z[h] * ex2_approx((run_m[h] - m) * c);
+#pragma unroll
+        for (int w = 0; w < kLmEpiWarps; ++w)
+          z += sh_z[w * kLmRows + j] * ex2_approx((sh_m[w * kLmRows + j] - m) * c);
+        if (cut.row_tiles == 1) {
+          run_m[h] = m;
+          run_z[h] = z;
+          run_arg[h] = arg;
+        }
+        if ((cut.row_tiles > 1 || it == n_items - 1) && x.slot < n_part) {
+          LmPartial* p = part + (size_t)grow * n_part + x.slot;
+          *reinterpret_cast<float2*>(p) = make_float2(m, z);
+          p->arg = arg;
+        }
       }
+      epi_sync();  // the shares are read before the next item's are written
     }
     if (!ok && lane == 0) raise_status(status, LIBRASPEC_ST_TIMEOUT);
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // neither CTA leaves while the other may still signal it
   tc_fence_after();
   if (warp == kLmMma)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kLmTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * kLmRows) : "memory");
 }
 
-// One warp per row: the row's n_tiles partials in binary64. Z = sum_n z_n
+// One warp per row (a programmatic dependent launch): the row's partials in binary64. Z = sum_n z_n
 // 2^((m_n - m) c); the argmax is the first column of the largest max (the
 // partials are in column order); the token probability is
 // 2^((x_tok - m) c) / Z.
 // A token outside [-1, V) sets LIBRASPEC_ST_BAD_TOKEN (probability NaN).
 __global__ void __launch_bounds__(128) lm_head_merge_kernel(const LmPartial* __restrict__ part, int M, int V,
-                                                            int n_tiles, const float* __restrict__ temperature,
+                                                            int n_part, const float* __restrict__ temperature,
                                                             int rows_per_seq, const int32_t* __restrict__ tokens,
                                                             float* __restrict__ row_stat,
                                                             int32_t* __restrict__ row_argmax,
                                                             float* __restrict__ token_prob, int* __restrict__ status) {
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * 4 + (threadIdx.x >> 5);
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every partial is written
   if (r >= M) return;
-  const LmPartial* p = part + (size_t)r * n_tiles;
+  const LmPartial* p = part + (size_t)r * n_part;
   float T = temperature ? temperature[r / rows_per_seq] : 1.f;
   if (!(T > 0.f)) T = 1.f;
   const double c = (double)log2e_over(T);
   float mx = -INFINITY;
   int arg = 0x7fffffff;
-  for (int n = lane; n < n_tiles; n += 32) argmax_combine(mx, arg, __ldg(&p[n].m), __ldg(&p[n].arg));
+  for (int n = lane; n < n_part; n += 32) argmax_combine(mx, arg, __ldcg(&p[n].m), __ldcg(&p[n].arg));
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const float m2 = __shfl_xor_sync(0xffffffffu, mx, off);
@@ -246,9 +346,9 @@ __global__ void __launch_bounds__(128) lm_head_merge_kernel(const LmPartial* __r
     argmax_combine(mx, arg, m2, a2);
   }
   double Z = 0.0;
-  for (int n = lane; n < n_tiles; n += 32) {
-    const float mn = __ldg(&p[n].m);
-    if (mn > -INFINITY) Z += (double)__ldg(&p[n].z) * exp2(((double)mn - (double)mx) * c);
+  for (int n = lane; n < n_part; n += 32) {
+    const float mn = __ldcg(&p[n].m);
+    if (mn > -INFINITY) Z += (double)__ldcg(&p[n].z) * exp2(((double)mn - (double)mx) * c);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, off);
@@ -264,7 +364,7 @@ __global__ void __launch_bounds__(128) lm_head_merge_kernel(const LmPartial* __r
         raise_status(status, LIBRASPEC_ST_BAD_TOKEN);
         token_prob[r] = __int_as_float(0x7fc00000);
       } else {
-        token_prob[r] = tok >= 0 ? (float)(exp2(((double)__ldg(&p[tok / kLmBN].xtok) - (double)mx) * c) / Z) : 0.f;
+        token_prob[r] = tok >= 0 ? (float)(exp2(((double)__ldcg(&p->xtok) - (double)mx) * c) / Z) : 0.f;
       }
     }
   }
@@ -272,10 +372,10 @@ __global__ void __launch_bounds__(128) lm_head_merge_kernel(const LmPartial* __r
 
 int num_sms_current();
 
-size_t lm_head_workspace_bytes(int M, int V) {
-  const size_t n_tiles = ((size_t)V + kLmBN - 1) / kLmBN;
-  return 256 + align256((size_t)M * n_tiles * sizeof(LmPartial));
-}
+// Partials per row: one per 128 columns, or one per CTA of the pairs that share the vocabulary (at least one pair).
+static int lm_parts(int V) { return std::max((V + kLmHalf - 1) / kLmHalf, 2); }
+
+size_t lm_head_workspace_bytes(int M, int V) { return 256 + align256((size_t)M * lm_parts(V) * sizeof(LmPartial)); }
 
 static bool make_2d_map(CUtensorMap* map, const void* base, int cols, int rows, int box_rows) {
   // box_rows <= 256 (TMA), a multiple of 8 (whole 1024-byte swizzle atoms)
@@ -291,27 +391,42 @@ static bool make_2d_map(CUtensorMap* map, const void* base, int cols, int rows, 
   return r == CUDA_SUCCESS;
 }
 
-// Workspace: the status word, then the partials [M, n_tiles].
+// Workspace: the status word, then the partials [M, n_part].
 cudaError_t launch_lm_head_stats(const uint16_t* H, const uint16_t* W, const float* temperature, int rows_per_seq,
                                  const int32_t* tokens, int M, int V, int Dm, float* row_stat, int32_t* row_argmax,
                                  float* token_prob, char* ws, cudaStream_t stream) {
   if (M == 0) return cudaSuccess;
-  const int m_tiles = (M + kLmBM - 1) / kLmBM, n_tiles = (V + kLmBN - 1) / kLmBN;
-  // one row tile: load only its rows (rounded up to 8), and spend the room on stages
-  const int a_rows = m_tiles == 1 ? (M + 7) / 8 * 8 : kLmBM;
-  const int slab_bytes = a_rows * kLmBK * 2 + (int)kLmBTile;
-  const int nk = Dm / kLmBK;
-  // k-slabs per stage: kLmSub, fewer while they do not divide Dm / 64 or leave under 3 stages
-  int sub = kLmSub, stages = 0;
-  for (;; sub >>= 1) {
-    stages = (kLmSmemMax - lm_smem_bytes(0, sub * slab_bytes)) / (sub * slab_bytes);
-    if (sub == 1 || (nk % sub == 0 && stages >= 3)) break;
+  const int max_pairs = std::max(num_sms_current() / 2, 1);
+  const int units = (M + 31) / 32;
+  LmCut cut;
+  cut.row_tiles = (M + kLmRows - 1) / kLmRows;
+  cut.big = (units + cut.row_tiles - 1) / cut.row_tiles * 32;
+  cut.n_big = cut.row_tiles - (cut.row_tiles * (cut.big / 32) - units);
+  int pairs, n_part;
+  if (cut.row_tiles == 1) {
+    // one range per pair, at most lm_parts(V) / 2 of them, each a multiple of 16 columns
+    pairs = std::min(max_pairs, lm_parts(V) / 2);
+    cut.range = ((V + pairs - 1) / pairs + 15) / 16 * 16;
+    pairs = (V + cut.range - 1) / cut.range;
+    cut.tiles = (cut.range + kLmTile - 1) / kLmTile;
+    cut.tail = ((cut.range - (cut.tiles - 1) * kLmTile) / 2 + 7) / 8 * 8;
+    n_part = 2 * pairs;
+  } else {
+    cut.range = V;
+    cut.tiles = (V + kLmTile - 1) / kLmTile;
+    cut.tail = kLmHalf;
+    pairs = (int)std::min<long long>((long long)cut.row_tiles * cut.tiles, max_pairs);
+    n_part = (V + kLmHalf - 1) / kLmHalf;
   }
+  const int slab_bytes = (int)kLmATile + cut.big * kLmBK;
+  const int sub = Dm / kLmBK % kLmSub == 0 ? kLmSub : 1;
   const int stage_bytes = sub * slab_bytes;
-  if (stages > kLmMaxStages) stages = kLmMaxStages;
-  const int smem = lm_smem_bytes(stages, stage_bytes);
-  CUtensorMap mapH, mapW;
-  if (!make_2d_map(&mapH, H, Dm, M, a_rows) || !make_2d_map(&mapW, W, Dm, V, kLmBN)) return cudaErrorInvalidValue;
+  const int stages = std::min((kLmSmemMax - kLmFixed) / stage_bytes, kLmMaxStages);
+  CUtensorMap mapH, mapHs, mapW, mapWt;
+  if (!make_2d_map(&mapH, H, Dm, M, cut.big / 2) ||
+      !make_2d_map(&mapHs, H, Dm, M, std::max(cut.big / 2 - 16, 16)) ||
+      !make_2d_map(&mapW, W, Dm, V, kLmHalf) || !make_2d_map(&mapWt, W, Dm, V, cut.tail))
+    return cudaErrorInvalidValue;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(lm_head_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -319,17 +434,25 @@ cudaError_t launch_lm_head_stats(const uint16_t* H, const uint16_t* W, const flo
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  const long long items = (long long)m_tiles * n_tiles;
-  const int grid = (int)(items < num_sms_current() ? items : num_sms_current());
   auto* part = reinterpret_cast<LmPartial*>(ws + 256);
   auto* status = reinterpret_cast<int*>(ws);
-  lm_head_stats_kernel<<<grid, kLmThreads, smem, stream>>>(mapH, mapW, temperature, rows_per_seq, tokens, M, V, Dm,
-                                                          m_tiles, n_tiles, a_rows, stages, sub, part, status);
+  lm_head_stats_kernel<<<2 * pairs, kLmThreads, kLmFixed + stages * stage_bytes, stream>>>(
+      mapH, mapHs, mapW, mapWt, temperature, rows_per_seq, tokens, M, V, Dm, cut, stages, sub,
+      n_part, part, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  lm_head_merge_kernel<<<(M + 3) / 4, 128, 0, stream>>>(part, M, V, n_tiles, temperature, rows_per_seq, tokens,
-                                                        row_stat, row_argmax, token_prob, status);
-  return cudaGetLastError();
+  // the merge's CTAs start beside the last tiles and wait for them
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((M + 3) / 4);
+  cfg.blockDim = dim3(128);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const LmPartial*)part, M, V, n_part, temperature,
+                            rows_per_seq, tokens, row_stat, row_argmax, token_prob, status);
 }
 
 }  // namespace libraspec

@@ -105,3 +105,22 @@ def test_lm_head_single_row_and_single_tile_vocabulary(orc):
         torch.cuda.synchronize()
         assert lr.libraspec_get_status(ws) == 0
         _check(orc, H, W, None, 1, tok.cpu().numpy(), out)
+
+
+@pytest.mark.parametrize("M,V,Dm", [(31, 130, 64), (32, 257, 192), (64, 40000, 128), (255, 300, 64), (256, 20011, 64),
+                                    (257, 129, 128), (288, 1000, 192), (513, 513, 128), (1100, 700, 64)])
+def test_lm_head_tile_edges(orc, M, V, Dm):
+    """Row tiles of 32 to 256 rows (one, and several of two sizes), vocabulary ranges with short last tiles and
+    columns past the last range, odd and even numbers of k-slabs. Tolerances as in _check: fp32 sums of Dm products."""
+    H, W = _inputs(M, V, Dm, seed=M * 31 + V + Dm)
+    rng = np.random.default_rng(M + V)
+    tok = rng.integers(-1, V, size=M).astype(np.int32)
+    tok[:2] = (0, V - 1)
+    T = torch.tensor([[0.0, 0.7, 1.3][i % 3] for i in range(M)], device=cuda())
+    ws = lr.LmHeadWorkspace(M, V)
+    for _ in range(2):  # a workspace is used again as it was left
+        out = lr.libraspec_lm_head_stats(H, W, ws, temperature=T, tokens=torch.from_numpy(tok).to(cuda()))
+    torch.cuda.synchronize()
+    assert lr.libraspec_get_status(ws) == 0
+    flag = _check(orc, H, W, T.cpu().numpy(), 1, tok, out)
+    assert flag.sum() <= max(1, M // 20)
