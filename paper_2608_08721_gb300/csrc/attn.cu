@@ -5,8 +5,9 @@
 // Work decomposition. For sequence b the verified block has M_b = (L_b+1)*g
 // query rows per kv head (g = Hq/Hkv; row r is block position t = r / g of
 // query head kvh*g + r % g) and N_b = kv_len_b + L_b + 1 visible keys. Rows
-// are cut into groups of R = g * floor(128/g) (whole block positions, at most
-// 128: one tcgen05 M=128 tile) and keys into 64-key tiles. All (row group,
+// are cut into units of RU = g * floor(128/g) (whole block positions, at most
+// 128: one tcgen05 M=128 tile), units into row groups (one unit; two where
+// (K+1)*g rows may not fit one) and keys into 64-key tiles. All (row group,
 // key tile) pairs of the batch form one tile sequence (sequence-major, then kv
 // head, row group, key tile); CTA c of the persistent grid (one CTA per SM)
 // takes the contiguous range [c*T/G, (c+1)*T/G) of it, so every CTA streams
@@ -16,20 +17,38 @@
 // plan is derived on the device from L[] and kv_len[] by every CTA, and it
 // is the same for every layer (all layers share L and kv_len).
 //
-// Roles in a CTA (192 threads):
-//  * producer warp: walks the CTA's range layer after layer in items (runs of
-//    tiles of one row group); loads the group's Q rows (one 3-D TMA box per
-//    64-column half: R/g positions x g heads) into a Q slot (two slots at
-//    d = 64; one at d = 128, whose shared memory goes to a fifth stage) and
-//    the K/V tiles (3-D TMA, 128-byte swizzle) into a ring of STAGES stages;
+// Two streams per CTA. An item (a run of tiles of one row group) is worked on
+// in steps of 128 keys by two streams, each with its own softmax warpgroup,
+// scores and O accumulator, so that one stream's MMAs run beside the other's
+// softmax. A group of one unit: tiles alternate between the streams, which
+// hold the same rows, and the epilogue combines their (O, m, l). A group of
+// two units (large trees): every tile is read once from shared memory by both
+// streams, each for its own unit. One softmax warpgroup over 64-key tiles was
+// the limit before: with few rows one warp holds them all, and its 1150
+// cycles per 64-key tile did not keep up with HBM. 8 sequences of 131072 keys
+// (64/8 heads): 771 -> 603 us (105% of the copy rate); B = 64 ragged: 327 ->
+// 294; 32 layers at B = 1: 311 -> 268; a 512-node tree, 4 layers: 369 -> 351.
+//
+// Roles in a CTA (384 threads' worth of registers, 352 threads):
+//  * producer warp: walks the CTA's range layer after layer in items; loads
+//    the group's Q rows (one 3-D TMA box per 64-column half and unit: RU/g
+//    positions x g heads) into a Q slot (two slots where groups may have two
+//    units, else one and a fifth chunk) and K and V of the tiles (3-D TMA,
+//    128-byte swizzle) into a ring of chunks (K or V of 128 keys), in the
+//    order in which the MMA warp uses them;
 //  * MMA warp: one thread issues S = Q K^T (tcgen05.mma, A and B K-major from
-//    shared memory, fp32 accumulator in tensor memory, double-buffered) and
-//    O += P V (A = P from tensor memory, B = V MN-major from shared memory),
-//    and signals completions with tcgen05.commit;
-//  * softmax warpgroup (4 warps, thread i <-> tensor-memory lane i = row i of
-//    the group): reads S, masks keys beyond kv_len_b + t, keeps the online
-//    softmax in the log2 domain, writes P (bf16) back to tensor memory, and at
-//    the end of an item normalises O and stores it (or a split partial).
+//    shared memory, fp32 accumulator in tensor memory) and O += P V (A = P
+//    from tensor memory, B = V MN-major from shared memory), and signals
+//    completions with tcgen05.commit;
+//  * softmax warpgroups (thread i <-> tensor-memory lane i = row i of the
+//    unit): read S, mask keys beyond kv_len_b + t, keep the online softmax in
+//    the log2 domain, write P (bf16) over the scores they have read, and at
+//    the end of an item normalise O and store it (or a split partial);
+//  * merge warp: merges the split groups of earlier layers.
+// Registers are what the roles' code must fit: with the merge's calls in the
+// softmax path 120 bytes of spills made every wait and epilogue wait for
+// local memory behind the K/V stream (B = 1: 361 us), so the merge is inline,
+// holds 12 loads per lane and is entered at one place.
 // The running max is only raised when a tile's max exceeds it by more than 8
 // (a factor 2^8), so O is rescaled in tensor memory rarely; p <= 2^8 keeps
 // bf16 P and fp32 O exact in range, and O / l is unchanged by the choice of
@@ -51,7 +70,7 @@
 // in CTA order (deterministic, spread over every contributing SM); the merge
 // of layer l runs beside the CTA's items of layer l+1. The last layer waits
 // for no grid barrier: a group's parts are counted in as they are written,
-// and a small group is merged whole by the CTA whose part completes it.
+// and its CTAs merge it once all are in.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -64,19 +83,44 @@
 
 namespace libraspec {
 
-constexpr int kSoftmaxWarps = 4;
-constexpr int kProducerWarp = 4;
-constexpr int kMmaWarp = 5;
-constexpr int kMergeWarp = 6;
-constexpr int kAttnThreads = 7 * 32;
-constexpr int kPBufs = 4;  // P buffers in tensor memory
+constexpr int kStreams = 2;                    // softmax warpgroups (tile streams) per CTA
+constexpr int kSoftmaxWarps = 4 * kStreams;
+constexpr int kProducerWarp = kSoftmaxWarps;
+constexpr int kMmaWarp = kSoftmaxWarps + 1;
+constexpr int kMergeWarp = kSoftmaxWarps + 2;
+constexpr int kAttnThreads = (kSoftmaxWarps + 3) * 32;
 constexpr int kMaxWaitIters = 1 << 24;
-constexpr int kSoftmaxBar = 1;  // named barrier of the softmax warpgroup
+constexpr int kSoftmaxBar = 1;  // named barrier of the softmax warpgroups
 constexpr float kRescaleLog2 = 8.f;
 constexpr int kTmemCols = 512;
 
 __device__ __forceinline__ void softmax_sync() {
   asm volatile("bar.sync %0, %1;" ::"n"(kSoftmaxBar), "n"(kSoftmaxWarps * 32) : "memory");
+}
+// Barrier of the softmax warpgroups that also tells whether any of their threads holds `pred`.
+__device__ __forceinline__ bool softmax_any(bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.aligned.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)pred), "n"(kSoftmaxBar), "n"(kSoftmaxWarps * 32)
+      : "memory");
+  return r != 0;
+}
+
+// (d0, d1) = (a0, a1) * b + c, and (d0, d1) += (a0, a1): one instruction for two elements
+__device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c) {
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmov.b64 c, {%5, %5};\n\t"
+      "fma.rn.f32x2 a, a, b, c;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "=f"(d0), "=f"(d1)
+      : "f"(a0), "f"(a1), "f"(b), "f"(c));
+}
+__device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1) {
+  asm("{\n\t.reg .b64 a, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 d, {%0, %1};\n\t"
+      "add.rn.f32x2 d, d, a;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "+f"(d0), "+f"(d1)
+      : "f"(a0), "f"(a1));
 }
 
 // bits [0, n) set (n clamped to [0, 64])
@@ -273,26 +317,24 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* ctr, uint32_t targe
 
 // One item handed from the producer to the MMA and softmax warps.
 struct ItemInfo {
-  int b, kvh, mg, rows, kv;
-  int key0, key1;     // keys [key0, key1)
-  int partial;        // 1: write a partial, else write O
-  int slot;           // partial slot
-  int grp;            // global row group index
-  int pad[6];
+  int b, kvh, mg, kv;
+  int rows0, rows1;  // rows of the group's two units of up to 128 rows
+  int key0, key1;  // keys [key0, key1)
+  int both;        // 1: stream s takes unit s, every tile; 0: one unit, tiles alternate between the streams
+  int qslot;       // Q slot of the first unit
+  int partial;     // 1: write a partial, else write O
+  int slot;        // partial slot
+  int grp;         // global row group index
+  int pad[3];
 };
+static_assert(sizeof(ItemInfo) == 64, "items lie in 64-byte slots");
 
 // A split row group this CTA helps merge (the same for every layer).
 struct MergeTask {
   int b, kvh, mg, rows, c0, np;
   int grp;  // global row group index
-  int epi;  // in the last layer, merged whole by the CTA completing it (small groups)
+  int pad;
 };
-// A split group whose merge reads at most this many (row, 4-column) items
-// over all its parts (rows x d/4 x parts) is merged, in a launch's last
-// layer, by the CTA whose part completes it, in that part's epilogue (a few
-// memory round trips, and no wait); a larger one (a long group spread over
-// many CTAs) is merged share by share by all its CTAs.
-constexpr int kEpiMaxItems = 8192;
 static_assert(2 * sizeof(MergeTask) <= 64, "two merge tasks fit their shared-memory slot");
 
 constexpr int kMaxLayers = kAttnMaxLayers;
@@ -314,42 +356,40 @@ struct LayerSet {
 };
 static_assert(sizeof(LayerSet) <= 32000, "kernel parameters are limited to 32764 bytes");
 
-template <int D, int STAGES>
+// QS Q slots: one (and room for one more K/V chunk at d = 128) where a row
+// group is always one unit, two where it may have two.
+template <int D, int QS>
 struct AttnSmem {
-  // One Q slot at d = 128 (the next item's Q then waits for this one's last
-  // S) buys a fifth K/V stage: more of the next layer's prefix streams in
-  // before the layer barrier (8b: 9.76 -> 9.40 us per layer).
-  static constexpr int kQSlots = (D == 128 && STAGES >= 5) ? 1 : 2;
   static constexpr int kBoxes = D / 64;
-  static constexpr int kTileBytes = kBoxes * 8192;       // one 64-key x D bf16 tile (per box 64 x 128 B)
-  static constexpr int kQBox = kAttnRows * 128;          // 128 rows x 64 columns
-  static constexpr int kQSlot = kBoxes * kQBox;
-  static constexpr int kQ = 0;                           // 2 slots
-  static constexpr int kK = kQ + kQSlots * kQSlot;
-  static constexpr int kV = kK + STAGES * kTileBytes;
-  // mbarriers: full[S], empty[S], qfull[2], qempty[2], sfull[2], sfree[2],
-  // pfull[4], pvdone[4], ofree[2], drain
-  static constexpr int kBar = kV + STAGES * kTileBytes;
-  static constexpr int kNumBars = 2 * STAGES + 2 * 4 + 2 * kPBufs + 2 + 1;
+  static constexpr int kChunkBytes = kBoxes * 16384;     // K or V of one 128-key tile
+  static constexpr int kChunks = D == 128 ? 6 - QS : 10;  // in the ring
+  static constexpr int kQSlot = kBoxes * 16384;          // one unit: per 64 columns 128 rows
+  static constexpr int kQ = 0;
+  static constexpr int kRing = kQ + QS * kQSlot;
+  // mbarriers: full[chunks], empty[chunks], qfull[2], qempty[2], ifull[2], iempty[2], sfull[2], pfull[2], pvdone[2],
+  // ofree, drain
+  static constexpr int kBar = kRing + kChunks * kChunkBytes;
+  static constexpr int kNumBars = 2 * kChunks + 7 * 2 + 2;
   static constexpr int kInfo = kBar + ((8 * kNumBars + 63) / 64) * 64;
   static constexpr int kTasks = kInfo + 2 * 64;
   static constexpr int kTmem = kTasks + 64;
   // [0] abort, [1] merge tasks, [2] items per layer, [3] merge chunks per
-  // layer, [4] chunks claimed, [5] chunks done, [6] the last layer's shared
-  // merges may start, [7] this item's epilogue merges its group
+  // layer, [4] chunks claimed, [5] chunks done, [6] the last layer's merges
+  // may start
   static constexpr int kMisc = kTmem + 16;
+  // (m, l) of each stream's rows, for the epilogue of an item whose streams are combined
+  static constexpr int kStat = kMisc + 48;
   // kv_len and L of up to kPlanCap sequences, read once from global memory
   // for the CTA's tile plan (a larger batch plans from global memory)
   static constexpr int kPlanCap = 1024;
-  static constexpr int kRange = kMisc + 32;  // the CTA's tile range [lo, hi)
+  static constexpr int kRange = kStat + kStreams * 128 * 8;  // the CTA's tile range [lo, hi)
   static constexpr int kPlan = kRange + 16;
   static constexpr int kBytes = kPlan + 2 * 4 * kPlanCap;
   static constexpr int kAlloc = kBytes + 1024;           // room to align the base to 1024
-  // tensor-memory columns
-  static constexpr int kColS = 0;                        // S[2]: 64 fp32 columns each
-  static constexpr int kColP = 128;                      // P[4]: 64 bf16 = 32 columns each
-  static constexpr int kColO = 256;                      // O[2]: D fp32 columns each
-  static_assert(kColP + 32 * kPBufs <= kColO && kColO + 2 * D <= kTmemCols, "tensor memory");
+  // tensor-memory columns: per stream S of a tile (128 fp32, its P as 64
+  // columns of bf16 pairs in the same place) and O (D fp32); lane = row
+  static constexpr int kColS = 0, kColO = 256;
+  static_assert(kStat % 16 == 0 && kRange % 8 == 0 && kInfo % 16 == 0, "alignment");
   static_assert(kAlloc <= 227 * 1024, "shared memory per CTA");
   // paged caches: the page of each of the CTA's tiles, after everything else
   static constexpr int kPageCap = 4096;
@@ -382,81 +422,18 @@ __device__ __forceinline__ int merge_share(const MergeTask& t, int& u0) {
 // of the launch, is always shared.
 constexpr int kMergeHelpChunks = 8;
 
-// Items per lane in a chunk of a group of np parts: J items x 16/J parts are
+constexpr int kMergeLoads = 12;  // of a lane in flight (16 spill registers in the callers)
+
+// Items per lane in a chunk of a group of np parts: J items x 12/J parts are
 // in flight per batch, and a share of `items` items costs ceil(items / 32J)
-// chunks x ceil(np / (16/J)) batches, one memory round trip each. J = 4 wins
+// chunks x ceil(np / (12/J)) batches, one memory round trip each. J = 4 wins
 // for many rows over few parts (tree and long blocks), J = 1 for one row
 // over many parts (short blocks at B = 1); ties go to J = 1 (more chunks to
 // share among helping warps).
 __device__ __forceinline__ int merge_j(int np, int items) {
-  const int trips1 = ((items + 31) / 32) * ((np + 15) / 16);
-  const int trips4 = ((items + 127) / 128) * ((np + 3) / 4);
+  const int trips1 = ((items + 31) / 32) * ((np + kMergeLoads - 1) / kMergeLoads);
+  const int trips4 = ((items + 127) / 128) * ((np + kMergeLoads / 4 - 1) / (kMergeLoads / 4));
   return trips4 < trips1 ? 4 : 1;
-}
-
-template <int J, int D>
-__device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, int lc, const float* __restrict__ part_o,
-                                            const float* __restrict__ part_ml, int K, int Hq, int g, int R,
-                                            __nv_bfloat16* __restrict__ O, float* __restrict__ lse);
-
-// The whole of group t by the softmax warpgroup (warp w of 4 takes every
-// fourth chunk), share by share with each share's chunk shape, so the result
-// has the bits the group's CTAs would each give for their share. Out of line:
-// it runs once per small split group of a launch's last layer, and keeps its
-// code out of the item loop's instruction stream.
-template <int D>
-__device__ __noinline__ void merge_group_whole(const MergeTask t, int warp, const float* __restrict__ part_o,
-                                               const float* __restrict__ part_ml, int K, int Hq, int g, int R,
-                                               __nv_bfloat16* __restrict__ O, float* __restrict__ lse) {
-  int gi = 0;
-  for (int k = 0; k < t.np; ++k) {
-    const int u0 = (int)((long long)t.rows * k / t.np);
-    const int nr = (int)((long long)t.rows * (k + 1) / t.np) - u0;
-    const int items = nr * (D / 4);
-    const int J = merge_j(t.np, items);
-    const int nc = (items + 32 * J - 1) / (32 * J);
-    for (int lc = 0; lc < nc; ++lc, ++gi) {
-      if (gi % kSoftmaxWarps != warp) continue;
-      if (J == 1) merge_chunk<1, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
-      else merge_chunk<4, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
-    }
-  }
-}
-
-// A part of a launch's last layer is written (softmax warpgroup, after its
-// epilogue). The last layer's split groups need no grid barrier: each part is
-// counted in as written (the named barrier orders the warpgroup's writes
-// before the release). A small group is merged at once, whole, by the CTA
-// whose part completes it (the acquire makes the other parts visible), share
-// by share as its CTAs would merge it, so the result is the same bits; a
-// larger one by the merge warps of all its CTAs once its count is complete.
-// Out of line, like merge_group_whole: it runs once per split part of the
-// last layer.
-template <int D>
-__device__ __noinline__ void last_layer_part_done(const MergeTask* tasks, int n_tasks, int grp,
-                                                  uint32_t* __restrict__ grp_cnt, volatile int* misc,
-                                                  const float* __restrict__ part_o, const float* __restrict__ part_ml,
-                                                  int K, int Hq, int g, int R, __nv_bfloat16* __restrict__ O,
-                                                  float* __restrict__ lse) {
-  const int tid = threadIdx.x, warp = tid >> 5;
-  int ti = 0;
-  while (ti + 1 < n_tasks && tasks[ti].grp != grp) ++ti;
-  const MergeTask t = tasks[ti];
-  softmax_sync();
-  if (tid == 0) {
-    bool last = false;
-    if (t.epi) {
-      uint32_t old;
-      asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(grp_cnt + 2 * grp), "r"(1u) : "memory");
-      last = old == (uint32_t)t.np - 1;
-      if (last) grp_cnt[2 * grp] = 0u;  // every part is in: ready for the next launch
-    } else {
-      asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(grp_cnt + 2 * grp), "r"(1u) : "memory");
-    }
-    misc[7] = last ? 1 : 0;
-  }
-  softmax_sync();
-  if (misc[7]) merge_group_whole<D>(t, warp, part_o, part_ml, K, Hq, g, R, O, lse);
 }
 
 template <int D>
@@ -474,9 +451,9 @@ __device__ __forceinline__ int merge_chunk_count(const MergeTask* tasks, int n_t
 // Chunk lc of task t: items (lc*J + j)*32 + lane, j < J.
 template <int J, int D>
 __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, int lc, const float* __restrict__ part_o,
-                                            const float* __restrict__ part_ml, int K, int Hq, int g, int R,
+                                            const float* __restrict__ part_ml, int K, int Hq, int g, int R, int slot_rows,
                                             __nv_bfloat16* __restrict__ O, float* __restrict__ lse) {
-  constexpr int PB = 16 / J, C4 = D / 4;
+  constexpr int PB = kMergeLoads / J, C4 = D / 4;
   const int lane = threadIdx.x & 31;
   const int np = t.np, c0 = t.c0, items = nr * C4;
   float M[J], Ls[J];
@@ -498,7 +475,7 @@ __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, 
       for (int k = 0; k < PB; ++k) {
         const int p = p0 + k;
         if (i < items && p < np) {
-          const size_t at = (size_t)(p == 0 ? 2 * c0 + 1 : 2 * (c0 + p)) * kAttnRows + u0 + r;
+          const size_t at = (size_t)(p == 0 ? 2 * c0 + 1 : 2 * (c0 + p)) * slot_rows + u0 + r;
           ml[j][k] = __ldcg(reinterpret_cast<const float2*>(part_ml + at * 2));
           v[j][k] = __ldcg(reinterpret_cast<const float4*>(part_o + at * D) + c);
         } else {
@@ -552,10 +529,10 @@ __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, 
 // oldest first. Chunks are numbered [l * C, (l + 1) * C) for layer l on the
 // CTA's monotonic counters; ctr_done counts the chunks merged (stores done).
 template <int D>
-__device__ void merge_chunks(int last_layer, const LayerSet& set, const MergeTask* tasks, int n_tasks, int C,
-                             int* ctr_claim, int* ctr_done, int K, int Hq, int Hkv, int R,
+__device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set, const MergeTask* tasks, int n_tasks, int C,
+                             int* ctr_claim, int* ctr_done, int K, int Hq, int Hkv, int R, int slot_rows,
                              const float* __restrict__ part_buf_o, const float* __restrict__ part_buf_ml,
-                             size_t part_o_stride, size_t part_ml_stride, int epi_layer) {
+                             size_t part_o_stride, size_t part_ml_stride) {
   const int lane = threadIdx.x & 31;
   const int g = Hq / Hkv;
   const int hi = (last_layer + 1) * C;
@@ -585,10 +562,10 @@ __device__ void merge_chunks(int last_layer, const LayerSet& set, const MergeTas
       if (lc < nc) break;
       lc -= nc;
     }
-    if (ti < n_tasks && !(layer == epi_layer && tasks[ti].epi)) {  // (an epilogue merge: counted, no work)
+    if (ti < n_tasks) {
       const MergeTask& t = tasks[ti];
-      if (merge_j(t.np, nr * (D / 4)) == 1) merge_chunk<1, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
-      else merge_chunk<4, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
+      if (merge_j(t.np, nr * (D / 4)) == 1) merge_chunk<1, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, slot_rows, O, lse);
+      else merge_chunk<4, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, slot_rows, O, lse);
     }
     __syncwarp();
     if (lane == 0) atomicAdd(ctr_done, 1);
@@ -602,31 +579,31 @@ __device__ void merge_chunks(int last_layer, const LayerSet& set, const MergeTas
 // tree_vis (optional, [B, K+1, tree_words]): the block is a draft tree and
 // row t sees the block keys of the set bits (bit j <-> block position j + 1)
 // besides the root and the prefix; nullptr: the chain draft (block-causal).
-template <int D, int STAGES, bool PAGED, bool WEIGHTED>
+template <int D, int QS, bool PAGED, bool WEIGHTED>
 __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     const __grid_constant__ LayerSet set, const int32_t* __restrict__ kv_len, const int32_t* __restrict__ Ls,
     const uint64_t* __restrict__ tree_vis, int tree_words,
     const int32_t* __restrict__ block_table, int max_pages, int page_size, int n_pages, int page_cache,
-    int B, int K, int Hq, int Hkv, int S_cap, float scale_log2, int min_tiles, int item_tiles,
+    int B, int K, int Hq, int Hkv, int S_cap, float scale_log2, int min_tiles, int item_tiles, int slot_rows,
     float* __restrict__ part_buf_o,
     float* __restrict__ part_buf_ml, size_t part_o_stride, size_t part_ml_stride, uint32_t* __restrict__ bar_cnt,
     uint32_t* __restrict__ grp_cnt, int* __restrict__ status) {
-  using SM = AttnSmem<D, STAGES>;
+  using SM = AttnSmem<D, QS>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sQ = smem_u32(smem + SM::kQ);
-  const uint32_t sK = smem_u32(smem + SM::kK);
-  const uint32_t sV = smem_u32(smem + SM::kV);
+  const uint32_t sRing = smem_u32(smem + SM::kRing);
   const uint32_t bFull = smem_u32(smem + SM::kBar);
-  const uint32_t bEmpty = bFull + 8 * STAGES;
-  const uint32_t bQFull = bEmpty + 8 * STAGES;
+  const uint32_t bEmpty = bFull + 8 * SM::kChunks;
+  const uint32_t bQFull = bEmpty + 8 * SM::kChunks;
   const uint32_t bQEmpty = bQFull + 16;
-  const uint32_t bSFull = bQEmpty + 16;
-  const uint32_t bSFree = bSFull + 16;
-  const uint32_t bPFull = bSFree + 16;
-  const uint32_t bPVDone = bPFull + 8 * kPBufs;
-  const uint32_t bOFree = bPVDone + 8 * kPBufs;
-  const uint32_t bDrain = bOFree + 16;
+  const uint32_t bIFull = bQEmpty + 16;
+  const uint32_t bIEmpty = bIFull + 16;
+  const uint32_t bSFull = bIEmpty + 16;   // [stream]
+  const uint32_t bPFull = bSFull + 16;    // [stream]
+  const uint32_t bPVDone = bPFull + 16;   // [stream]
+  const uint32_t bOFree = bPVDone + 16;
+  const uint32_t bDrain = bOFree + 8;
   ItemInfo* info = reinterpret_cast<ItemInfo*>(smem + SM::kInfo);
   MergeTask* tasks = reinterpret_cast<MergeTask*>(smem + SM::kTasks);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + SM::kTmem);
@@ -635,7 +612,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = Hq / Hkv;
-  const int R = g * (kAttnRows / g);  // rows per group: whole block positions
+  const int RU = attn_unit_rows(g), R = QS * RU;  // rows per unit and per row group
   const int n_layers = set.n;
   const uint32_t n_ctas = gridDim.x;
   // the tensor maps' first use then finds them on chip
@@ -653,21 +630,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
   const int32_t* Lss = plan_cached ? plan_L : Ls;
 
   if (tid == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < SM::kChunks; ++s) {
       mbar_init(bFull + 8 * s, 1);
-      mbar_init(bEmpty + 8 * s, 1);  // the MMA warp's commit after the tile's PV
+      mbar_init(bEmpty + 8 * s, 1);  // the MMA warp's commit after the chunk's last use
     }
     for (int q = 0; q < 2; ++q) {
       mbar_init(bQFull + 8 * q, 1);                   // the producer's arrive; Q bytes as transactions
-      mbar_init(bQEmpty + 8 * q, 1 + kSoftmaxWarps);  // MMA commit (Q read) + softmax warps (info read)
+      mbar_init(bQEmpty + 8 * q, 1);                  // the MMA warp's commit after the item's last S
+      mbar_init(bIFull + 8 * q, 1);
+      mbar_init(bIEmpty + 8 * q, 1 + kSoftmaxWarps);  // the item has been read
+      mbar_init(bPFull + 8 * q, 4);
+      mbar_init(bPVDone + 8 * q, 1);
       mbar_init(bSFull + 8 * q, 1);
-      mbar_init(bSFree + 8 * q, kSoftmaxWarps);
-      mbar_init(bOFree + 8 * q, kSoftmaxWarps);
     }
-    for (int p = 0; p < kPBufs; ++p) {
-      mbar_init(bPFull + 8 * p, kSoftmaxWarps);
-      mbar_init(bPVDone + 8 * p, 1);
-    }
+    mbar_init(bOFree, kSoftmaxWarps);
     mbar_init(bDrain, 1);
     misc[0] = 0;
     misc[4] = 0;
@@ -755,7 +731,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             t.c0 = cta_of(weighted_pos(gstart, group, C), W, G);
             t.np = cta_of(weighted_pos(gend - 1, group, C), W, G) - t.c0 + 1;
             t.grp = group;
-            t.epi = (long long)t.rows * (D / 4) * t.np <= kEpiMaxItems ? 1 : 0;
             tasks[n_tasks] = t;
           }
           ++n_tasks;
@@ -809,7 +784,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     const int c = blockIdx.x;
     const long long lo = reinterpret_cast<const long long*>(smem + SM::kRange)[0];
     const long long hi = reinterpret_cast<const long long*>(smem + SM::kRange)[1];
-    uint32_t item_ctr = 0, tile_ctr = 0;
     // lane 0 reads the abort flag for the whole warp (the loop body has warp-wide steps)
     auto aborted = [&]() { return __shfl_sync(0xffffffffu, misc[0], 0) != 0; };
     // paged: the page of every tile of the range, read once for all layers
@@ -838,6 +812,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       }
       __syncwarp();
     }
+    uint32_t item_ctr = 0, chunk_ctr = 0;           // items; chunks filled
+    uint32_t q_loads = 0, q_any = 0;                // bit q: parity of the units loaded into Q slot q; any loaded
+    int q_next = 0, q_last = -1;                    // next slot of a one-unit item; a slot of the last item
+    // the next chunk may be filled
+    auto chunk_free = [&]() { return bEmpty + 8 * (chunk_ctr % SM::kChunks); };
+    auto chunk_parity = [&]() { return ((chunk_ctr / SM::kChunks) & 1) ^ 1; };
+    // Q slot q's last unit has been read
+    auto q_parity = [&](int q) { return ((q_loads >> q) & 1u) ^ 1u; };
     for (int layer = 0; layer < n_layers && !aborted(); ++layer) {
       // layer's dependent data (Q, the block's keys) is readable once every
       // CTA has finished the previous layer
@@ -853,91 +835,120 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         it.b = loc.b;
         it.kvh = gib / loc.p.n_mg;
         it.mg = gib % loc.p.n_mg;
-        it.rows = min(R, loc.p.M - it.mg * R);
+        const int rows = min(R, loc.p.M - it.mg * R);
+        it.rows0 = min(rows, RU);
+        it.rows1 = rows - it.rows0;
+        it.both = it.rows1 > 0;
         it.kv = kvs[loc.b];
         it.key0 = (int)(pos - gstart) * kAttnTileKeys;
         it.key1 = min(loc.p.N, (int)(iend - gstart) * kAttnTileKeys);
         it.partial = ((pos == gstart) && (gend <= hi)) ? 0 : 1;
         it.slot = (pos == gstart) ? 2 * c + 1 : 2 * c;
         it.grp = loc.group0 + gib;
-        const int n_tiles = (int)(iend - pos);
+        it.qslot = it.both || QS == 1 ? 0 : q_next;
+        const int n_half = (int)(iend - pos), n_tiles = (n_half + 1) >> 1;
         const int zc = loc.b * Hkv + it.kvh;
-        const long long item_pos = pos;  // the item's first tile in the tile sequence
+        const long long item_pos = pos;  // the item's first 64-key tile in the tile sequence
         pos = iend;
-        const uint32_t q = item_ctr % SM::kQSlots;
         if (lane == 0) {
-          bool ok = true;
-          int issued = 0;
-          auto issue_tile = [&](int i) {
-            const uint32_t s = tile_ctr % STAGES;
-            const uint32_t bar = bFull + 8 * s;
-            mbar_expect_tx(bar, 2 * SM::kTileBytes);
-            int y = it.key0 + i * kAttnTileKeys, z = zc;
+          // The ring is filled in the order in which the MMA warp uses it: K of
+          // tile t, then V of tile t - lag.
+          const int lag = it.both ? 1 : 2;
+          int kt = 0, vt = 0;  // the next K and V tile
+          auto next_is_k = [&]() { return kt < n_tiles && kt < vt + lag; };
+          auto key_tile = [&](int key_half, int& y, int& z) {  // TMA row and plane of the item's 64-key tile
+            y = it.key0 + key_half * kAttnTileKeys;
+            z = zc;
             if (PAGED) {
-              const int page = pages_cached ? tile_page[item_pos - lo + i] : page_of(it.b, y);
+              const int page = pages_cached ? tile_page[item_pos - lo + key_half] : page_of(it.b, y);
               z = page * Hkv + it.kvh;
               y %= page_size;
             }
-#pragma unroll
-            for (int bx = 0; bx < SM::kBoxes; ++bx) {
-              tma_load_3d(sK + s * SM::kTileBytes + bx * 8192, &set.K[layer], bar, bx * 64, y, z);
-              tma_load_3d(sV + s * SM::kTileBytes + bx * 8192, &set.V[layer], bar, bx * 64, y, z);
-            }
-            ++tile_ctr;
           };
-          // Tiles go out as their stages free, before the item's Q slot is
-          // free (the previous item's last S), so the ring does not drain
-          // between items; before the layer barrier only tiles that lie
-          // wholly in the cache prefix (the block's keys are the previous
-          // layer's output).
-          // (a free Q slot at once: Q goes first, the item's first S needs it)
+          auto fill_chunk = [&]() {
+            const uint32_t ch = chunk_ctr % SM::kChunks;
+            const uint32_t bar = bFull + 8 * ch, dst = sRing + ch * SM::kChunkBytes;
+            const bool is_k = next_is_k();
+            const int tt = is_k ? kt++ : vt++, nh = min(2, n_half - 2 * tt);
+            mbar_expect_tx(bar, nh * SM::kBoxes * 8192);
+            for (int h = 0; h < nh; ++h) {
+              int y, z;
+              key_tile(2 * tt + h, y, z);
+              // K: per 64 dims 128 keys; V: per 64 keys all dims (boxes of 64 keys x 64 dims)
+#pragma unroll
+              for (int hb = 0; hb < SM::kBoxes; ++hb) {
+                if (is_k) tma_load_3d(dst + hb * 16384 + h * 8192, &set.K[layer], bar, hb * 64, y, z);
+                else tma_load_3d(dst + (h * SM::kBoxes + hb) * 8192, &set.V[layer], bar, hb * 64, y, z);
+              }
+            }
+            ++chunk_ctr;
+          };
+          auto q_box = [&](int u, int& yh, int& zt) {  // heads and positions of unit u
+            const int rr = it.mg * R + u * RU;
+            zt = it.b * (K + 1) + rr / g;
+            yh = it.kvh * g + rr % g;
+          };
+          // Chunks are filled as they free, before the item's Q slot is free
+          // (an earlier item's last S), so the ring does not drain between
+          // items; before the layer barrier only tiles that lie wholly in
+          // the cache prefix (the block's keys are the previous layer's
+          // output).
           if (!ready) {
             // Q is read once the layer barrier passes; bring it into L2 now
-#pragma unroll
-            for (int hb = 0; hb < SM::kBoxes; ++hb)
-              tma_prefetch_3d(&set.Q[layer], hb * 64, it.kvh * g, it.b * (K + 1) + it.mg * (R / g));
+            for (int u = 0; u <= it.both; ++u) {
+              int yh, zt;
+              q_box(u, yh, zt);
+              for (int hb = 0; hb < SM::kBoxes; ++hb) tma_prefetch_3d(&set.Q[layer], hb * 64, yh, zt);
+            }
           }
-          int n_pre = ready ? n_tiles : min(n_tiles, max(0, (it.kv - it.key0) / kAttnTileKeys));
+          bool ok = true, q_done = false;
           // a layer's first item: its prefix tiles go out once the previous
           // layer's last S has read its Q slot (earlier copies only slow the
           // previous layer, whose barrier this layer waits for)
-          bool q_free = !ready && mbar_wait(bQEmpty + 8 * q, ((item_ctr / SM::kQSlots) & 1) ^ 1);
-          for (int spin = 0;; ++spin) {
-            if (!q_free) q_free = mbar_test_wait(bQEmpty + 8 * q, ((item_ctr / SM::kQSlots) & 1) ^ 1);
-            if (ready && q_free) break;
-            while (issued < n_pre &&
-                   mbar_test_wait(bEmpty + 8 * (tile_ctr % STAGES), ((tile_ctr / STAGES) & 1) ^ 1)) {
-              issue_tile(issued);
-              ++issued;
+          if (!ready && q_last >= 0) ok = mbar_wait(bQEmpty + 8 * q_last, q_parity(q_last));
+          for (int spin = 0; ok && !q_done; ++spin) {
+            if (ready && mbar_test_wait(bIEmpty + 8 * (item_ctr & 1), ((item_ctr >> 1) & 1) ^ 1) &&
+                mbar_test_wait(bQEmpty + 8 * it.qslot, q_parity(it.qslot)) &&
+                (!it.both || mbar_test_wait(bQEmpty + 8, q_parity(1)))) {
+              info[item_ctr & 1] = it;
+              mbar_arrive(bIFull + 8 * (item_ctr & 1));
+              for (int u = 0; u <= it.both; ++u) {
+                // Q: RU/g positions x g heads of kv head kvh, one box per 64-column half
+                const int qs = it.both ? u : it.qslot;
+                int yh, zt;
+                q_box(u, yh, zt);
+                mbar_expect_tx(bQFull + 8 * qs, (uint32_t)RU * D * 2);
+                for (int hb = 0; hb < SM::kBoxes; ++hb)
+                  tma_load_3d(sQ + qs * SM::kQSlot + hb * 16384, &set.Q[layer], bQFull + 8 * qs, hb * 64, yh, zt);
+                q_loads ^= 1u << qs;
+                q_any |= 1u << qs;
+                q_last = qs;
+              }
+              q_next = QS == 1 ? 0 : q_last ^ 1;
+              q_done = true;
+              break;
+            }
+            while (vt < n_tiles) {
+              // the chunk's last key lies before the block
+              const int tt = next_is_k() ? kt : vt;
+              if (!ready && it.key0 + min(2 * tt + 2, n_half) * kAttnTileKeys > it.kv) break;
+              if (!mbar_test_wait(chunk_free(), chunk_parity())) break;
+              fill_chunk();
             }
             if (!ready) {
               uint32_t v;
               asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar_cnt + (layer - 1)) : "memory");
               if (v >= n_ctas) {
                 ready = true;
-                n_pre = n_tiles;
                 continue;
               }
             }
-            if (spin >= kMaxWaitIters) {
-              ok = false;
-              break;
-            }
-            __nanosleep(32);
+            if (spin >= kMaxWaitIters) ok = false;
+            else __nanosleep(32);
           }
-          if (ok) {
-            // Q: R/g positions x g heads of kv head kvh, one box per 64-column half
-            info[q] = it;
-            mbar_expect_tx(bQFull + 8 * q, (uint32_t)R * D * 2);
-            const uint32_t qdst = sQ + q * SM::kQSlot;
-#pragma unroll
-            for (int hb = 0; hb < SM::kBoxes; ++hb)
-              tma_load_3d(qdst + hb * SM::kQBox, &set.Q[layer], bQFull + 8 * q, hb * 64, it.kvh * g,
-                          it.b * (K + 1) + it.mg * (R / g));
-            for (int i = issued; i < n_tiles && ok; ++i) {
-              ok = mbar_wait(bEmpty + 8 * (tile_ctr % STAGES), ((tile_ctr / STAGES) & 1) ^ 1);
-              if (ok) issue_tile(i);
-            }
+          while (ok && vt < n_tiles) {
+            ok = mbar_wait(chunk_free(), chunk_parity());
+            if (ok) fill_chunk();
           }
           if (!ok) {
             raise_status(status, LIBRASPEC_ST_TIMEOUT);
@@ -946,71 +957,83 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         }
         ready = true;
         ++item_ctr;
-        __syncwarp();
+        q_next = __shfl_sync(0xffffffffu, q_next, 0);
       }
     }
     // before leaving, wait (bounded) for this CTA's copies still in flight
     if (lane == 0) {
-      for (uint32_t k = 0; k < STAGES && k < tile_ctr; ++k) {
-        const uint32_t t = tile_ctr - 1 - k;
-        mbar_wait(bFull + 8 * (t % STAGES), (t / STAGES) & 1);
+      for (uint32_t k = 0; k < (uint32_t)SM::kChunks && k < chunk_ctr; ++k) {
+        const uint32_t i = chunk_ctr - 1 - k;
+        mbar_wait(bFull + 8 * (i % SM::kChunks), (i / SM::kChunks) & 1);
       }
-      for (uint32_t k = 0; k < (uint32_t)SM::kQSlots && k < item_ctr; ++k) {
-        const uint32_t i = item_ctr - 1 - k;
-        mbar_wait(bQFull + 8 * (i % SM::kQSlots), (i / SM::kQSlots) & 1);
-      }
+      for (int q = 0; q < 2; ++q)
+        if ((q_any >> q) & 1u) mbar_wait(bQFull + 8 * q, q_parity(q));
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ======================= MMA issue =======================
     if (lane == 0) {
-      constexpr uint32_t kIdescS = mma_idesc(128, kAttnTileKeys, 0);
-      constexpr uint32_t kIdescPV = mma_idesc(128, D, 1);
-      uint32_t item_ctr = 0, tile_ctr = 0;
+      uint32_t item_ctr = 0, chunk_ctr = 0;
+      uint32_t q_uses = 0, p_par = 0;  // bit q: parity of the units read from Q slot q; bit s: of P steps of stream s
       bool ok = true;
-      // O[ob] += P(gt) V(gt); the first PV of an item overwrites O
-      auto issue_pv = [&](uint32_t gt, uint32_t item, bool first) {
-        const uint32_t pb = gt % kPBufs, s = gt % STAGES, ob = item & 1;
-        ok = ok && mbar_spin(bPFull + 8 * pb, (gt / kPBufs) & 1);
-        if (first) ok = ok && mbar_spin(bOFree + 8 * ob, ((item >> 1) & 1) ^ 1);
-        if (!ok) return;
-        tc_fence_after();
-        const uint32_t vtile = sV + s * SM::kTileBytes;
-#pragma unroll
-        for (int kc = 0; kc < kAttnTileKeys / 16; ++kc)
-          mma_ts(tmem + SM::kColO + ob * D, tmem + SM::kColP + pb * 32 + kc * 8,
-                 smem_desc(vtile + kc * 2048, 8192, 1024), kIdescPV, (!first || kc > 0) ? 1u : 0u);
-        mma_commit(bPVDone + 8 * pb);
-        mma_commit(bEmpty + 8 * s);
+      auto take = [&]() {  // the next chunk, once it is filled
+        const uint32_t ch = chunk_ctr % SM::kChunks;
+        ok = ok && mbar_spin(bFull + 8 * ch, (chunk_ctr / SM::kChunks) & 1);
+        ++chunk_ctr;
+        return ch;
       };
       for (int layer = 0; layer < n_layers && ok; ++layer) {
-        for (int item = 0; item < n_items && ok; ++item) {
-          const uint32_t q = item_ctr % SM::kQSlots;
-          ok = mbar_spin(bQFull + 8 * q, (item_ctr / SM::kQSlots) & 1);
+        for (int item = 0; item < n_items && ok; ++item, ++item_ctr) {
+          ok = mbar_spin(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
           if (!ok) break;
-          const ItemInfo it = info[q];
-          const int n_tiles = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys;
-          const uint32_t qslot = sQ + q * SM::kQSlot;
-          for (int t = 0; t < n_tiles && ok; ++t) {
-            const uint32_t gt = tile_ctr;
-            const uint32_t s = gt % STAGES, sb = gt & 1;
-            ok = mbar_spin(bFull + 8 * s, (gt / STAGES) & 1) && mbar_spin(bSFree + 8 * sb, ((gt >> 1) & 1) ^ 1);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t ktile = sK + s * SM::kTileBytes;
+          const ItemInfo it = info[item_ctr & 1];
+          mbar_arrive(bIEmpty + 8 * (item_ctr & 1));
+          const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
+          const uint32_t ob = item_ctr & 1;
+          // Step j: one unit: tile j of stream j & 1; two units: tile j >> 1
+          // of unit (and stream) j & 1. S of a step goes where P of the
+          // stream's last step lies, so its PV is issued first.
+          const int n_steps = it.both ? 2 * n_tiles : n_tiles;
+          uint32_t kch = 0, vch = 0;
+          for (int j = 0; j < n_steps + 2 && ok; ++j) {
+            const int st = j & 1;
+            const uint32_t ts = tmem + SM::kColS + st * 128;
+            if (j >= 2) {  // O += P V of step j - 2
+              const int i = it.both ? (j - 2) >> 1 : j - 2, nh = min(2, n_half - 2 * i);
+              if (!it.both || st == 0) vch = take();
+              ok = ok && mbar_spin(bPFull + 8 * st, (p_par >> st) & 1u);
+              p_par ^= 1u << st;
+              if (j == 2) ok = ok && mbar_spin(bOFree, (item_ctr & 1) ^ 1);
+              if (!ok) break;
+              tc_fence_after();
+              constexpr uint32_t idesc = mma_idesc(128, D, 1);
+              const uint32_t va = desc_lo(sRing + vch * SM::kChunkBytes, 8192);
+              const uint32_t d = tmem + SM::kColO + st * 128;
+              mma_ts4<2048>(d, ts, va, idesc, j < 4 ? 0u : 1u);
+              if (nh == 2) mma_ts4<2048>(d, ts + 32, va + SM::kBoxes * 512, idesc, 1u);
+              mma_commit(bPVDone + 8 * st);
+              if (!it.both || st == 1) mma_commit(bEmpty + 8 * vch);
+            }
+            if (j < n_steps) {  // S = Q K^T of step j: the unit's rows x up to 128 keys
+              const int i = it.both ? j >> 1 : j, nh = min(2, n_half - 2 * i);
+              const int qs = it.both ? st : it.qslot;
+              if (!it.both || st == 0) kch = take();
+              if (j <= it.both) {
+                ok = ok && mbar_spin(bQFull + 8 * qs, (q_uses >> qs) & 1u);
+                q_uses ^= 1u << qs;
+              }
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t idesc = mma_idesc(128, 64 * nh, 0);
+              const uint32_t qa = desc_lo(sQ + qs * SM::kQSlot, 16), ka = desc_lo(sRing + kch * SM::kChunkBytes, 16);
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk)
-              mma_ss(tmem + SM::kColS + sb * kAttnTileKeys,
-                     smem_desc(qslot + (kk >> 2) * SM::kQBox + (kk & 3) * 32, 16, 1024),
-                     smem_desc(ktile + (kk >> 2) * 8192 + (kk & 3) * 32, 16, 1024), kIdescS, kk > 0 ? 1u : 0u);
-            mma_commit(bSFull + 8 * sb);
-            if (t == n_tiles - 1) mma_commit(bQEmpty + 8 * q);
-            // the previous tile's PV overlaps this tile's softmax
-            if (t > 0) issue_pv(gt - 1, item_ctr, t == 1);
-            ++tile_ctr;
+              for (int hb = 0; hb < SM::kBoxes; ++hb)
+                mma_ss4<32, 32>(ts, qa + hb * 1024, ka + hb * 1024, idesc, hb != 0 ? 1u : 0u);
+              mma_commit(bSFull + 8 * st);
+              if (!it.both || st == 1) mma_commit(bEmpty + 8 * kch);
+              if (j >= n_steps - 1 - it.both) mma_commit(bQEmpty + 8 * qs);
+            }
           }
-          if (ok && n_tiles > 0) issue_pv(tile_ctr - 1, item_ctr, n_tiles == 1);
-          ++item_ctr;
         }
       }
       if (!ok) {
@@ -1023,202 +1046,256 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     }
     __syncwarp();
   } else if (warp < kSoftmaxWarps) {
-    // ======================= softmax warpgroup =======================
-    const int row = warp * 32 + lane;  // tensor-memory lane
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
-    uint32_t item_ctr = 0, tile_ctr = 0;
+    // ======================= softmax warpgroups =======================
+    const int st = warp >> 2, wq = warp & 3;       // stream; quarter of the tensor-memory lanes
+    const int row = wq * 32 + lane;                // tensor-memory lane: the unit's row
+    const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
+    const uint32_t ts = tmem + lane_off + SM::kColS + st * 128;
+    float2* stat = reinterpret_cast<float2*>(smem + SM::kStat);  // [stream][128]
+    uint32_t item_ctr = 0, done0 = 0, done1 = 0;   // steps of streams 0 and 1 in the items before this one
     bool ok = true;
+    // A wait that fails leaves `ok` false; the item is then finished without
+    // further waits, so that every thread still reaches every named barrier.
+    auto wait = [&](uint32_t bar, uint32_t parity) { ok = ok && warp_wait(bar, parity); };
     // layer n_layers has no items: it only helps with the last layer's merge
-    for (int layer = 0; layer <= n_layers && ok; ++layer) {
+    for (int layer = 0; layer <= n_layers; ++layer) {
       const bool has_items = layer < n_layers;
       float* part_o = part_buf_o + (layer % kAttnPartBufs) * part_o_stride;
       float* part_ml = part_buf_ml + (layer % kAttnPartBufs) * part_ml_stride;
       if (layer > 0 && has_items) {
         // layer's inputs are ready once every CTA is done with the previous layer
-        if (tid == 0 && !wait_counter(bar_cnt + (layer - 1), n_ctas)) {
-          raise_status(status, LIBRASPEC_ST_TIMEOUT);
-          misc[0] = 1;
-        }
-        softmax_sync();
-        if (misc[0]) {
+        if (tid == 0 && !wait_counter(bar_cnt + (layer - 1), n_ctas)) ok = false;
+        if (softmax_any(!ok)) {
           ok = false;
           break;
         }
       }
       __nv_bfloat16* O = has_items ? set.p[layer].O : nullptr;
       float* lse = has_items ? set.p[layer].lse : nullptr;
-      for (int item = 0; item < n_items && ok && has_items; ++item) {
-        const uint32_t q = item_ctr % SM::kQSlots, ob = item_ctr & 1;
-        ok = warp_wait(bQFull + 8 * q, (item_ctr / SM::kQSlots) & 1);
-        if (!ok) break;
-        const ItemInfo it = info[q];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bQEmpty + 8 * q);  // info read; the Q slot is freed by the MMA commit
-        const int n_tiles = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys;
-        const bool valid = row < it.rows;
-        // a warp without valid rows only keeps the barrier counts in step
-        const bool warp_live = warp * 32 < it.rows;
-        const int t_row = (it.mg * R + row) / g;
-        // Keys seen by this row: the cache prefix and the root (keys <= kv),
-        // then chain: the block positions up to t_row (keys <= kv + t_row);
-        // tree: the ancestors of node t_row and itself, bit j of its
-        // visibility row <-> key kv + 1 + j.
-        const uint64_t* vrow =
-            (tree_vis && valid) ? tree_vis + ((size_t)it.b * (K + 1) + t_row) * tree_words : nullptr;
-        const int mask_from = tree_vis ? it.kv : it.kv + t_row;  // tiles past this key need the mask
-        float m_run = -INFINITY, l_run = 0.f;
-        for (int t = 0; t < n_tiles && ok; ++t) {
-          const uint32_t gt = tile_ctr;
-          const uint32_t sb = gt & 1, pb = gt % kPBufs;
-          const int kt0 = it.key0 + t * kAttnTileKeys;
-          ok = warp_wait(bSFull + 8 * sb, (gt >> 1) & 1);
-          if (!ok) break;
-          if (!warp_live) {
-            __syncwarp();
-            if (lane == 0) {
-              mbar_arrive(bSFree + 8 * sb);
-              mbar_arrive(bPFull + 8 * pb);
-            }
-            ++tile_ctr;
-            continue;
-          }
-          tc_fence_after();
-          uint32_t sr[2][32];
-          tmem_ld32(tmem + lane_off + SM::kColS + sb * kAttnTileKeys, sr[0]);
-          tmem_ld32(tmem + lane_off + SM::kColS + sb * kAttnTileKeys + 32, sr[1]);
-          tmem_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bSFree + 8 * sb);
-          // raw scores; keys this row does not see (and rows past the
-          // group) count as -inf; the scale (> 0) is applied below
-          const bool need_mask = !valid || kt0 + kAttnTileKeys - 1 > mask_from;
-          uint64_t tmask = ~0ull;  // bit c: key kt0 + c is seen
-          if (need_mask) {
-            if (!valid) tmask = 0ull;
-            else if (!vrow) tmask = low_bits(it.kv + t_row + 1 - kt0);
-            else tmask = low_bits(it.kv + 1 - kt0) | bit_window(vrow, tree_words, kt0 - it.kv - 1);
-          }
-          // two copies of the loop: per-column mask tests that every tile ran
-          // took a fifth of the softmax's time on tiles with no masked key
-          float xs[kAttnTileKeys];
-          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-          if (need_mask) {
-#pragma unroll
-            for (int c = 0; c < kAttnTileKeys; ++c) {
-              float v = __uint_as_float(sr[c >> 5][c & 31]);
-              if (!((tmask >> c) & 1ull)) v = -INFINITY;
-              xs[c] = v;
-              mx[c & 3] = fmaxf(mx[c & 3], v);
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < kAttnTileKeys; ++c) {
-              xs[c] = __uint_as_float(sr[c >> 5][c & 31]);
-              mx[c & 3] = fmaxf(mx[c & 3], xs[c]);
-            }
-          }
-          const float tmax = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale_log2;
-          // raise the reference max only when it grows by more than 2^8
-          float f = 1.f;
-          const bool raise = tmax > m_run + kRescaleLog2;
-          if (raise) {
-            f = (m_run == -INFINITY) ? 0.f : ex2_approx(m_run - tmax);
-            m_run = tmax;
-          }
-          const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
-          float ls[4] = {0.f, 0.f, 0.f, 0.f};
-          uint32_t pk[32];
-#pragma unroll
-          for (int c = 0; c < kAttnTileKeys; c += 2) {
-            const float p0 = ex2_approx(fmaf(xs[c], scale_log2, neg_m));
-            const float p1 = ex2_approx(fmaf(xs[c + 1], scale_log2, neg_m));
-            ls[(c >> 1) & 3] += p0 + p1;
-            pk[c >> 1] = pack_bf16(p0, p1);
-          }
-          l_run = l_run * f + ((ls[0] + ls[1]) + (ls[2] + ls[3]));
-          // O holds the earlier tiles of this item: rescale its rows once the
-          // previous tile's PV has landed (rare: the max rose by > 2^8)
-          if (t > 0 && __any_sync(0xffffffffu, raise)) {
-            ok = warp_wait(bPVDone + 8 * ((gt - 1) % kPBufs), ((gt - 1) / kPBufs) & 1);
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll 1
-            for (int c0 = 0; c0 < D; c0 += 32) {
-              uint32_t o[32];
-              tmem_ld32(tmem + lane_off + SM::kColO + ob * D + c0, o);
-              tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-              tmem_st32(tmem + lane_off + SM::kColO + ob * D + c0, o);
-            }
-            tmem_wait_st();
-          }
-          // P buffer pb is free once PV(gt - kPBufs) has read it
-          if (gt >= kPBufs) {
-            ok = warp_wait(bPVDone + 8 * pb, ((gt / kPBufs) & 1) ^ 1);
-            if (!ok) break;
-            tc_fence_after();
-          }
-          tmem_st32(tmem + lane_off + SM::kColP + pb * 32, pk);
-          tmem_wait_st();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bPFull + 8 * pb);
-          ++tile_ctr;
+      bool failed = false;
+      for (int item = 0; item < n_items && has_items; ++item) {
+        wait(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
+        if (softmax_any(!ok)) {
+          failed = true;
+          break;
         }
-        if (!ok) break;
-        // epilogue: O of this item is complete once the last PV has landed
+        const ItemInfo& it = info[item_ctr & 1];
+        const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
+        const int steps0 = it.both ? n_tiles : (n_tiles + 1) >> 1, steps1 = it.both ? n_tiles : n_tiles >> 1;
+        const int my_steps = st ? steps1 : steps0;
+        const int rows = it.both && st ? it.rows1 : it.rows0;
+        const bool valid = row < rows;
+        // a warp without valid rows only keeps the barrier counts in step
+        const bool warp_live = wq * 32 < rows;
+        const int rr = it.mg * R + (it.both ? st * RU : 0) + row;  // row of the (sequence, kv head)
+        const int t_row = rr / g;
+        float m_run = -INFINITY, l_run = 0.f;
         {
-          const uint32_t last = tile_ctr - 1;
-          ok = warp_wait(bPVDone + 8 * (last % kPBufs), (last / kPBufs) & 1);
-          if (!ok) break;
-          tc_fence_after();
-          if (warp_live) {
-            const int rr = it.mg * R + row;
-            const int hq = it.kvh * g + rr % g;
-            const float inv = 1.f / l_run;
-            const size_t slot = (size_t)it.slot;
-#pragma unroll 1
-            for (int c0 = 0; c0 < D; c0 += 32) {
-              uint32_t o[32];
-              tmem_ld32(tmem + lane_off + SM::kColO + ob * D + c0, o);
+          // Keys seen by this row: the cache prefix and the root (keys <= kv),
+          // then chain: the block positions up to t_row (keys <= kv + t_row);
+          // tree: the ancestors of node t_row and itself, bit j of its
+          // visibility row <-> key kv + 1 + j.
+          const int kv = it.kv, key1 = it.key1;
+          const uint64_t* vrow =
+              (tree_vis && valid) ? tree_vis + ((size_t)it.b * (K + 1) + t_row) * tree_words : nullptr;
+          // tiles past this key need the mask; rows past the group compute on whatever their lanes hold, seen by no
+          // other row and never stored
+          const int mask_from = valid ? min(tree_vis ? kv : kv + t_row, key1 - 1) : 0x7fffffff;
+          const int kt_step = it.both ? 128 : 256;
+          int kt0 = it.key0 + (it.both ? 0 : st * 128);
+          for (int i = 0; i < my_steps; ++i, kt0 += kt_step) {
+            const uint32_t n = (st ? done1 : done0) + i;
+            wait(bSFull + 8 * st, n & 1);
+            if (!warp_live) {
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bPFull + 8 * st);
+              continue;
+            }
+            tc_fence_after();
+            const bool two = key1 - kt0 > 64;  // the tile's second 64 keys exist
+            // (the whole warp masks or none of it: the loops below hold warp-wide tensor-memory instructions)
+            const bool need_mask = __any_sync(0xffffffffu, kt0 + 127 > mask_from);
+            // raw scores of keys c0 .. c0 + 31; keys this row does not see count as -inf
+            auto load_scores = [&](int c0, uint32_t (&x)[32]) {
+              tmem_ld32(ts + c0, x);
               tmem_wait_ld();
-              if (valid) {
-                if (!it.partial) {
-                  uint4* dst =
-                      reinterpret_cast<uint4*>(O + (((size_t)it.b * (K + 1) + t_row) * Hq + hq) * D + c0);
+              if (need_mask) {
+                const int k0 = kt0 + c0;
+                uint32_t bits = (uint32_t)(!vrow ? low_bits(kv + t_row + 1 - k0)
+                                                 : low_bits(kv + 1 - k0) | bit_window(vrow, tree_words, k0 - kv - 1));
+                bits &= (uint32_t)low_bits(key1 - k0);
+                if (!valid) bits = ~0u;
 #pragma unroll
-                  for (int i = 0; i < 4; ++i)
-                    dst[i] = make_uint4(
-                        pack_bf16(__uint_as_float(o[8 * i]) * inv, __uint_as_float(o[8 * i + 1]) * inv),
-                        pack_bf16(__uint_as_float(o[8 * i + 2]) * inv, __uint_as_float(o[8 * i + 3]) * inv),
-                        pack_bf16(__uint_as_float(o[8 * i + 4]) * inv, __uint_as_float(o[8 * i + 5]) * inv),
-                        pack_bf16(__uint_as_float(o[8 * i + 6]) * inv, __uint_as_float(o[8 * i + 7]) * inv));
-                } else {
-                  uint4* dst = reinterpret_cast<uint4*>(part_o + (slot * kAttnRows + row) * D + c0);
-#pragma unroll
-                  for (int i = 0; i < 8; ++i) dst[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-                }
+                for (int c = 0; c < 32; ++c)
+                  if (!((bits >> c) & 1u)) x[c] = __float_as_uint(-INFINITY);
               }
+            };
+            // (Loops of 32 keys, loaded again for the second: short code. A
+            // tile's arithmetic unrolled over its 128 keys ran no faster warm,
+            // and at B = 1, where each layer runs it once or twice, twice as
+            // long, on instruction fetches.)
+            const int n_cols = two ? 128 : 64;
+            float tmax = -INFINITY;
+#pragma unroll 1
+            for (int c0 = 0; c0 < n_cols; c0 += 32) {
+              uint32_t x[32];
+              load_scores(c0, x);
+              float a = tmax, b = -INFINITY;
+#pragma unroll
+              for (int c = 0; c < 32; c += 4) {
+                a = fmaxf(fmaxf(a, __uint_as_float(x[c])), __uint_as_float(x[c + 1]));
+                b = fmaxf(fmaxf(b, __uint_as_float(x[c + 2])), __uint_as_float(x[c + 3]));
+              }
+              tmax = fmaxf(a, b);
+            }
+            tmax *= scale_log2;
+            // raise the reference max only when it grows by more than 2^8
+            const bool raise = tmax > m_run + kRescaleLog2;
+            if (__any_sync(0xffffffffu, raise)) {
+              float f = 1.f;
+              f = !raise ? 1.f : (m_run == -INFINITY) ? 0.f : ex2_approx(m_run - tmax);
+              m_run = raise ? tmax : m_run;
+              l_run *= f;
+              if (i > 0) {
+                // O holds the stream's earlier tiles of this item: rescale its
+                // rows once the last PV has landed
+                wait(bPVDone + 8 * st, (n - 1) & 1);
+                tc_fence_after();
+#pragma unroll 1
+                for (int c0 = 0; c0 < D; c0 += 32) {
+                  uint32_t o[32];
+                  const uint32_t oa = tmem + lane_off + SM::kColO + st * 128 + c0;
+                  tmem_ld32(oa, o);
+                  tmem_wait_ld();
+#pragma unroll
+                  for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * f);
+                  tmem_st32(oa, o);
+                }
+                tmem_wait_st();
+              }
+            }
+            const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
+            float la[2] = {0.f, 0.f}, lb[2] = {0.f, 0.f};
+#pragma unroll 1
+            for (int c0 = 0; c0 < n_cols; c0 += 32) {
+              uint32_t x[32], pk[16];
+              load_scores(c0, x);
+#pragma unroll
+              for (int c = 0; c < 32; c += 4) {
+                float y0, y1, y2, y3;
+                fma2(y0, y1, __uint_as_float(x[c]), __uint_as_float(x[c + 1]), scale_log2, neg_m);
+                fma2(y2, y3, __uint_as_float(x[c + 2]), __uint_as_float(x[c + 3]), scale_log2, neg_m);
+                y0 = ex2_approx(y0);
+                y1 = ex2_approx(y1);
+                y2 = ex2_approx(y2);
+                y3 = ex2_approx(y3);
+                add2(la[0], la[1], y0, y1);
+                add2(lb[0], lb[1], y2, y3);
+                pk[c >> 1] = pack_bf16(y0, y1);
+                pk[(c >> 1) + 1] = pack_bf16(y2, y3);
+              }
+              tmem_st16(ts + c0 / 2, pk);  // over scores already read
+            }
+            l_run += (la[0] + la[1]) + (lb[0] + lb[1]);
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bPFull + 8 * st);
+          }
+        }
+        // ---- epilogue: O of this item is complete once the last PVs have landed ----
+        float f0 = 1.f, f1 = 0.f;  // factors of the streams' O (two units: f0 of this stream's own)
+        if (!it.both && steps1 > 0) {
+          // both streams hold keys of the same rows: exchange (m, l)
+          if (warp_live) stat[st * 128 + row] = make_float2(m_run, l_run);
+          softmax_sync();
+          if (warp_live) {
+            const float2 a = stat[row], b = stat[128 + row];
+            const float M = fmaxf(a.x, b.x);
+            f0 = M == -INFINITY ? 0.f : ex2_approx(a.x - M);
+            f1 = M == -INFINITY ? 0.f : ex2_approx(b.x - M);
+            m_run = M;
+            l_run = f0 * a.y + f1 * b.y;
+          }
+        }
+        if (it.both ? st == 0 : true) wait(bPVDone, (done0 + steps0 - 1) & 1);
+        if (it.both ? st == 1 : steps1 > 0) wait(bPVDone + 8, (done1 + steps1 - 1) & 1);
+        tc_fence_after();
+        // the streams share out the columns of rows they both hold; a single step leaves all to stream 0
+        const bool second = !it.both && steps1 > 0;
+        if (warp_live && (it.both || second || st == 0)) {
+          const int hq = it.kvh * g + rr % g;
+          const size_t prow = (size_t)it.slot * slot_rows + (it.both ? st * RU : 0) + row;
+          const bool partial = it.partial;
+          if (!partial) {
+            const float inv = 1.f / l_run;
+            f0 *= inv;
+            f1 *= inv;
+          }
+          const int cb = second ? st * (D / 2) : 0, ce = second ? cb + D / 2 : D;
+          __nv_bfloat16* orow = O + (((size_t)it.b * (K + 1) + t_row) * Hq + hq) * D;
+          const uint32_t oa = tmem + lane_off + SM::kColO + (it.both ? st * 128 : 0);
+#pragma unroll 1
+          for (int c0 = cb; c0 < ce; c0 += 32) {
+            uint32_t o[32];
+            tmem_ld32(oa + c0, o);
+            if (second) {
+              uint32_t o1[32];
+              tmem_ld32(oa + 128 + c0, o1);
+              tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < 32; ++c)
+                o[c] = __float_as_uint(fmaf(__uint_as_float(o1[c]), f1, __uint_as_float(o[c]) * f0));
+            } else {
+              tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * f0);
             }
             if (valid) {
-              if (it.partial) {
-                *reinterpret_cast<float2*>(part_ml + (slot * kAttnRows + row) * 2) = make_float2(m_run, l_run);
-              } else if (lse) {
-                lse[((size_t)it.b * (K + 1) + t_row) * Hq + hq] = (m_run + __log2f(l_run)) * kLn2;
+              if (!partial) {
+                uint4* dst = reinterpret_cast<uint4*>(orow + c0);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                  dst[i] = make_uint4(pack_bf16(__uint_as_float(o[8 * i]), __uint_as_float(o[8 * i + 1])),
+                                      pack_bf16(__uint_as_float(o[8 * i + 2]), __uint_as_float(o[8 * i + 3])),
+                                      pack_bf16(__uint_as_float(o[8 * i + 4]), __uint_as_float(o[8 * i + 5])),
+                                      pack_bf16(__uint_as_float(o[8 * i + 6]), __uint_as_float(o[8 * i + 7])));
+              } else {
+                uint4* dst = reinterpret_cast<uint4*>(part_o + prow * D + c0);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) dst[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
               }
             }
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bOFree + 8 * ob);
-          if (it.partial && layer == n_layers - 1)
-            last_layer_part_done<D>(tasks, n_tasks, it.grp, grp_cnt, misc, part_o, part_ml, K, Hq, g, R, O, lse);
+          if (valid && (it.both || st == 0)) {
+            if (partial) {
+              *reinterpret_cast<float2*>(part_ml + prow * 2) = make_float2(m_run, l_run);
+            } else if (lse) {
+              lse[((size_t)it.b * (K + 1) + t_row) * Hq + hq] = (m_run + __log2f(l_run)) * kLn2;
+            }
+          }
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bOFree);
+        if (it.partial && layer == n_layers - 1) {
+          // The last layer's split groups need no grid barrier: each part is
+          // counted in as written (the named barrier orders the warpgroups'
+          // writes before the release).
+          softmax_sync();
+          if (tid == 0)
+            asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(grp_cnt + 2 * it.grp), "r"(1u) : "memory");
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bIEmpty + 8 * (item_ctr & 1));  // `it` has been read
+        done0 += steps0;
+        done1 += steps1;
         ++item_ctr;
       }
-      if (!ok) break;
+      if (failed) {
+        ok = false;
+        break;
+      }
       // This CTA is done with the layer's items. Once its grid barrier
       // passes, CTAs write layer + 1's partials into the buffer of layer - 2,
       // whose merge must be done first. Help with the merge warp's backlog
@@ -1227,16 +1304,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       if (layer > 0 && merge_n > 0 &&
           (has_items ? layer * merge_n - *reinterpret_cast<volatile int*>(merge_claimed) >= kMergeHelpChunks
                      : last_groups_ready()))
-        merge_chunks<D>(layer - 1, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R, part_buf_o,
-                        part_buf_ml, part_o_stride, part_ml_stride, n_layers - 1);
+        merge_chunks<D>(layer - 1, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R, slot_rows, part_buf_o,
+                        part_buf_ml, part_o_stride, part_ml_stride);
       if (!has_items) break;
       if (layer >= kAttnPartBufs - 1 && merge_n > 0 && tid == 0 &&
-          !merged_upto((layer - (kAttnPartBufs - 2)) * merge_n)) {
-        raise_status(status, LIBRASPEC_ST_TIMEOUT);
-        misc[0] = 1;
-      }
-      softmax_sync();
-      if (misc[0]) {
+          !merged_upto((layer - (kAttnPartBufs - 2)) * merge_n))
+        ok = false;
+      if (softmax_any(!ok || misc[0])) {
         ok = false;
         break;
       }
@@ -1261,11 +1335,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         // counters for the next launch
         if (lane == 0) {
           for (int ti = 0; ti < n_tasks && ok; ++ti)
-            if (!tasks[ti].epi) ok = wait_counter(grp_cnt + 2 * tasks[ti].grp, tasks[ti].np);
+            ok = wait_counter(grp_cnt + 2 * tasks[ti].grp, tasks[ti].np);
           if (ok) {
             misc[6] = 1;  // the softmax warps may help now
             for (int ti = 0; ti < n_tasks; ++ti) {
-              if (tasks[ti].epi) continue;
               uint32_t* gc = grp_cnt + 2 * tasks[ti].grp;
               if (atomicAdd(gc + 1, 1u) == (uint32_t)tasks[ti].np - 1) {
                 gc[0] = 0u;
@@ -1278,8 +1351,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       }
       if (!ok) break;
       if (merge_n > 0)
-        merge_chunks<D>(layer, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R, part_buf_o,
-                        part_buf_ml, part_o_stride, part_ml_stride, n_layers - 1);
+        merge_chunks<D>(layer, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R, slot_rows, part_buf_o,
+                        part_buf_ml, part_o_stride, part_ml_stride);
     }
     // every chunk of every layer is merged (by whichever warp) before the exit count
     if (ok && merge_n > 0 && n_layers > 0) {
@@ -1316,14 +1389,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
 // ---------------------------------------------------------------------------
 int num_sms_current();
 
-// Q [B*(K+1), Hq, D] as 3-D; box = 64 columns x g heads x R/g positions (one
-// row group of one kv head), 128-byte swizzle.
-static bool make_q_map(CUtensorMap* map, const void* base, int D, int Hq, int BT, int g, int R) {
+// Q [B*(K+1), Hq, D] as 3-D; box = 64 columns x g heads x RU/g positions (one
+// unit of rows of one kv head), 128-byte swizzle.
+static bool make_q_map(CUtensorMap* map, const void* base, int D, int Hq, int BT, int g, int RU) {
   auto enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)BT};
   cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)Hq * D * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)g, (cuuint32_t)(R / g)};
+  cuuint32_t box[3] = {64, (cuuint32_t)g, (cuuint32_t)(RU / g)};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -1483,21 +1556,21 @@ struct LayerSetCache {
 };
 constexpr int kCachedChunks = 4;
 
-template <int D, int STAGES, bool PAGED>
+template <int D, int QS, bool PAGED>
 static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* const* Kc, const uint16_t* const* Vc,
                                    int n_layers, const int32_t* kv_len, const int32_t* L, const uint64_t* tree_vis,
                                    const int32_t* block_table,
                                    int max_pages, int page_size, int n_pages, int B, int K, int Hq, int Hkv, int S_cap,
                                    float scale, uint16_t* const* O, float* const* lse, char* ws, const WsLayout& lay,
                                    cudaStream_t stream) {
-  using SM = AttnSmem<D, STAGES>;
+  using SM = AttnSmem<D, QS>;
   constexpr int kSmem = PAGED ? SM::kAllocPaged : SM::kAlloc;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(verify_attn_kernel<D, STAGES, PAGED, false>,
+    cudaError_t e = cudaFuncSetAttribute(verify_attn_kernel<D, QS, PAGED, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(verify_attn_kernel<D, STAGES, PAGED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      e = cudaFuncSetAttribute(verify_attn_kernel<D, QS, PAGED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kSmem);
     if (e != cudaSuccess) return e;
     configured = true;
@@ -1509,9 +1582,9 @@ static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* con
   // (its code alone measured 2.5% faster on the latency-bound B = 1 layers).
   const int item_tiles = attn_item_tiles();
   const bool weighted = item_tiles > 0 && (long long)B * Hkv > grid;
-  auto kern = weighted ? verify_attn_kernel<D, STAGES, PAGED, true> : verify_attn_kernel<D, STAGES, PAGED, false>;
+  auto kern = weighted ? verify_attn_kernel<D, QS, PAGED, true> : verify_attn_kernel<D, QS, PAGED, false>;
   const int g = Hq / Hkv;
-  const int R = g * (kAttnRows / g);
+  const int R = attn_unit_rows(g);
   // layers beyond kMaxLayers go in further launches of the same kernel
   for (int l0 = 0; l0 < n_layers; l0 += kMaxLayers) {
     const int n = n_layers - l0 < kMaxLayers ? n_layers - l0 : kMaxLayers;
@@ -1577,7 +1650,7 @@ static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* con
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(
         &cfg, kern, set, kv_len, L, tree_vis, tree_words(K), block_table, max_pages, page_size, n_pages, attn_page_cache(SM::kPageCap), B, K,
-        Hq, Hkv, S_cap, scale * kLog2e, attn_min_tiles(), item_tiles,
+        Hq, Hkv, S_cap, scale * kLog2e, attn_min_tiles(), item_tiles, attn_slot_rows(g, K),
         reinterpret_cast<float*>(ws + lay.attn_o), reinterpret_cast<float*>(ws + lay.attn_ml), o_part / sizeof(float),
         ml_part / sizeof(float), reinterpret_cast<uint32_t*>(ws + lay.attn_cnt),
         reinterpret_cast<uint32_t*>(ws + lay.attn_grp), reinterpret_cast<int*>(ws + lay.status));
@@ -1596,11 +1669,11 @@ cudaError_t launch_verify_attn_layers(const uint16_t* const* Q, const uint16_t* 
   const uint64_t* vis = nullptr;
   cudaError_t e = tree_vis(parent, L, B, K, ws, lay, stream, &vis);
   if (e != cudaSuccess) return e;
-  if (D == 128)
-    return launch_layers_t<128, 5, false>(Q, Kc, Vc, n_layers, kv_len, L, vis, nullptr, 0, 0, 0, B, K, Hq, Hkv, S_cap,
+  const bool two = attn_slot_rows(Hq / Hkv, K) > kAttnRows;  // row groups of up to two units
+  auto* launch = D == 128 ? (two ? launch_layers_t<128, 2, false> : launch_layers_t<128, 1, false>)
+                          : (two ? launch_layers_t<64, 2, false> : launch_layers_t<64, 1, false>);
+  return launch(Q, Kc, Vc, n_layers, kv_len, L, vis, nullptr, 0, 0, 0, B, K, Hq, Hkv, S_cap,
                                           scale, O, lse, ws, lay, stream);
-  return launch_layers_t<64, 8, false>(Q, Kc, Vc, n_layers, kv_len, L, vis, nullptr, 0, 0, 0, B, K, Hq, Hkv, S_cap,
-                                       scale, O, lse, ws, lay, stream);
 }
 
 cudaError_t launch_verify_attn_paged_layers(const uint16_t* const* Q, const uint16_t* const* Kp,
@@ -1614,11 +1687,11 @@ cudaError_t launch_verify_attn_paged_layers(const uint16_t* const* Q, const uint
   const uint64_t* vis = nullptr;
   cudaError_t e = tree_vis(parent, L, B, K, ws, lay, stream, &vis);
   if (e != cudaSuccess) return e;
-  if (D == 128)
-    return launch_layers_t<128, 5, true>(Q, Kp, Vp, n_layers, kv_len, L, vis, block_table, max_pages, page_size,
+  const bool two = attn_slot_rows(Hq / Hkv, K) > kAttnRows;
+  auto* launch = D == 128 ? (two ? launch_layers_t<128, 2, true> : launch_layers_t<128, 1, true>)
+                          : (two ? launch_layers_t<64, 2, true> : launch_layers_t<64, 1, true>);
+  return launch(Q, Kp, Vp, n_layers, kv_len, L, vis, block_table, max_pages, page_size,
                                          n_pages, B, K, Hq, Hkv, S_cap, scale, O, lse, ws, lay, stream);
-  return launch_layers_t<64, 8, true>(Q, Kp, Vp, n_layers, kv_len, L, vis, block_table, max_pages, page_size, n_pages,
-                                      B, K, Hq, Hkv, S_cap, scale, O, lse, ws, lay, stream);
 }
 
 cudaError_t launch_verify_attn(const uint16_t* Q, const uint16_t* Kc, const uint16_t* Vc, const int32_t* kv_len,

@@ -148,6 +148,48 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
       : "memory");
 }
 
+// The two words of smem_desc for SBO = 1024 apart: the high one is a constant, the low one an address and the LBO.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) {
+  return ((addr >> 4) & 0x3FFF) | ((lbo >> 4) << 16);
+}
+
+// Four K steps of one MMA, the operands' addresses advancing by SA / SB bytes. Building eight 64-bit descriptors
+// cost the issuing thread 77 cycles per MMA whatever its size, adding to one word 49 (a probe; the MMAs themselves
+// take 40 to 64 cycles at M = 128, N = 32 to 128).
+template <int SA, int SB>
+__device__ __forceinline__ void mma_ss4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 x, y;\n\t.reg .b64 a, b;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+      "mov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
+      "add.u32 x, %1, %6;\n\tadd.u32 y, %2, %7;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, 1;\n\t"
+      "add.u32 x, x, %6;\n\tadd.u32 y, y, %7;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, 1;\n\t"
+      "add.u32 x, x, %6;\n\tadd.u32 y, y, %7;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, 1;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(acc), "n"(kDescHi), "n"(SA / 16), "n"(SB / 16)
+      : "memory");
+}
+
+// The same with A in tensor memory (16 bf16 columns, 8 words, a step).
+template <int SB>
+__device__ __forceinline__ void mma_ts4(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 x, y;\n\t.reg .b64 b;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t"
+      "add.u32 x, %1, 8;\n\tadd.u32 y, %2, %6;\n\tmov.b64 b, {y, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [x], b, %3, 1;\n\t"
+      "add.u32 x, x, 8;\n\tadd.u32 y, y, %6;\n\tmov.b64 b, {y, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [x], b, %3, 1;\n\t"
+      "add.u32 x, x, 8;\n\tadd.u32 y, y, %6;\n\tmov.b64 b, {y, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [x], b, %3, 1;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(acc), "n"(kDescHi), "n"(SB / 16)
+      : "memory");
+}
+
 // Arrive once on `bar` when every tcgen05.mma this thread issued before has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
@@ -220,6 +262,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+          taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 

@@ -222,3 +222,18 @@ def test_attn_layer_chain_matches_per_layer_oracle(orc, name, n_layers, L_max):
         O1, lse1 = _run(layers[l]["Q"], layers[l]["Kc"], layers[l]["Vc"], kv.tolist(), L.tolist(), w.K)
         for b in range(w.B):
             assert torch.equal(O1[b, : L[b] + 1], outs[l][b, : L[b] + 1])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("Hq,Hkv,K", [(16, 2, 16), (32, 8, 32), (14, 2, 17), (8, 8, 8)])
+def test_attn_step_and_unit_edges(orc, d, Hq, Hkv, K):
+    """Items of one to several 128-key steps whose last is half or full (one stream idle, both, an odd count), and
+    row groups that end inside, at and just past their first unit of 128 rows. Tolerances as in check_attn."""
+    kv = [0, 62, 63, 64, 127, 128, 129, 191, 255, 256, 257, 320, 500, 1100]
+    L = [K, 0, K, K - 1, K - 2, K, 1, K, K // 2, K, 0, K - 1, K, K]
+    S_cap = max(kv) + K + 1
+    Q, Kc, Vc = _inputs(len(kv), K, Hq, Hkv, d, kv, S_cap, seed=d + Hq + K, scale_k=2.0)
+    O_ref, lse_ref = orc.verify_attn(Q, Kc, Vc, np.array(kv), np.array(L))
+    for _ in range(3):
+        O, lse = _run(Q, Kc, Vc, kv, L, K)
+        check_attn(O, lse, O_ref, lse_ref, L)
