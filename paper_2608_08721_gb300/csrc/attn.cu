@@ -10,11 +10,9 @@
 // (K+1)*g rows may not fit one) and keys into 64-key tiles. All (row group,
 // key tile) pairs of the batch form one tile sequence (sequence-major, then kv
 // head, row group, key tile); CTA c of the persistent grid (one CTA per SM)
-// takes the contiguous range [c*T/G, (c+1)*T/G) of it, so every CTA streams
-// the same number of tiles whatever the ragged lengths; with more (sequence,
-// kv head) pairs than CTAs the ranges are cut by cost instead (each row
-// group weighs its tiles plus an item's fixed cost; tile_of_weighted). The
-// plan is derived on the device from L[] and kv_len[] by every CTA, and it
+// takes a contiguous range of it, cut by cost (each row group weighs its
+// tiles plus an item's fixed cost; tile_of_weighted), so that CTAs finish
+// together whatever the ragged lengths. The plan is derived on the device from L[] and kv_len[] by every CTA, and it
 // is the same for every layer (all layers share L and kv_len).
 //
 // Two streams per CTA. An item (a run of tiles of one row group) is worked on
@@ -260,7 +258,11 @@ __device__ __forceinline__ int cta_of(long long t, long long T, int G) {
 // merge, in tile-equivalents), placed before its tiles; the batch weighs
 // W = T + C * groups, and CTA c takes the tiles of the weighted range
 // [c W / G, (c+1) W / G). A boundary inside a group's C falls on the
-// group's first tile. C = 0 is the plain split by tiles.
+// group's first tile. C = 0 is the plain split by tiles. C is 4, or a quarter
+// of a CTA's tiles if that is less (a cost of several tiles would leave CTAs
+// with few tiles without any): 16 paged sequences 110 -> 102 us (2 layers), a
+// tree of 512 nodes 352 -> 339 (4 layers), ragged B = 64 312 -> 296; C = 8 and
+// 12 gave ragged 298 and 301, the tree 332.
 __device__ long long tile_of_weighted(long long x, long long W, long long T, int C, int B, const int32_t* kv_len,
                                       const int32_t* Ls, int K, int g, int R, int Hkv, int S_cap) {
   if (x >= W) return T;
@@ -579,7 +581,7 @@ __device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set
 // tree_vis (optional, [B, K+1, tree_words]): the block is a draft tree and
 // row t sees the block keys of the set bits (bit j <-> block position j + 1)
 // besides the root and the prefix; nullptr: the chain draft (block-causal).
-template <int D, int QS, bool PAGED, bool WEIGHTED>
+template <int D, int QS, bool PAGED>
 __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     const __grid_constant__ LayerSet set, const int32_t* __restrict__ kv_len, const int32_t* __restrict__ Ls,
     const uint64_t* __restrict__ tree_vis, int tree_words,
@@ -691,16 +693,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       if ((long long)G > g_cap) G = (int)g_cap;
     }
     const int c = blockIdx.x;
-    // weighted length (the unweighted instantiation splits by tiles alone)
-    const long long W = WEIGHTED ? T + (long long)item_tiles * NG : T;
+    // an item's fixed cost in tiles, less where a CTA has few
+    const int C = T > 0 ? (int)min((long long)item_tiles, div_nn(T, 4 * (long long)G)) : 0;
+    const long long W = T + (long long)C * NG;  // weighted length
     long long lo = 0, hi = 0;
     if (T > 0 && c < G) {
-      if constexpr (WEIGHTED) {
-        lo = tile_of_weighted(range_lo(c, W, G), W, T, item_tiles, B, kvs, Lss, K, g, R, Hkv, S_cap);
-        hi = tile_of_weighted(range_lo(c + 1, W, G), W, T, item_tiles, B, kvs, Lss, K, g, R, Hkv, S_cap);
-      } else {
-        lo = range_lo(c, T, G);
-        hi = range_lo(c + 1, T, G);
+      lo = range_lo(c, W, G);
+      hi = range_lo(c + 1, W, G);
+      if (C > 0) {
+        lo = tile_of_weighted(lo, W, T, C, B, kvs, Lss, K, g, R, Hkv, S_cap);
+        hi = tile_of_weighted(hi, W, T, C, B, kvs, Lss, K, g, R, Hkv, S_cap);
       }
     }
     int n_items = 0, n_tasks = 0;
@@ -727,7 +729,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             t.kvh = gib / loc.p.n_mg;
             t.mg = gib % loc.p.n_mg;
             t.rows = min(R, loc.p.M - t.mg * R);
-            const int C = WEIGHTED ? item_tiles : 0;
             t.c0 = cta_of(weighted_pos(gstart, group, C), W, G);
             t.np = cta_of(weighted_pos(gend - 1, group, C), W, G) - t.c0 + 1;
             t.grp = group;
@@ -1417,11 +1418,13 @@ static bool make_kv_map(CUtensorMap* map, const void* base, int D, int S_cap, in
   return r == CUDA_SUCCESS;
 }
 
-// Smallest tile range per CTA; the LIBRASPEC_ATTN_MIN_TILES environment
+// Smallest tile range per CTA (1: as many CTAs as there are tiles; at 2, half
+// the CTAs work on 3 sequences of 900 keys and 32 layers take 319 us instead
+// of 235); the LIBRASPEC_ATTN_MIN_TILES environment
 // variable overrides the default, read once per process.
 static int attn_min_tiles() {
   static int t = [] {
-    int v = 2;
+    int v = 1;
     if (const char* e = getenv("LIBRASPEC_ATTN_MIN_TILES")) {
       int a = 0;
       if (sscanf(e, "%d", &a) == 1 && a >= 1 && a <= 4096) v = a;
@@ -1436,7 +1439,7 @@ static int attn_min_tiles() {
 // overrides the default, read once per process.
 static int attn_item_tiles() {
   static int t = [] {
-    int v = 2;
+    int v = 4;
     if (const char* e = getenv("LIBRASPEC_ATTN_ITEM_TILES")) {
       int a = 0;
       if (sscanf(e, "%d", &a) == 1 && a >= 0 && a <= 64) v = a;
@@ -1567,22 +1570,15 @@ static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* con
   constexpr int kSmem = PAGED ? SM::kAllocPaged : SM::kAlloc;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(verify_attn_kernel<D, QS, PAGED, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(verify_attn_kernel<D, QS, PAGED, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmem);
+    cudaError_t e = cudaFuncSetAttribute(verify_attn_kernel<D, QS, PAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kSmem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
   int grid = num_sms_current();  // one CTA per SM (it holds all 512 tensor-memory columns)
   if (grid > kAttnMaxCtas) grid = kAttnMaxCtas;
-  // The cost-weighted split pays where CTAs hold many items: more (sequence,
-  // kv head) pairs than CTAs. Otherwise the instantiation without it runs
-  // (its code alone measured 2.5% faster on the latency-bound B = 1 layers).
+  auto kern = verify_attn_kernel<D, QS, PAGED>;
   const int item_tiles = attn_item_tiles();
-  const bool weighted = item_tiles > 0 && (long long)B * Hkv > grid;
-  auto kern = weighted ? verify_attn_kernel<D, QS, PAGED, true> : verify_attn_kernel<D, QS, PAGED, false>;
   const int g = Hq / Hkv;
   const int R = attn_unit_rows(g);
   // layers beyond kMaxLayers go in further launches of the same kernel
