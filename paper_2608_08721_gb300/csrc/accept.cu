@@ -174,93 +174,106 @@ __device__ __forceinline__ void race_combine(float& E, float& y, int& i, float E
   }
 }
 
-// The best candidate that any lane of the warp holds, (bEw, byw); bEw = inf
-// when no lane has one. Lanes rank their candidates by the log2 key
-// log2(bE) - by c with the fast logarithm: a slightly wrong pick only makes
-// the screen below a little looser, never unsafe, since the picked
-// candidate is a token some lane has drawn. All 32 lanes take part.
-__device__ __forceinline__ void warp_best_candidate(float bE, float by, float c, float& bEw, float& byw) {
-  const bool has = bE < INFINITY;
-  const float lk = has ? __log2f(bE) - by * c : INFINITY;
-  float mn = lk;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-  const unsigned ball = __ballot_sync(0xffffffffu, has && lk == mn);
-  const int src = ball ? __ffs(ball) - 1 : 0;
-  const float e = __shfl_sync(0xffffffffu, bE, src);
-  byw = __shfl_sync(0xffffffffu, by, src);
-  bEw = ball ? e : INFINITY;
+// Order-preserving map of floats to ints (for atomicMin on shared memory) and back.
+__device__ __forceinline__ int float_order(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float order_float(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
+
+// The smallest value any lane of the warp holds (all 32 lanes take part).
+__device__ __forceinline__ float warp_fmin(float x) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
 }
 
-// Token v (logit y, Philox word w) in the bonus race. v beats a candidate
-// (E, y') iff E_v = -ln u_v < X = E 2^((y - y') c), i.e. u_v > exp(-X). The
-// screen tests that against the warp's best candidate (bEw, byw), a token
-// already drawn, with a margin of 2^-12 above the fast exponentials' error,
-// so every token that can still win the race passes it; a token that
-// passes takes the exact logarithm and is compared with the lane's own
-// candidate (bE, by, bi). Screening against the warp's candidate rather
-// than the lane's own skips the logarithm for most of the slice: a warp
-// runs the exact step whenever any of its lanes needs it.
-__device__ __forceinline__ void bonus_race_token(float y, uint32_t w, int v, float c, float bEw, float byw, float& bE,
-                                                 float& by, int& bi) {
-  const float u = word_to_uniform(w);
-  if (bEw < INFINITY) {
-    const float Xw = bEw * ex2_approx((y - byw) * c);
-    if (!(u > ex2_approx(-Xw * kLog2e) * 0.999755859375f)) return;
-  }
-  const float Ev = -logf(u);
-  if (!(bE < INFINITY) || Ev < bE * ex2_approx((y - by) * c)) {
-    bE = Ev; by = y; bi = v;
-  }
-}
-
-// The bonus race over logits [c0, c1) of row j (sampling at c = log2(e)/T):
-// uniforms from Philox at (v >> 2, j, seq, purpose 1), word v & 3. Four
-// groups of four logits are loaded before any is used. The trip counts are
-// the warp's (lanes past the slice's end idle), so that every lane joins
-// the refreshes of the warp's candidate: after the first token, then
-// before every later group.
-template <bool VEC, typename E>
-__device__ __forceinline__ void bonus_race_slice(const E* __restrict__ yr, int c0, int c1, int V, float c,
-                                                 uint64_t seed, uint32_t j, uint32_t seq, uint64_t round_offset,
-                                                 float& bE, float& by, int& bi) {
+// A race over logits [c0, c1) of one row: token v's key is E_v / w_v with
+// E_v = -ln u_v, u_v the uniform of word v & 3 of the Philox block (v >> 2, j,
+// seq, purpose), and log2 w_v <= y_v c + off. The smallest key wins.
+//
+// Bound by issue (a Philox block alone is about 60 instructions per four
+// tokens), so almost no token is worked out: since -ln u >= 1 - u, a token
+// can only beat the best log2 key `thr` known so far if
+//   1 - u_v < 2^(thr + off + y_v c),
+// and the eight tokens of two Philox blocks are dismissed by one such test on
+// their largest uniform and their largest logit. If it passes, they are tested one
+// by one, and eval(y, u, v) takes those that pass exactly. `thr` is the best
+// key of any lane of the CTA: the lanes' own() keys (log2, a fast logarithm
+// is enough) by warp minimum, the warps' through s_thr, refreshed after the
+// first token of each lane and whenever a test of the warp has passed. The
+// margins (2^0.004, and 2^-21 of |y c| in the exponent) are far above the
+// rounding of the test, so every possible winner passes.
+// Before (each token tested with two exponentials, exact steps whenever a
+// lane of the warp passed): 70 instructions per token; 2 trees of 257 nodes,
+// V = 152064, bf16: 148 us; now 23 instructions, 90 us (the integer
+// multiplies alone: 36 us).
+// Loads run two trips ahead of the eight logits in use (two Philox blocks and
+// one copy of the exact step per trip: short code, and two chains to
+// interleave); the trip counts are the warp's, so that every lane joins the
+// votes.
+template <bool VEC, typename E, typename Own, typename Eval>
+__device__ __forceinline__ void race_slice(const E* __restrict__ yr, int c0, int c1, int V, float c, float off,
+                                           uint64_t seed, uint32_t j, uint32_t seq, uint32_t purpose,
+                                           uint64_t round_offset, int* s_thr, Own own, Eval eval) {
   const int g1 = (c1 + 3) >> 2;
   const int lane = threadIdx.x & 31;
-  float bEw = INFINITY, byw = 0.f;
-  bool first = true;
-  for (int gw = (c0 >> 2) + (int)(threadIdx.x & ~31u); gw < g1; gw += 4 * kRowThreads) {
-    const int g = gw + lane;
-    float yv[4][4];
+  const float slack = c * 4.76837158203125e-7f;
+  const float add = off + 0.004f;
+  float thr = INFINITY;
+  auto bound = [&](float y) { return ex2_approx(thr + (fmaf(fabsf(y), slack, add) + y * c)); };
+  auto refresh = [&]() {
+    const float m = warp_fmin(own());
+    if (lane == 0 && m < thr) atomicMin(s_thr, float_order(m));
+    thr = fminf(thr, m);
+  };
+  using Raw4 = typename Logit<E>::Raw4;
+  auto load = [&](int g, Raw4 (&raw)[2]) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 2; ++k) {
       const int gg = g + k * kRowThreads;
-      if (gg < g1) {
-        if (VEC) {
-          Logit<E>::stream4(yr + 4 * gg, yv[k]);
-        } else {
-#pragma unroll
-          for (int t = 0; t < 4; ++t) yv[k][t] = 4 * gg + t < V ? Logit<E>::at(yr, 4 * gg + t) : -INFINITY;
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) yv[k][t] = -INFINITY;
-      }
+      if (VEC) raw[k] = gg < g1 ? Logit<E>::load4(yr + 4 * gg) : Logit<E>::none4();
+      else raw[k] = Logit<E>::gather4(yr + 4 * (size_t)gg, gg < g1 ? V - 4 * gg : 0);
     }
+  };
+  const int gw0 = (c0 >> 2) + (int)(threadIdx.x & ~31u);
+  Raw4 next[2], after[2];
+  load(gw0 + lane, next);
+  load(gw0 + 2 * kRowThreads + lane, after);
+#pragma unroll 1
+  for (int gw = gw0; gw < g1; gw += 2 * kRowThreads) {
+    const int g = gw + lane;
+    float y[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (gw + k * kRowThreads >= g1) break;  // the same for the whole warp
-      if (!first) warp_best_candidate(bE, by, c, bEw, byw);
-      const int gg = g + k * kRowThreads;
-      uint4 w4 = make_uint4(0u, 0u, 0u, 0u);
-      if (gg < g1) w4 = philox_block(seed, (uint32_t)gg, j, seq, 1u, round_offset);
-      const uint32_t ws[4] = {w4.x, w4.y, w4.z, w4.w};
+    for (int k = 0; k < 2; ++k) {
+      float y4[4];
+      Logit<E>::unpack4(next[k], y4);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int v = 4 * gg + t;
-        if (v < c1 && yv[k][t] > -INFINITY) bonus_race_token(yv[k][t], ws[t], v, c, bEw, byw, bE, by, bi);
-        if (t == 0 && first) warp_best_candidate(bE, by, c, bEw, byw);
+      for (int t = 0; t < 4; ++t) y[4 * k + t] = y4[t];
+      next[k] = after[k];
+    }
+    load(g + 4 * kRowThreads, after);
+    const uint4 wa = philox_block(seed, (uint32_t)g, j, seq, purpose, round_offset);
+    const uint4 wb = philox_block(seed, (uint32_t)(g + kRowThreads), j, seq, purpose, round_offset);
+    const uint32_t ws[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+    if (gw == gw0) {
+      if (4 * g < c1 && y[0] > -INFINITY) eval(y[0], word_to_uniform(ws[0]), 4 * g);
+      refresh();
+    }
+    thr = fminf(thr, order_float(*reinterpret_cast<volatile int*>(s_thr)));
+    const float ym = fmaxf(fmaxf(fmaxf(y[0], y[1]), fmaxf(y[2], y[3])), fmaxf(fmaxf(y[4], y[5]), fmaxf(y[6], y[7])));
+    const uint32_t wm = max(max(max(ws[0], ws[1]), max(ws[2], ws[3])), max(max(ws[4], ws[5]), max(ws[6], ws[7])));
+    const bool pass = word_to_uniform(~wm) < bound(ym);  // word ~w: exactly 1 - u
+    if (__any_sync(0xffffffffu, pass)) {
+      if (pass) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const int v = 4 * (g + (t >> 2) * kRowThreads) + (t & 3);
+          if (v < c1 && y[t] > -INFINITY && word_to_uniform(~ws[t]) < bound(y[t])) eval(y[t], word_to_uniform(ws[t]), v);
+        }
       }
-      first = false;
+      __syncwarp();
+      refresh();
     }
   }
 }
@@ -293,87 +306,6 @@ __device__ __forceinline__ int seq_of_row(const int* start, int B, int r) {
     else hi = mid - 1;
   }
   return lo;
-}
-
-// The smallest key any lane of the warp holds (all 32 lanes take part).
-__device__ __forceinline__ float warp_min_key(float k) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) k = fminf(k, __shfl_xor_sync(0xffffffffu, k, off));
-  return k;
-}
-
-// Residual race of queued entry e over slice s: w_v = max(0, p_v - q_v),
-// key E_v / w_v, uniforms at (v >> 2, n, seq, purpose 1). The screen tests
-// each token against the smaller of the lane's best key and the warp's best
-// at its last refresh (a key some lane has drawn); the trip counts are the
-// warp's, so every lane joins the refreshes.
-template <bool VEC, typename E>
-__device__ __forceinline__ void residual_race_slice(const E* __restrict__ yr, const E* __restrict__ dr, int c0,
-                                                    int c1, int V, float c, float mp, float invZp, float mq,
-                                                    float invZq, uint64_t seed, uint32_t n, uint32_t seq,
-                                                    uint64_t round_offset, float& best, int& besti) {
-  const int g1 = (c1 + 3) >> 2;
-  const int lane = threadIdx.x & 31;
-  float bw = INFINITY;
-  bool first = true;
-  for (int gw = (c0 >> 2) + (int)(threadIdx.x & ~31u); gw < g1; gw += 2 * kRowThreads) {
-    const int g = gw + lane;
-    float yv[2][4], dv[2][4];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int gg = g + k * kRowThreads;
-      if (gg < g1) {
-        if (VEC) {
-          Logit<E>::stream4(yr + 4 * gg, yv[k]);
-          Logit<E>::stream4(dr + 4 * gg, dv[k]);
-        } else {
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int v = 4 * gg + t;
-            yv[k][t] = v < V ? Logit<E>::at(yr, v) : -INFINITY;
-            dv[k][t] = v < V ? Logit<E>::at(dr, v) : 0.f;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          yv[k][t] = -INFINITY;
-          dv[k][t] = 0.f;
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      if (gw + k * kRowThreads >= g1) break;  // the same for the whole warp
-      if (!first) bw = warp_min_key(best);
-      const int gg = g + k * kRowThreads;
-      uint4 w4 = make_uint4(0u, 0u, 0u, 0u);
-      if (gg < g1) w4 = philox_block(seed, (uint32_t)gg, n, seq, 1u, round_offset);
-      const uint32_t ws[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int v = 4 * gg + t;
-        if (v < c1 && gg < g1) {
-          // exponents are <= 0 (below the row maxima), so the fast base-2
-          // exponential is exact to a few ulp
-          const float wv = ex2_approx((yv[k][t] - mp) * c) * invZp - ex2_approx((dv[k][t] - mq) * c) * invZq;
-          if (wv > 0.f) {
-            // E / w < thr  <=>  u > exp(-thr * w): a candidate whose uniform is
-            // below that (with a margin far above the rounding of the test)
-            // cannot win, and skips the logarithm
-            const float u = word_to_uniform(ws[t]);
-            const float thr = fminf(best, bw);
-            if (thr == INFINITY || u > ex2_approx(-thr * wv * kLog2e) * (1.f - 9.5367431640625e-7f)) {
-              const float Ev = -logf(u);
-              argmin_combine(best, besti, __fdividef(Ev, wv), v);
-            }
-          }
-        }
-        if (t == 0 && first) bw = warp_min_key(best);
-      }
-      first = false;
-    }
-  }
 }
 
 // CTA argmin of (key, index); result in thread 0.
@@ -707,6 +639,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) accept_race_kernel(const Accep
   __shared__ int sh[2];
   __shared__ ResEntry s_en;
   __shared__ float s_c;
+  __shared__ int s_thr;
   const int s = blockIdx.x, b = blockIdx.y;
   // a greedy sequence has no draw (and publishes none): its CTAs leave at
   // once, so they hold no slot while the sampling races wait and run
@@ -715,6 +648,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) accept_race_kernel(const Accep
     sh[0] = wait_published(a.ready + b, a.status);
     s_en = a.res[b];
     s_c = log2e_over(a.temperature[b]);  // once per CTA: a binary32 division and reciprocal
+    s_thr = float_order(INFINITY);
   }
   __syncthreads();
   if (!sh[0]) return;
@@ -747,11 +681,30 @@ __global__ void __launch_bounds__(kRowThreads, 4) accept_race_kernel(const Accep
     const E* dr = a.draft + ((size_t)b * K + n) * V;
     const float mq = a.dstat[2 * ((size_t)b * K + n)];
     const float invZq = 1.0f / a.dstat[2 * ((size_t)b * K + n) + 1];
-    residual_race_slice<VEC, E>(yr, dr, c0, c1, V, c, en.mp, en.invZp, mq, invZq, seed, (uint32_t)n, seq,
-                                round_offset, bE, bi);
+    // weight max(0, p - q): at most p, which bounds the key; the drafter's
+    // logit is read for the tokens that pass
+    race_slice<VEC, E>(
+        yr, c0, c1, V, c, __log2f(en.invZp) - en.mp * c, seed, (uint32_t)n, seq, 1u, round_offset, &s_thr,
+        [&]() { return bi == 0x7fffffff ? INFINITY : __log2f(bE); },
+        [&](float y, float u, int v) {
+          // exponents are <= 0 (below the row maxima), so the fast base-2
+          // exponential is exact to a few ulp
+          const float w = ex2_approx((y - en.mp) * c) * en.invZp - ex2_approx((Logit<E>::at(dr, v) - mq) * c) * invZq;
+          if (w > 0.f) argmin_combine(bE, bi, __fdividef(-logf(u), w), v);
+        });
     cta_reduce_min(bE, bi, smk, smi);
   } else {
-    bonus_race_slice<VEC, E>(yr, c0, c1, V, c, seed, (uint32_t)n, seq, round_offset, bE, by, bi);
+    race_slice<VEC, E>(
+        yr, c0, c1, V, c, 0.f, seed, (uint32_t)n, seq, 1u, round_offset, &s_thr,
+        [&]() { return bE < INFINITY ? __log2f(bE) - by * c : INFINITY; },
+        [&](float y, float u, int v) {
+          const float Ev = -logf(u);
+          if (!(bE < INFINITY) || Ev < bE * ex2_approx((y - by) * c)) {
+            bE = Ev;
+            by = y;
+            bi = v;
+          }
+        });
     cta_reduce_race(bE, by, bi, c, smk, smy, smi);
   }
   if (tid == 0) {
@@ -824,20 +777,19 @@ __global__ void selftest_wait_kernel(const uint32_t* __restrict__ flag, uint64_t
 // at once. A greedy sequence (temperature 0) takes the argmax of the node's
 // target row; a sampling one draws from softmax(row / T) by the exponential
 // race x = argmin_v key_v, key_v = log2(E_v) - y_v log2(e) / T, E_v = -ln u_v,
-// u_v from Philox at (v >> 2, node t, sequence, purpose 2), word v & 3. The
-// race is carried as an argmax of -key so the partials merge like argmaxes
-// (lowest index on ties). A candidate can only win if key_v < best, i.e.
-// u_v > exp(-2^(best + y_v c)); that test (two fast exponentials, with a
-// margin above their error) skips the logarithms of almost every token.
+// u_v from Philox at (v >> 2, node t, sequence, purpose 2), word v & 3
+// (race_slice). The race is carried as an argmax of -key so the partials
+// merge like argmaxes (lowest index on ties).
 // The draw of node t lands in stat[b, t].arg for the walk.
 // ---------------------------------------------------------------------------
 template <bool VEC, typename E>
-__global__ void __launch_bounds__(kRowThreads) tree_rows_kernel(
+__global__ void __launch_bounds__(kRowThreads, 4) tree_rows_kernel(
     const E* __restrict__ target, const int32_t* __restrict__ Ls, const float* __restrict__ temperature, int K,
     int V, int nsplit, int chunk, uint64_t seed, uint64_t round_offset, uint32_t seq_offset,
     RowPartial* __restrict__ part, uint32_t* __restrict__ cnt, RowStat* __restrict__ stat, int* __restrict__ status) {
   __shared__ float smf[64];
   __shared__ int smi[32];
+  __shared__ int s_thr;
   __shared__ int last;
   const int split = blockIdx.x, j = blockIdx.y, b = blockIdx.z;
   const int Lb = Ls[b];
@@ -865,48 +817,11 @@ __global__ void __launch_bounds__(kRowThreads) tree_rows_kernel(
     const uint32_t seq = seq_offset + (uint32_t)b;
     float best = INFINITY;
     int besti = 0x7fffffff;
-    // the screen's threshold: the smaller of the lane's best key and the
-    // warp's best at its last refresh (a key some lane has drawn), refreshed
-    // after the first token and then before groups 1, 2, 3 and every fourth;
-    // the trip counts are the warp's, so every lane joins the refreshes
-    float bw = INFINITY;
-    const int lane = threadIdx.x & 31;
-    int it = 0;
-    for (int gw = (c0 >> 2) + (int)(threadIdx.x & ~31u); 4 * gw < c1; gw += kRowThreads, ++it) {
-      if (it > 0 && (it < 4 || (it & 3) == 0)) bw = warp_min_key(best);
-      const int g = gw + lane;
-      const bool live = 4 * g < c1;
-      uint4 w4 = make_uint4(0u, 0u, 0u, 0u);
-      float yv[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-      if (live) {
-        w4 = philox_block(seed, (uint32_t)g, (uint32_t)j, seq, 2u, round_offset);
-        if (VEC) {
-          Logit<E>::stream4(xr + 4 * g, yv);
-        } else {
-#pragma unroll
-          for (int t = 0; t < 4; ++t) yv[t] = 4 * g + t < V ? Logit<E>::at(xr, 4 * g + t) : -INFINITY;
-        }
-      }
-      const uint32_t ws[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int v = 4 * g + t;
-        const float yc = yv[t] * c;
-        if (v < c1 && yc > -INFINITY) {
-          const float u = word_to_uniform(ws[t]);
-          // key < thr  <=>  u > exp(-2^(thr + yc)) =: h. The fast exponentials
-          // give h to a relative 2e-4 while h is a normal float (exponent above
-          // -150; below, h flushes to 0 and every candidate passes): a margin of
-          // 2^-12 keeps every possible winner, whose key is then compared exactly.
-          const float thr = fminf(best, bw);
-          if (thr == INFINITY || u > ex2_approx(-ex2_approx(thr + yc) * kLog2e) * 0.999755859375f) {
-            const float key = log2f(-logf(u)) - yc;
-            argmin_combine(best, besti, key, v);
-          }
-        }
-        if (t == 0 && it == 0) bw = warp_min_key(best);
-      }
-    }
+    if (threadIdx.x == 0) s_thr = float_order(INFINITY);
+    __syncthreads();
+    race_slice<VEC, E>(
+        xr, c0, c1, V, c, 0.f, seed, (uint32_t)j, seq, 2u, round_offset, &s_thr, [&]() { return best; },
+        [&](float y, float u, int v) { argmin_combine(best, besti, log2f(-logf(u)) - y * c, v); });
     m = -best;
     arg = besti;
   }
@@ -1025,7 +940,11 @@ cudaError_t launch_accept_tree(const T* target, const int32_t* tokens, const int
   auto* st = reinterpret_cast<int*>(ws + lay.status);
   auto* rstat = reinterpret_cast<RowStat*>(ws + lay.row_stat);
   const long rows = (long)B * (K + 1);
-  const int nsplit0 = row_splits(rows, V, sms, kRowMaxSplits, 4096);
+  // The draws' rows: as few slices as make one wave of resident CTAs (4 per SM), since a race settles its threshold
+  // anew in each (2 trees of 257 nodes: 100 us at 16 CTAs per SM, 94 at 8, 90 at 4, 99 at 2); the argmax rows: more,
+  // for the loads.
+  const int nsplit0 = temperature == nullptr ? row_splits(rows, V, sms, kRowMaxSplits, 4096)
+                                             : wave_splits(rows, V, 4L * sms, kRowMaxSplits, 4096);
   const int chunk = row_chunk(V, nsplit0);
   const int nsplit = (V + chunk - 1) / chunk;
   dim3 grid(nsplit, K + 1, B);

@@ -229,8 +229,18 @@ struct Logit<float> {
     const float4 a = ld_stream4(p);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
   }
-  // 4 elements from an address aligned to 4 elements
-  __device__ static __forceinline__ void stream4(const float* p, float (&v)[4]) { stream_vec(p, v); }
+  // 4 elements as loaded (from an address aligned to 4 elements), their values, and four of minus infinity
+  using Raw4 = float4;
+  __device__ static __forceinline__ Raw4 load4(const float* p) { return ld_stream4(p); }
+  __device__ static __forceinline__ void unpack4(Raw4 a, float (&v)[4]) {
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  }
+  __device__ static __forceinline__ Raw4 none4() { return make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY); }
+  // the first n elements from any address, minus infinity for the rest
+  __device__ static __forceinline__ Raw4 gather4(const float* p, int n) {
+    return make_float4(n > 0 ? p[0] : -INFINITY, n > 1 ? p[1] : -INFINITY, n > 2 ? p[2] : -INFINITY,
+                       n > 3 ? p[3] : -INFINITY);
+  }
 };
 
 template <>
@@ -252,10 +262,20 @@ struct Logit<uint16_t> {
     v[0] = bf16_lo(w0); v[1] = bf16_hi(w0); v[2] = bf16_lo(w1); v[3] = bf16_hi(w1);
     v[4] = bf16_lo(w2); v[5] = bf16_hi(w2); v[6] = bf16_lo(w3); v[7] = bf16_hi(w3);
   }
-  __device__ static __forceinline__ void stream4(const uint16_t* p, float (&v)[4]) {
-    uint32_t w0, w1;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(w0), "=r"(w1) : "l"(p));
-    v[0] = bf16_lo(w0); v[1] = bf16_hi(w0); v[2] = bf16_lo(w1); v[3] = bf16_hi(w1);
+  using Raw4 = uint2;
+  __device__ static __forceinline__ Raw4 load4(const uint16_t* p) {
+    uint2 w;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(w.x), "=r"(w.y) : "l"(p));
+    return w;
+  }
+  __device__ static __forceinline__ void unpack4(Raw4 w, float (&v)[4]) {
+    v[0] = bf16_lo(w.x); v[1] = bf16_hi(w.x); v[2] = bf16_lo(w.y); v[3] = bf16_hi(w.y);
+  }
+  __device__ static __forceinline__ Raw4 none4() { return make_uint2(0xff80ff80u, 0xff80ff80u); }
+  __device__ static __forceinline__ Raw4 gather4(const uint16_t* p, int n) {
+    const uint32_t a = n > 0 ? p[0] : 0xff80u, b = n > 1 ? p[1] : 0xff80u, c = n > 2 ? p[2] : 0xff80u,
+                   d = n > 3 ? p[3] : 0xff80u;
+    return make_uint2(a | (b << 16), c | (d << 16));
   }
 };
 

@@ -230,17 +230,22 @@ __device__ __forceinline__ void warp_merge_partials(const RowPartial* __restrict
   s_out = s;
 }
 
-// Choose how many CTAs share a row: enough CTAs in total to fill the GPU
-// several times over, each with at least min_elems elements.
-inline int row_splits(long rows, int V, int num_sms, int max_splits, int min_elems) {
+// CTAs that share a row, for `target` CTAs in total, each with at least
+// min_elems elements.
+inline int wave_splits(long rows, int V, long target, int max_splits, int min_elems) {
   if (rows <= 0) return 1;
-  const long target = 2L * 8 * num_sms;
   long ns = (target + rows - 1) / rows;
-  const long cap = (V + min_elems - 1) / min_elems;  // at least min_elems per CTA
+  const long cap = (V + min_elems - 1) / min_elems;
   if (ns > cap) ns = cap;
   if (ns > max_splits) ns = max_splits;
   if (ns < 1) ns = 1;
   return (int)ns;
+}
+
+// Choose how many CTAs share a row: enough CTAs in total to fill the GPU
+// several times over.
+inline int row_splits(long rows, int V, int num_sms, int max_splits, int min_elems) {
+  return wave_splits(rows, V, 2L * 8 * num_sms, max_splits, min_elems);
 }
 
 // Splits per drafter row for the confidence pass: the fewest that give about
@@ -250,14 +255,7 @@ inline int row_splits(long rows, int V, int num_sms, int max_splits, int min_ele
 // rows 37.2 us at 10 splits, 33.1 at 3; ragged's 2048 rows 156.7 us at 2,
 // 152.2 at 1).
 inline int conf_row_splits(long rows, int V, int num_sms, int max_splits, int min_elems) {
-  if (rows <= 0) return 1;
-  const long target = (6L * 8 * num_sms + 9) / 10;
-  long ns = (target + rows - 1) / rows;
-  const long cap = (V + min_elems - 1) / min_elems;
-  if (ns > cap) ns = cap;
-  if (ns > max_splits) ns = max_splits;
-  if (ns < 1) ns = 1;
-  return (int)ns;
+  return wave_splits(rows, V, (6L * 8 * num_sms + 9) / 10, max_splits, min_elems);
 }
 
 // Split length: a multiple of 8 elements (whole 128-bit loads of fp32 or bf16).

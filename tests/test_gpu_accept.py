@@ -172,3 +172,37 @@ def test_accept_race_degenerate_rows(orc, V):
         assert bonus[2] == 17 or flag[2], "the dominant token wins the bonus draw"
         assert bonus[4] in (3, V // 2, V - 1) and bonus[1] % 2 == 1, "only finite logits can be drawn"
     assert unflagged >= 16, "%d of 20 draws unflagged" % unflagged
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [5, 1023, 2048, 4104, 9001])
+@pytest.mark.parametrize("scale,T", [(0.0, 1.0), (3.0, 0.8), (30.0, 0.3), (3000.0, 1.0)])
+def test_races_on_flat_steep_and_short_rows(orc, dtype, V, scale, T):
+    """The races dismiss eight tokens by one bound: flat rows (every token near the bound), steep ones (its
+    exponentials overflow and underflow, |y c| up to 1e4), rows shorter than a warp and ragged last groups, for the
+    chain's draws and a tree's. A draw may differ only where the oracle flags it (keys within binary32 rounding)."""
+    B, K = 12, 3
+    g = torch.Generator(device="cuda").manual_seed(V + int(scale))
+    tgt = (torch.randn((B, K + 1, V), generator=g, device=cuda()) * scale).to(dtype)
+    dr = (tgt[:, :K].float() + torch.randn((B, K, V), generator=g, device=cuda())).to(dtype)
+    # the drafter's argmax (q >= 1/V): a random token of a steep row has p and q below binary32's range, and the
+    # decision then compares 0 with 0 where binary64 does not, whatever the draws do
+    tok = dr.argmax(-1).int()
+    temp = torch.full((B,), T, device=cuda())
+    inp = {"target_logits": tgt, "draft_logits": dr, "draft_tokens": tok, "temperature": temp}
+    wide = dict(inp, target_logits=tgt.float(), draft_logits=dr.float())  # (widened exactly)
+    L = np.arange(B, dtype=np.int32) % (K + 1)
+    n, bonus = _gpu_accept(inp, L, 77, round_offset=2)
+    n_ref, b_ref, flag = _oracle_accept(orc, wide, L, 77, round_offset=2)
+    assert_exact_unless_flagged(n, n_ref, flag, "n_accepted")
+    assert_exact_unless_flagged(bonus, b_ref, flag, "bonus_token")
+    par = torch.from_numpy(workloads.draft_tree(B, K, K, 5, "random")).to(cuda())
+    L_t = torch.full((B,), K, dtype=torch.int32, device=cuda())
+    ws = lr.Workspace(B, K, V, device=cuda())
+    out = lr.libraspec_accept_tree(tgt, tok, par, L_t, temp, 78, ws, round_offset=3)
+    torch.cuda.synchronize()
+    assert lr.libraspec_get_status(ws) == 0
+    *ref, flag = orc.accept_tree(wide["target_logits"].cpu().numpy(), tok.cpu().numpy(), par.cpu().numpy(),
+                                 L_t.cpu().numpy(), temp.cpu().numpy(), 78, 3)
+    for a, r, what in zip(out, ref, ("n_accepted", "last_node", "bonus_token")):
+        assert_exact_unless_flagged(a.cpu().numpy(), r, flag, what)
