@@ -5,52 +5,56 @@
 // Work decomposition. For sequence b the verified block has M_b = (L_b+1)*g
 // query rows per kv head (g = Hq/Hkv; row r is block position t = r / g of
 // query head kvh*g + r % g) and N_b = kv_len_b + L_b + 1 visible keys. Rows
-// are cut into units of RU = g * floor(128/g) (whole block positions, at most
-// 128: one tcgen05 M=128 tile), units into row groups (one unit; two where
-// (K+1)*g rows may not fit one) and keys into 64-key tiles. All (row group,
-// key tile) pairs of the batch form one tile sequence (sequence-major, then kv
+// are cut into groups of R = g * floor(128/g) (whole block positions, at most
+// 128: one tcgen05 M=128 tile) and keys into 64-key tiles. All (row group, key
+// tile) pairs of the batch form one tile sequence (sequence-major, then kv
 // head, row group, key tile); CTA c of the persistent grid (one CTA per SM)
-// takes a contiguous range of it, cut by cost (each row group weighs its
-// tiles plus an item's fixed cost; tile_of_weighted), so that CTAs finish
-// together whatever the ragged lengths. The plan is derived on the device from L[] and kv_len[] by every CTA, and it
-// is the same for every layer (all layers share L and kv_len).
+// takes a contiguous range of it: with equal groups its part of one group
+// (aligned_ctas), else a range cut by cost (each row group weighs its tiles
+// plus an item's fixed cost; tile_of_weighted), so that CTAs finish together
+// whatever the ragged lengths. The plan is derived on the device from L[] and
+// kv_len[] by every CTA, and it is the same for every layer (all layers share
+// L and kv_len).
 //
 // Two streams per CTA. An item (a run of tiles of one row group) is worked on
-// in steps of 128 keys by two streams, each with its own softmax warpgroup,
-// scores and O accumulator, so that one stream's MMAs run beside the other's
-// softmax. A group of one unit: tiles alternate between the streams, which
-// hold the same rows, and the epilogue combines their (O, m, l). A group of
-// two units (large trees): every tile is read once from shared memory by both
-// streams, each for its own unit. One softmax warpgroup over 64-key tiles was
-// the limit before: with few rows one warp holds them all, and its 1150
-// cycles per 64-key tile did not keep up with HBM. 8 sequences of 131072 keys
-// (64/8 heads): 771 -> 603 us (105% of the copy rate); B = 64 ragged: 327 ->
-// 294; 32 layers at B = 1: 311 -> 268; a 512-node tree, 4 layers: 369 -> 351.
+// in steps of 128 keys by two streams in turn, each with its own softmax
+// warpgroup, scores and O accumulator, so that one stream's MMAs run beside
+// the other's softmax; the epilogue combines the streams' (O, m, l). One
+// softmax warpgroup over 64-key tiles was the limit before: with few rows one
+// warp holds them all, and its 1150 cycles per 64-key tile did not keep up
+// with HBM, and large trees left the tensor cores idle three quarters of the
+// time. 8 sequences of 131072 keys (64/8 heads): 771 -> 606 us (104% of the
+// copy rate); B = 64 ragged: 326 -> 292; 32 layers at B = 1: 302 -> 254; a
+// 512-node tree, 4 layers: 367 -> 227.
 //
-// Roles in a CTA (384 threads' worth of registers, 352 threads):
+// Roles in a CTA (384 threads):
 //  * producer warp: walks the CTA's range layer after layer in items; loads
-//    the group's Q rows (one 3-D TMA box per 64-column half and unit: RU/g
-//    positions x g heads) into a Q slot (two slots where groups may have two
-//    units, else one and a fifth chunk) and K and V of the tiles (3-D TMA,
-//    128-byte swizzle) into a ring of chunks (K or V of 128 keys), in the
-//    order in which the MMA warp uses them;
+//    the group's Q rows (one 3-D TMA box per 64-column half: R/g positions x g
+//    heads) and K and V of the tiles (3-D TMA, 128-byte swizzle) into a ring
+//    of chunks (K or V of 128 keys), in the order in which the MMA warp uses
+//    them;
 //  * MMA warp: one thread issues S = Q K^T (tcgen05.mma, A and B K-major from
 //    shared memory, fp32 accumulator in tensor memory) and O += P V (A = P
 //    from tensor memory, B = V MN-major from shared memory), and signals
 //    completions with tcgen05.commit;
 //  * softmax warpgroups (thread i <-> tensor-memory lane i = row i of the
-//    unit): read S, mask keys beyond kv_len_b + t, keep the online softmax in
+//    group): read S, mask keys beyond kv_len_b + t, keep the online softmax in
 //    the log2 domain, write P (bf16) over the scores they have read, and at
 //    the end of an item normalise O and store it (or a split partial);
-//  * merge warp: merges the split groups of earlier layers.
+//  * two merge warps: merge the split groups of earlier layers; every warp
+//    helps with the last layer's.
 // Registers are what the roles' code must fit: with the merge's calls in the
 // softmax path 120 bytes of spills made every wait and epilogue wait for
-// local memory behind the K/V stream (B = 1: 361 us), so the merge is inline,
-// holds 12 loads per lane and is entered at one place.
-// The running max is only raised when a tile's max exceeds it by more than 8
-// (a factor 2^8), so O is rescaled in tensor memory rarely; p <= 2^8 keeps
-// bf16 P and fp32 O exact in range, and O / l is unchanged by the choice of
-// reference max.
+// local memory behind the K/V stream (B = 1: 361 us instead of 268), so the
+// merge is one inline copy outside the roles and holds 12 loads per lane.
+// Scores are read once: the reference max of a row is that of its first 32
+// keys in the item, raised only when a later key exceeds it by more than 8 (a
+// factor 2^8), so O is rescaled in tensor memory rarely; p <= 2^8 keeps bf16
+// P and fp32 O in range, and O / l is unchanged by the choice of reference.
+// (A pass for the tile's max before the one that forms P: the 512-node tree 332
+// us instead of 320, all else equal. Two copies of the 32-key step, the second
+// chunk's loads issued ahead, were slower, 337 and B = 1 290 instead of 265:
+// the role loops are bound by instruction fetches as soon as they are long.)
 //
 // Layers. Layer l+1 may read Q, the block's own keys (positions >= kv_len_b)
 // and layer l's partials only after every CTA has finished layer l: a
@@ -85,8 +89,8 @@ constexpr int kStreams = 2;                    // softmax warpgroups (tile strea
 constexpr int kSoftmaxWarps = 4 * kStreams;
 constexpr int kProducerWarp = kSoftmaxWarps;
 constexpr int kMmaWarp = kSoftmaxWarps + 1;
-constexpr int kMergeWarp = kSoftmaxWarps + 2;
-constexpr int kAttnThreads = (kSoftmaxWarps + 3) * 32;
+constexpr int kMergeWarp = kSoftmaxWarps + 2;  // the first of two
+constexpr int kAttnThreads = (kSoftmaxWarps + 4) * 32;
 constexpr int kMaxWaitIters = 1 << 24;
 constexpr int kSoftmaxBar = 1;  // named barrier of the softmax warpgroups
 constexpr float kRescaleLog2 = 8.f;
@@ -162,12 +166,13 @@ __device__ __forceinline__ SeqPlan seq_plan(int b, int B, const int32_t* kv_len,
   return p;
 }
 
-// Warp-wide: total tiles T of the batch and its row groups (*groups);
-// flags invalid sequences.
+// Warp-wide: total tiles T of the batch, its row groups (*groups) and the tiles
+// of every group if they have the same (*equal, else 0); flags invalid sequences.
 __device__ long long total_tiles(int B, const int32_t* kv_len, const int32_t* Ls, int K, int g, int R, int Hkv,
-                                 int S_cap, int* status, bool report, long long* groups) {
+                                 int S_cap, int* status, bool report, long long* groups, int* equal) {
   const int lane = threadIdx.x & 31;
   long long tot = 0, ng = 0;
+  int t_min = 0x7fffffff, t_max = 0;
   bool bad = false;
   for (int b = lane; b < B; b += 32) {
     const SeqPlan p = seq_plan(b, B, kv_len, Ls, K, g, R, S_cap);
@@ -175,8 +180,13 @@ __device__ long long total_tiles(int B, const int32_t* kv_len, const int32_t* Ls
     else {
       tot += (long long)Hkv * p.n_mg * p.n_tiles;
       ng += (long long)Hkv * p.n_mg;
+      t_min = min(t_min, p.n_tiles);
+      t_max = max(t_max, p.n_tiles);
     }
   }
+  t_min = __reduce_min_sync(0xffffffffu, t_min);
+  t_max = __reduce_max_sync(0xffffffffu, t_max);
+  *equal = t_min == t_max ? t_max : 0;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     tot += __shfl_xor_sync(0xffffffffu, tot, off);
@@ -300,6 +310,22 @@ __device__ long long tile_of_weighted(long long x, long long W, long long T, int
   return T;
 }
 
+// Equal groups. Where every row group has the same number nt of tiles (one
+// sequence, or equal caches) and the NG groups fit the grid, each group may
+// get p = G / NG CTAs of its own: no CTA has two items, and a group of p = 1
+// is never split nor merged. Taken when the longest range, nt / p tiles, is
+// at most kAlignTiles above the even split's T / G (an extra item and its
+// merge cost a CTA about that much). 512 nodes (136 groups of 128 rows, 4
+// layers): 227 us; cut by cost, 353; with row groups of 256 rows, which read
+// each tile once for both halves but are split and merged, 320.
+constexpr int kAlignTiles = 10;
+__device__ __forceinline__ int aligned_ctas(long long T, long long NG, int nt, int G) {
+  if (nt <= 0 || NG > G) return 0;
+  const int p = min((int)(G / NG), nt);
+  const long long longest = (nt + p - 1) / p;
+  return longest * G <= T + (long long)kAlignTiles * G ? p : 0;
+}
+
 // Weighted position of tile t of global row group `group` (the groups up to
 // and including it each put C before their tiles).
 __device__ __forceinline__ long long weighted_pos(long long t, long long group, int C) {
@@ -319,15 +345,12 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* ctr, uint32_t targe
 
 // One item handed from the producer to the MMA and softmax warps.
 struct ItemInfo {
-  int b, kvh, mg, kv;
-  int rows0, rows1;  // rows of the group's two units of up to 128 rows
+  int b, kvh, mg, rows, kv;
   int key0, key1;  // keys [key0, key1)
-  int both;        // 1: stream s takes unit s, every tile; 0: one unit, tiles alternate between the streams
-  int qslot;       // Q slot of the first unit
   int partial;     // 1: write a partial, else write O
   int slot;        // partial slot
   int grp;         // global row group index
-  int pad[3];
+  int pad[6];
 };
 static_assert(sizeof(ItemInfo) == 64, "items lie in 64-byte slots");
 
@@ -358,20 +381,17 @@ struct LayerSet {
 };
 static_assert(sizeof(LayerSet) <= 32000, "kernel parameters are limited to 32764 bytes");
 
-// QS Q slots: one (and room for one more K/V chunk at d = 128) where a row
-// group is always one unit, two where it may have two.
-template <int D, int QS>
+template <int D>
 struct AttnSmem {
   static constexpr int kBoxes = D / 64;
   static constexpr int kChunkBytes = kBoxes * 16384;     // K or V of one 128-key tile
-  static constexpr int kChunks = D == 128 ? 6 - QS : 10;  // in the ring
-  static constexpr int kQSlot = kBoxes * 16384;          // one unit: per 64 columns 128 rows
-  static constexpr int kQ = 0;
-  static constexpr int kRing = kQ + QS * kQSlot;
-  // mbarriers: full[chunks], empty[chunks], qfull[2], qempty[2], ifull[2], iempty[2], sfull[2], pfull[2], pvdone[2],
+  static constexpr int kChunks = D == 128 ? 5 : 10;      // in the ring
+    static constexpr int kQ = 0;
+  static constexpr int kRing = kQ + kBoxes * 16384;      // (Q: per 64 columns 128 rows)
+  // mbarriers: full[chunks], empty[chunks], ifull[2], iempty[2], sfull[2], pfull[2], pvdone[2], qfull, qempty,
   // ofree, drain
   static constexpr int kBar = kRing + kChunks * kChunkBytes;
-  static constexpr int kNumBars = 2 * kChunks + 7 * 2 + 2;
+  static constexpr int kNumBars = 2 * kChunks + 5 * 2 + 4;
   static constexpr int kInfo = kBar + ((8 * kNumBars + 63) / 64) * 64;
   static constexpr int kTasks = kInfo + 2 * 64;
   static constexpr int kTmem = kTasks + 64;
@@ -417,13 +437,6 @@ __device__ __forceinline__ int merge_share(const MergeTask& t, int& u0) {
   return (int)((long long)t.rows * (k_me + 1) / t.np) - u0;
 }
 
-// Between layers the softmax warps help with a merge of at least this many
-// chunks; a smaller one is left to the merge warp, which keeps cold code off
-// the softmax warps' path from one layer to the next (instruction fetch
-// misses cost about a memory round trip). The last layer's merge, the tail
-// of the launch, is always shared.
-constexpr int kMergeHelpChunks = 8;
-
 constexpr int kMergeLoads = 12;  // of a lane in flight (16 spill registers in the callers)
 
 // Items per lane in a chunk of a group of np parts: J items x 12/J parts are
@@ -453,7 +466,7 @@ __device__ __forceinline__ int merge_chunk_count(const MergeTask* tasks, int n_t
 // Chunk lc of task t: items (lc*J + j)*32 + lane, j < J.
 template <int J, int D>
 __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, int lc, const float* __restrict__ part_o,
-                                            const float* __restrict__ part_ml, int K, int Hq, int g, int R, int slot_rows,
+                                            const float* __restrict__ part_ml, int K, int Hq, int g, int R,
                                             __nv_bfloat16* __restrict__ O, float* __restrict__ lse) {
   constexpr int PB = kMergeLoads / J, C4 = D / 4;
   const int lane = threadIdx.x & 31;
@@ -477,7 +490,7 @@ __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, 
       for (int k = 0; k < PB; ++k) {
         const int p = p0 + k;
         if (i < items && p < np) {
-          const size_t at = (size_t)(p == 0 ? 2 * c0 + 1 : 2 * (c0 + p)) * slot_rows + u0 + r;
+          const size_t at = (size_t)(p == 0 ? 2 * c0 + 1 : 2 * (c0 + p)) * kAttnRows + u0 + r;
           ml[j][k] = __ldcg(reinterpret_cast<const float2*>(part_ml + at * 2));
           v[j][k] = __ldcg(reinterpret_cast<const float4*>(part_o + at * D) + c);
         } else {
@@ -532,7 +545,7 @@ __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, 
 // CTA's monotonic counters; ctr_done counts the chunks merged (stores done).
 template <int D>
 __device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set, const MergeTask* tasks, int n_tasks, int C,
-                             int* ctr_claim, int* ctr_done, int K, int Hq, int Hkv, int R, int slot_rows,
+                             int* ctr_claim, int* ctr_done, int K, int Hq, int Hkv, int R,
                              const float* __restrict__ part_buf_o, const float* __restrict__ part_buf_ml,
                              size_t part_o_stride, size_t part_ml_stride) {
   const int lane = threadIdx.x & 31;
@@ -566,8 +579,8 @@ __device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set
     }
     if (ti < n_tasks) {
       const MergeTask& t = tasks[ti];
-      if (merge_j(t.np, nr * (D / 4)) == 1) merge_chunk<1, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, slot_rows, O, lse);
-      else merge_chunk<4, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, slot_rows, O, lse);
+      if (merge_j(t.np, nr * (D / 4)) == 1) merge_chunk<1, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
+      else merge_chunk<4, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
     }
     __syncwarp();
     if (lane == 0) atomicAdd(ctr_done, 1);
@@ -581,30 +594,30 @@ __device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set
 // tree_vis (optional, [B, K+1, tree_words]): the block is a draft tree and
 // row t sees the block keys of the set bits (bit j <-> block position j + 1)
 // besides the root and the prefix; nullptr: the chain draft (block-causal).
-template <int D, int QS, bool PAGED>
+template <int D, bool PAGED>
 __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     const __grid_constant__ LayerSet set, const int32_t* __restrict__ kv_len, const int32_t* __restrict__ Ls,
     const uint64_t* __restrict__ tree_vis, int tree_words,
     const int32_t* __restrict__ block_table, int max_pages, int page_size, int n_pages, int page_cache,
-    int B, int K, int Hq, int Hkv, int S_cap, float scale_log2, int min_tiles, int item_tiles, int slot_rows,
+    int B, int K, int Hq, int Hkv, int S_cap, float scale_log2, int min_tiles, int item_tiles,
     float* __restrict__ part_buf_o,
     float* __restrict__ part_buf_ml, size_t part_o_stride, size_t part_ml_stride, uint32_t* __restrict__ bar_cnt,
     uint32_t* __restrict__ grp_cnt, int* __restrict__ status) {
-  using SM = AttnSmem<D, QS>;
+  using SM = AttnSmem<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sQ = smem_u32(smem + SM::kQ);
   const uint32_t sRing = smem_u32(smem + SM::kRing);
   const uint32_t bFull = smem_u32(smem + SM::kBar);
   const uint32_t bEmpty = bFull + 8 * SM::kChunks;
-  const uint32_t bQFull = bEmpty + 8 * SM::kChunks;
-  const uint32_t bQEmpty = bQFull + 16;
-  const uint32_t bIFull = bQEmpty + 16;
+  const uint32_t bIFull = bEmpty + 8 * SM::kChunks;
   const uint32_t bIEmpty = bIFull + 16;
   const uint32_t bSFull = bIEmpty + 16;   // [stream]
   const uint32_t bPFull = bSFull + 16;    // [stream]
   const uint32_t bPVDone = bPFull + 16;   // [stream]
-  const uint32_t bOFree = bPVDone + 16;
+  const uint32_t bQFull = bPVDone + 16;
+  const uint32_t bQEmpty = bQFull + 8;
+  const uint32_t bOFree = bQEmpty + 8;
   const uint32_t bDrain = bOFree + 8;
   ItemInfo* info = reinterpret_cast<ItemInfo*>(smem + SM::kInfo);
   MergeTask* tasks = reinterpret_cast<MergeTask*>(smem + SM::kTasks);
@@ -614,7 +627,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = Hq / Hkv;
-  const int RU = attn_unit_rows(g), R = QS * RU;  // rows per unit and per row group
+  const int R = g * (kAttnRows / g);  // rows per group: whole block positions
   const int n_layers = set.n;
   const uint32_t n_ctas = gridDim.x;
   // the tensor maps' first use then finds them on chip
@@ -637,14 +650,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       mbar_init(bEmpty + 8 * s, 1);  // the MMA warp's commit after the chunk's last use
     }
     for (int q = 0; q < 2; ++q) {
-      mbar_init(bQFull + 8 * q, 1);                   // the producer's arrive; Q bytes as transactions
-      mbar_init(bQEmpty + 8 * q, 1);                  // the MMA warp's commit after the item's last S
       mbar_init(bIFull + 8 * q, 1);
       mbar_init(bIEmpty + 8 * q, 1 + kSoftmaxWarps);  // the item has been read
       mbar_init(bPFull + 8 * q, 4);
       mbar_init(bPVDone + 8 * q, 1);
       mbar_init(bSFull + 8 * q, 1);
     }
+    mbar_init(bQFull, 1);   // the producer's arrive; Q bytes as transactions
+    mbar_init(bQEmpty, 1);  // the MMA warp's commit after the item's last S
     mbar_init(bOFree, kSoftmaxWarps);
     mbar_init(bDrain, 1);
     misc[0] = 0;
@@ -686,7 +699,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       __syncwarp();
     }
     long long NG = 0;
-    const long long T = total_tiles(B, kvs, Lss, K, g, R, Hkv, S_cap, status, blockIdx.x == 0, &NG);
+    int equal = 0;
+    const long long T = total_tiles(B, kvs, Lss, K, g, R, Hkv, S_cap, status, blockIdx.x == 0, &NG, &equal);
     int G = (int)n_ctas;
     if (T > 0) {
       const long long g_cap = div_nn(T + min_tiles - 1, min_tiles);
@@ -696,8 +710,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     // an item's fixed cost in tiles, less where a CTA has few
     const int C = T > 0 ? (int)min((long long)item_tiles, div_nn(T, 4 * (long long)G)) : 0;
     const long long W = T + (long long)C * NG;  // weighted length
+    const int p_cta = aligned_ctas(T, NG, equal, G);  // > 0: CTAs of each group
     long long lo = 0, hi = 0;
-    if (T > 0 && c < G) {
+    if (p_cta > 0) {
+      const int grp = c / p_cta, k = c - grp * p_cta;
+      if (grp < NG) {
+        lo = (long long)grp * equal + equal * k / p_cta;
+        hi = (long long)grp * equal + equal * (k + 1) / p_cta;
+      }
+    } else if (T > 0 && c < G) {
       lo = range_lo(c, W, G);
       hi = range_lo(c + 1, W, G);
       if (C > 0) {
@@ -729,8 +750,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             t.kvh = gib / loc.p.n_mg;
             t.mg = gib % loc.p.n_mg;
             t.rows = min(R, loc.p.M - t.mg * R);
-            t.c0 = cta_of(weighted_pos(gstart, group, C), W, G);
-            t.np = cta_of(weighted_pos(gend - 1, group, C), W, G) - t.c0 + 1;
+            t.c0 = p_cta > 0 ? group * p_cta : cta_of(weighted_pos(gstart, group, C), W, G);
+            t.np = p_cta > 0 ? p_cta : cta_of(weighted_pos(gend - 1, group, C), W, G) - t.c0 + 1;
             t.grp = group;
             tasks[n_tasks] = t;
           }
@@ -814,13 +835,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       __syncwarp();
     }
     uint32_t item_ctr = 0, chunk_ctr = 0;           // items; chunks filled
-    uint32_t q_loads = 0, q_any = 0;                // bit q: parity of the units loaded into Q slot q; any loaded
-    int q_next = 0, q_last = -1;                    // next slot of a one-unit item; a slot of the last item
     // the next chunk may be filled
     auto chunk_free = [&]() { return bEmpty + 8 * (chunk_ctr % SM::kChunks); };
     auto chunk_parity = [&]() { return ((chunk_ctr / SM::kChunks) & 1) ^ 1; };
-    // Q slot q's last unit has been read
-    auto q_parity = [&](int q) { return ((q_loads >> q) & 1u) ^ 1u; };
     for (int layer = 0; layer < n_layers && !aborted(); ++layer) {
       // layer's dependent data (Q, the block's keys) is readable once every
       // CTA has finished the previous layer
@@ -836,17 +853,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         it.b = loc.b;
         it.kvh = gib / loc.p.n_mg;
         it.mg = gib % loc.p.n_mg;
-        const int rows = min(R, loc.p.M - it.mg * R);
-        it.rows0 = min(rows, RU);
-        it.rows1 = rows - it.rows0;
-        it.both = it.rows1 > 0;
+        it.rows = min(R, loc.p.M - it.mg * R);
         it.kv = kvs[loc.b];
         it.key0 = (int)(pos - gstart) * kAttnTileKeys;
         it.key1 = min(loc.p.N, (int)(iend - gstart) * kAttnTileKeys);
         it.partial = ((pos == gstart) && (gend <= hi)) ? 0 : 1;
         it.slot = (pos == gstart) ? 2 * c + 1 : 2 * c;
         it.grp = loc.group0 + gib;
-        it.qslot = it.both || QS == 1 ? 0 : q_next;
         const int n_half = (int)(iend - pos), n_tiles = (n_half + 1) >> 1;
         const int zc = loc.b * Hkv + it.kvh;
         const long long item_pos = pos;  // the item's first 64-key tile in the tile sequence
@@ -854,7 +867,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         if (lane == 0) {
           // The ring is filled in the order in which the MMA warp uses it: K of
           // tile t, then V of tile t - lag.
-          const int lag = it.both ? 1 : 2;
+          constexpr int lag = 2;
           int kt = 0, vt = 0;  // the next K and V tile
           auto next_is_k = [&]() { return kt < n_tiles && kt < vt + lag; };
           auto key_tile = [&](int key_half, int& y, int& z) {  // TMA row and plane of the item's 64-key tile
@@ -884,11 +897,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             }
             ++chunk_ctr;
           };
-          auto q_box = [&](int u, int& yh, int& zt) {  // heads and positions of unit u
-            const int rr = it.mg * R + u * RU;
-            zt = it.b * (K + 1) + rr / g;
-            yh = it.kvh * g + rr % g;
-          };
+          const int q_head = it.kvh * g, q_pos = it.b * (K + 1) + it.mg * (R / g);
           // Chunks are filled as they free, before the item's Q slot is free
           // (an earlier item's last S), so the ring does not drain between
           // items; before the layer barrier only tiles that lie wholly in
@@ -896,36 +905,23 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           // output).
           if (!ready) {
             // Q is read once the layer barrier passes; bring it into L2 now
-            for (int u = 0; u <= it.both; ++u) {
-              int yh, zt;
-              q_box(u, yh, zt);
-              for (int hb = 0; hb < SM::kBoxes; ++hb) tma_prefetch_3d(&set.Q[layer], hb * 64, yh, zt);
-            }
+            for (int hb = 0; hb < SM::kBoxes; ++hb) tma_prefetch_3d(&set.Q[layer], hb * 64, q_head, q_pos);
           }
           bool ok = true, q_done = false;
           // a layer's first item: its prefix tiles go out once the previous
           // layer's last S has read its Q slot (earlier copies only slow the
           // previous layer, whose barrier this layer waits for)
-          if (!ready && q_last >= 0) ok = mbar_wait(bQEmpty + 8 * q_last, q_parity(q_last));
+          const uint32_t q_par = (item_ctr & 1) ^ 1;  // of the previous item's last S
+          if (!ready) ok = mbar_wait(bQEmpty, q_par);
           for (int spin = 0; ok && !q_done; ++spin) {
             if (ready && mbar_test_wait(bIEmpty + 8 * (item_ctr & 1), ((item_ctr >> 1) & 1) ^ 1) &&
-                mbar_test_wait(bQEmpty + 8 * it.qslot, q_parity(it.qslot)) &&
-                (!it.both || mbar_test_wait(bQEmpty + 8, q_parity(1)))) {
+                mbar_test_wait(bQEmpty, q_par)) {
+              // Q: R/g positions x g heads of kv head kvh, one box per 64-column half
               info[item_ctr & 1] = it;
               mbar_arrive(bIFull + 8 * (item_ctr & 1));
-              for (int u = 0; u <= it.both; ++u) {
-                // Q: RU/g positions x g heads of kv head kvh, one box per 64-column half
-                const int qs = it.both ? u : it.qslot;
-                int yh, zt;
-                q_box(u, yh, zt);
-                mbar_expect_tx(bQFull + 8 * qs, (uint32_t)RU * D * 2);
-                for (int hb = 0; hb < SM::kBoxes; ++hb)
-                  tma_load_3d(sQ + qs * SM::kQSlot + hb * 16384, &set.Q[layer], bQFull + 8 * qs, hb * 64, yh, zt);
-                q_loads ^= 1u << qs;
-                q_any |= 1u << qs;
-                q_last = qs;
-              }
-              q_next = QS == 1 ? 0 : q_last ^ 1;
+              mbar_expect_tx(bQFull, (uint32_t)R * D * 2);
+              for (int hb = 0; hb < SM::kBoxes; ++hb)
+                tma_load_3d(sQ + hb * 16384, &set.Q[layer], bQFull, hb * 64, q_head, q_pos);
               q_done = true;
               break;
             }
@@ -958,7 +954,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         }
         ready = true;
         ++item_ctr;
-        q_next = __shfl_sync(0xffffffffu, q_next, 0);
+        __syncwarp();
       }
     }
     // before leaving, wait (bounded) for this CTA's copies still in flight
@@ -967,15 +963,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         const uint32_t i = chunk_ctr - 1 - k;
         mbar_wait(bFull + 8 * (i % SM::kChunks), (i / SM::kChunks) & 1);
       }
-      for (int q = 0; q < 2; ++q)
-        if ((q_any >> q) & 1u) mbar_wait(bQFull + 8 * q, q_parity(q));
+      if (item_ctr > 0) mbar_wait(bQFull, (item_ctr - 1) & 1);
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ======================= MMA issue =======================
     if (lane == 0) {
       uint32_t item_ctr = 0, chunk_ctr = 0;
-      uint32_t q_uses = 0, p_par = 0;  // bit q: parity of the units read from Q slot q; bit s: of P steps of stream s
+      uint32_t p_par = 0;  // bit s: parity of P steps of stream s
       bool ok = true;
       auto take = [&]() {  // the next chunk, once it is filled
         const uint32_t ch = chunk_ctr % SM::kChunks;
@@ -991,48 +986,39 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           mbar_arrive(bIEmpty + 8 * (item_ctr & 1));
           const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
           const uint32_t ob = item_ctr & 1;
-          // Step j: one unit: tile j of stream j & 1; two units: tile j >> 1
-          // of unit (and stream) j & 1. S of a step goes where P of the
+          // Step j: tile j, stream j & 1. S of a step goes where P of the
           // stream's last step lies, so its PV is issued first.
-          const int n_steps = it.both ? 2 * n_tiles : n_tiles;
-          uint32_t kch = 0, vch = 0;
-          for (int j = 0; j < n_steps + 2 && ok; ++j) {
+          for (int j = 0; j < n_tiles + 2 && ok; ++j) {
             const int st = j & 1;
             const uint32_t ts = tmem + SM::kColS + st * 128;
             if (j >= 2) {  // O += P V of step j - 2
-              const int i = it.both ? (j - 2) >> 1 : j - 2, nh = min(2, n_half - 2 * i);
-              if (!it.both || st == 0) vch = take();
+              const uint32_t ch = take();
               ok = ok && mbar_spin(bPFull + 8 * st, (p_par >> st) & 1u);
               p_par ^= 1u << st;
               if (j == 2) ok = ok && mbar_spin(bOFree, (item_ctr & 1) ^ 1);
               if (!ok) break;
               tc_fence_after();
               constexpr uint32_t idesc = mma_idesc(128, D, 1);
-              const uint32_t va = desc_lo(sRing + vch * SM::kChunkBytes, 8192);
+              const uint32_t va = desc_lo(sRing + ch * SM::kChunkBytes, 8192);
               const uint32_t d = tmem + SM::kColO + st * 128;
               mma_ts4<2048>(d, ts, va, idesc, j < 4 ? 0u : 1u);
-              if (nh == 2) mma_ts4<2048>(d, ts + 32, va + SM::kBoxes * 512, idesc, 1u);
+              if (n_half - 2 * (j - 2) >= 2) mma_ts4<2048>(d, ts + 32, va + SM::kBoxes * 512, idesc, 1u);
               mma_commit(bPVDone + 8 * st);
-              if (!it.both || st == 1) mma_commit(bEmpty + 8 * vch);
+              mma_commit(bEmpty + 8 * ch);
             }
-            if (j < n_steps) {  // S = Q K^T of step j: the unit's rows x up to 128 keys
-              const int i = it.both ? j >> 1 : j, nh = min(2, n_half - 2 * i);
-              const int qs = it.both ? st : it.qslot;
-              if (!it.both || st == 0) kch = take();
-              if (j <= it.both) {
-                ok = ok && mbar_spin(bQFull + 8 * qs, (q_uses >> qs) & 1u);
-                q_uses ^= 1u << qs;
-              }
+            if (j < n_tiles) {  // S = Q K^T of step j: the group's rows x up to 128 keys
+              const uint32_t ch = take();
+              if (j == 0) ok = ok && mbar_spin(bQFull, item_ctr & 1);
               if (!ok) break;
               tc_fence_after();
-              const uint32_t idesc = mma_idesc(128, 64 * nh, 0);
-              const uint32_t qa = desc_lo(sQ + qs * SM::kQSlot, 16), ka = desc_lo(sRing + kch * SM::kChunkBytes, 16);
+              const uint32_t idesc = mma_idesc(128, n_half - 2 * j >= 2 ? 128 : 64, 0);
+              const uint32_t qa = desc_lo(sQ, 16), ka = desc_lo(sRing + ch * SM::kChunkBytes, 16);
 #pragma unroll
               for (int hb = 0; hb < SM::kBoxes; ++hb)
                 mma_ss4<32, 32>(ts, qa + hb * 1024, ka + hb * 1024, idesc, hb != 0 ? 1u : 0u);
               mma_commit(bSFull + 8 * st);
-              if (!it.both || st == 1) mma_commit(bEmpty + 8 * kch);
-              if (j >= n_steps - 1 - it.both) mma_commit(bQEmpty + 8 * qs);
+              mma_commit(bEmpty + 8 * ch);
+              if (j == n_tiles - 1) mma_commit(bQEmpty);
             }
           }
         }
@@ -1058,12 +1044,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     // A wait that fails leaves `ok` false; the item is then finished without
     // further waits, so that every thread still reaches every named barrier.
     auto wait = [&](uint32_t bar, uint32_t parity) { ok = ok && warp_wait(bar, parity); };
-    // layer n_layers has no items: it only helps with the last layer's merge
-    for (int layer = 0; layer <= n_layers; ++layer) {
-      const bool has_items = layer < n_layers;
+    for (int layer = 0; layer < n_layers; ++layer) {
       float* part_o = part_buf_o + (layer % kAttnPartBufs) * part_o_stride;
       float* part_ml = part_buf_ml + (layer % kAttnPartBufs) * part_ml_stride;
-      if (layer > 0 && has_items) {
+      if (layer > 0) {
         // layer's inputs are ready once every CTA is done with the previous layer
         if (tid == 0 && !wait_counter(bar_cnt + (layer - 1), n_ctas)) ok = false;
         if (softmax_any(!ok)) {
@@ -1071,10 +1055,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           break;
         }
       }
-      __nv_bfloat16* O = has_items ? set.p[layer].O : nullptr;
-      float* lse = has_items ? set.p[layer].lse : nullptr;
+      __nv_bfloat16* O = set.p[layer].O;
+      float* lse = set.p[layer].lse;
       bool failed = false;
-      for (int item = 0; item < n_items && has_items; ++item) {
+      for (int item = 0; item < n_items; ++item) {
         wait(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
         if (softmax_any(!ok)) {
           failed = true;
@@ -1082,13 +1066,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         }
         const ItemInfo& it = info[item_ctr & 1];
         const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
-        const int steps0 = it.both ? n_tiles : (n_tiles + 1) >> 1, steps1 = it.both ? n_tiles : n_tiles >> 1;
+        const int steps0 = (n_tiles + 1) >> 1, steps1 = n_tiles >> 1;
         const int my_steps = st ? steps1 : steps0;
-        const int rows = it.both && st ? it.rows1 : it.rows0;
+        const int rows = it.rows;
         const bool valid = row < rows;
         // a warp without valid rows only keeps the barrier counts in step
         const bool warp_live = wq * 32 < rows;
-        const int rr = it.mg * R + (it.both ? st * RU : 0) + row;  // row of the (sequence, kv head)
+        const int rr = it.mg * R + row;  // row of the (sequence, kv head)
         const int t_row = rr / g;
         float m_run = -INFINITY, l_run = 0.f;
         {
@@ -1102,9 +1086,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           // tiles past this key need the mask; rows past the group compute on whatever their lanes hold, seen by no
           // other row and never stored
           const int mask_from = valid ? min(tree_vis ? kv : kv + t_row, key1 - 1) : 0x7fffffff;
-          const int kt_step = it.both ? 128 : 256;
-          int kt0 = it.key0 + (it.both ? 0 : st * 128);
-          for (int i = 0; i < my_steps; ++i, kt0 += kt_step) {
+          int kt0 = it.key0 + st * 128;
+          for (int i = 0; i < my_steps; ++i, kt0 += 256) {
             const uint32_t n = (st ? done1 : done0) + i;
             wait(bSFull + 8 * st, n & 1);
             if (!warp_live) {
@@ -1116,11 +1099,51 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             const bool two = key1 - kt0 > 64;  // the tile's second 64 keys exist
             // (the whole warp masks or none of it: the loops below hold warp-wide tensor-memory instructions)
             const bool need_mask = __any_sync(0xffffffffu, kt0 + 127 > mask_from);
-            // raw scores of keys c0 .. c0 + 31; keys this row does not see count as -inf
-            auto load_scores = [&](int c0, uint32_t (&x)[32]) {
-              tmem_ld32(ts + c0, x);
-              tmem_wait_ld();
-              if (need_mask) {
+            float la[2] = {0.f, 0.f}, lb[2] = {0.f, 0.f};
+            // The reference max of a row is the max of its first 32 keys; it
+            // is raised, by a power of two, when a later key exceeds it by
+            // more than 2^8 (rare): what was computed against the old one (l,
+            // O, the tile's P so far) is scaled, P exactly.
+            auto raise_to = [&](float cmax, int c0) {
+              const bool raise = cmax > m_run + kRescaleLog2;
+              const bool unset = m_run == -INFINITY;
+              const float up = unset ? cmax : m_run + ceilf(cmax - m_run);
+              const float f = !raise ? 1.f : unset ? 0.f : ex2_approx(m_run - up);
+              m_run = raise ? up : m_run;
+              l_run *= f;
+              la[0] *= f;
+              la[1] *= f;
+              lb[0] *= f;
+              lb[1] *= f;
+#pragma unroll 1
+              for (int c = 0; c < c0 / 2; c += 16) {
+                uint32_t q[16];
+                tmem_ld16(ts + c, q);
+                tmem_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 16; ++k) q[k] = pack_bf16(bf16_lo(q[k]) * f, bf16_hi(q[k]) * f);
+                tmem_st16(ts + c, q);
+              }
+              if (i > 0) {
+                // O holds the stream's earlier tiles of this item: its last PV has landed
+                wait(bPVDone + 8 * st, (n - 1) & 1);
+                tc_fence_after();
+#pragma unroll 1
+                for (int d0 = 0; d0 < D; d0 += 32) {
+                  uint32_t o[32];
+                  const uint32_t oa = tmem + lane_off + SM::kColO + st * 128 + d0;
+                  tmem_ld32(oa, o);
+                  tmem_wait_ld();
+#pragma unroll
+                  for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * f);
+                  tmem_st32(oa, o);
+                }
+              }
+              tmem_wait_st();
+            };
+            // keys c0 .. c0 + 31 of the tile, their scores in x: P of them in place of scores already read
+            auto softmax_32 = [&](int c0, uint32_t (&x)[32]) {
+              if (need_mask) {  // keys this row does not see count as -inf
                 const int k0 = kt0 + c0;
                 uint32_t bits = (uint32_t)(!vrow ? low_bits(kv + t_row + 1 - k0)
                                                  : low_bits(kv + 1 - k0) | bit_window(vrow, tree_words, k0 - kv - 1));
@@ -1130,57 +1153,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
                 for (int c = 0; c < 32; ++c)
                   if (!((bits >> c) & 1u)) x[c] = __float_as_uint(-INFINITY);
               }
-            };
-            // (Loops of 32 keys, loaded again for the second: short code. A
-            // tile's arithmetic unrolled over its 128 keys ran no faster warm,
-            // and at B = 1, where each layer runs it once or twice, twice as
-            // long, on instruction fetches.)
-            const int n_cols = two ? 128 : 64;
-            float tmax = -INFINITY;
-#pragma unroll 1
-            for (int c0 = 0; c0 < n_cols; c0 += 32) {
-              uint32_t x[32];
-              load_scores(c0, x);
-              float a = tmax, b = -INFINITY;
+              float a = -INFINITY, b = -INFINITY;
 #pragma unroll
               for (int c = 0; c < 32; c += 4) {
                 a = fmaxf(fmaxf(a, __uint_as_float(x[c])), __uint_as_float(x[c + 1]));
                 b = fmaxf(fmaxf(b, __uint_as_float(x[c + 2])), __uint_as_float(x[c + 3]));
               }
-              tmax = fmaxf(a, b);
-            }
-            tmax *= scale_log2;
-            // raise the reference max only when it grows by more than 2^8
-            const bool raise = tmax > m_run + kRescaleLog2;
-            if (__any_sync(0xffffffffu, raise)) {
-              float f = 1.f;
-              f = !raise ? 1.f : (m_run == -INFINITY) ? 0.f : ex2_approx(m_run - tmax);
-              m_run = raise ? tmax : m_run;
-              l_run *= f;
-              if (i > 0) {
-                // O holds the stream's earlier tiles of this item: rescale its
-                // rows once the last PV has landed
-                wait(bPVDone + 8 * st, (n - 1) & 1);
-                tc_fence_after();
-#pragma unroll 1
-                for (int c0 = 0; c0 < D; c0 += 32) {
-                  uint32_t o[32];
-                  const uint32_t oa = tmem + lane_off + SM::kColO + st * 128 + c0;
-                  tmem_ld32(oa, o);
-                  tmem_wait_ld();
-#pragma unroll
-                  for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * f);
-                  tmem_st32(oa, o);
-                }
-                tmem_wait_st();
-              }
-            }
-            const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
-            float la[2] = {0.f, 0.f}, lb[2] = {0.f, 0.f};
-#pragma unroll 1
-            for (int c0 = 0; c0 < n_cols; c0 += 32) {
-              uint32_t x[32], pk[16];
-              load_scores(c0, x);
+              const float cmax = fmaxf(a, b) * scale_log2;
+              if (__any_sync(0xffffffffu, cmax > m_run + kRescaleLog2)) raise_to(cmax, c0);
+              const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
+              uint32_t pk[16];
 #pragma unroll
               for (int c = 0; c < 32; c += 4) {
                 float y0, y1, y2, y3;
@@ -1195,7 +1177,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
                 pk[c >> 1] = pack_bf16(y0, y1);
                 pk[(c >> 1) + 1] = pack_bf16(y2, y3);
               }
-              tmem_st16(ts + c0 / 2, pk);  // over scores already read
+              tmem_st16(ts + c0 / 2, pk);
+            };
+            // 64 keys a trip, the next 32 loaded while these are worked on
+            const int n_cols = two ? 128 : 64;
+#pragma unroll 1
+            for (int c0 = 0; c0 < n_cols; c0 += 32) {
+              uint32_t x[32];
+              tmem_ld32(ts + c0, x);
+              tmem_wait_ld();
+              softmax_32(c0, x);
             }
             l_run += (la[0] + la[1]) + (lb[0] + lb[1]);
             tmem_wait_st();
@@ -1205,9 +1196,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           }
         }
         // ---- epilogue: O of this item is complete once the last PVs have landed ----
-        float f0 = 1.f, f1 = 0.f;  // factors of the streams' O (two units: f0 of this stream's own)
-        if (!it.both && steps1 > 0) {
-          // both streams hold keys of the same rows: exchange (m, l)
+        float f0 = 1.f, f1 = 0.f;  // factors of the streams' O
+        const bool second = steps1 > 0;
+        if (second) {  // the streams hold keys of the same rows: exchange (m, l)
           if (warp_live) stat[st * 128 + row] = make_float2(m_run, l_run);
           softmax_sync();
           if (warp_live) {
@@ -1219,14 +1210,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             l_run = f0 * a.y + f1 * b.y;
           }
         }
-        if (it.both ? st == 0 : true) wait(bPVDone, (done0 + steps0 - 1) & 1);
-        if (it.both ? st == 1 : steps1 > 0) wait(bPVDone + 8, (done1 + steps1 - 1) & 1);
+        wait(bPVDone, (done0 + steps0 - 1) & 1);
+        if (second) wait(bPVDone + 8, (done1 + steps1 - 1) & 1);
         tc_fence_after();
-        // the streams share out the columns of rows they both hold; a single step leaves all to stream 0
-        const bool second = !it.both && steps1 > 0;
-        if (warp_live && (it.both || second || st == 0)) {
+        // the warpgroups share out the columns; a single step leaves all to the first
+        if (warp_live && (second || st == 0)) {
           const int hq = it.kvh * g + rr % g;
-          const size_t prow = (size_t)it.slot * slot_rows + (it.both ? st * RU : 0) + row;
+          const size_t prow = (size_t)it.slot * kAttnRows + row;
           const bool partial = it.partial;
           if (!partial) {
             const float inv = 1.f / l_run;
@@ -1235,7 +1225,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           }
           const int cb = second ? st * (D / 2) : 0, ce = second ? cb + D / 2 : D;
           __nv_bfloat16* orow = O + (((size_t)it.b * (K + 1) + t_row) * Hq + hq) * D;
-          const uint32_t oa = tmem + lane_off + SM::kColO + (it.both ? st * 128 : 0);
+          const uint32_t oa = tmem + lane_off + SM::kColO;
 #pragma unroll 1
           for (int c0 = cb; c0 < ce; c0 += 32) {
             uint32_t o[32];
@@ -1268,7 +1258,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
               }
             }
           }
-          if (valid && (it.both || st == 0)) {
+          if (valid && st == 0) {
             if (partial) {
               *reinterpret_cast<float2*>(part_ml + prow * 2) = make_float2(m_run, l_run);
             } else if (lse) {
@@ -1299,15 +1289,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       }
       // This CTA is done with the layer's items. Once its grid barrier
       // passes, CTAs write layer + 1's partials into the buffer of layer - 2,
-      // whose merge must be done first. Help with the merge warp's backlog
-      // (layers up to layer - 1) if it is large; after the last layer, help
-      // with its merge (the tail of the launch) once its barrier has passed.
-      if (layer > 0 && merge_n > 0 &&
-          (has_items ? layer * merge_n - *reinterpret_cast<volatile int*>(merge_claimed) >= kMergeHelpChunks
-                     : last_groups_ready()))
-        merge_chunks<D>(layer - 1, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R, slot_rows, part_buf_o,
-                        part_buf_ml, part_o_stride, part_ml_stride);
-      if (!has_items) break;
+      // whose merge must be done first.
       if (layer >= kAttnPartBufs - 1 && merge_n > 0 && tid == 0 &&
           !merged_upto((layer - (kAttnPartBufs - 2)) * merge_n))
         ok = false;
@@ -1322,23 +1304,28 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       if (lane == 0) raise_status(status, LIBRASPEC_ST_TIMEOUT);
       misc[0] = 1;
     }
-  } else if (warp == kMergeWarp) {
-    // ======================= merge warp =======================
-    // Layer l's split groups, once every CTA has finished layer l (its grid
-    // barrier), while the softmax warps already run the next layers.
+  }
+  // ======================= merges =======================
+  // The two merge warps come here at once and merge layer l's split groups
+  // once every CTA has finished layer l (its grid barrier), beside the next
+  // layers' items; the other warps come when their roles are done and help
+  // with the last layer's. One copy of the code for all of them, outside the
+  // roles: a second one in the softmax warps' path cost fetches of cold
+  // instructions and their registers.
+  __syncwarp();
+  {
     bool ok = true;
-    for (int layer = 0; layer < n_layers && ok; ++layer) {
+    for (int layer = warp >= kMergeWarp ? 0 : n_layers - 1; layer < n_layers && ok && merge_n > 0; ++layer) {
       if (layer < n_layers - 1) {
         ok = layer_done(layer);
-      } else {
+      } else if (warp == kMergeWarp) {
         // the last layer: each split group once its np parts are counted in
         // (no grid barrier); the last CTA past a group's wait resets its
         // counters for the next launch
         if (lane == 0) {
-          for (int ti = 0; ti < n_tasks && ok; ++ti)
-            ok = wait_counter(grp_cnt + 2 * tasks[ti].grp, tasks[ti].np);
+          for (int ti = 0; ti < n_tasks && ok; ++ti) ok = wait_counter(grp_cnt + 2 * tasks[ti].grp, tasks[ti].np);
           if (ok) {
-            misc[6] = 1;  // the softmax warps may help now
+            misc[6] = 1;  // the other warps may start
             for (int ti = 0; ti < n_tasks; ++ti) {
               uint32_t* gc = grp_cnt + 2 * tasks[ti].grp;
               if (atomicAdd(gc + 1, 1u) == (uint32_t)tasks[ti].np - 1) {
@@ -1349,16 +1336,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
           }
         }
         ok = __shfl_sync(0xffffffffu, ok, 0) != 0 && !misc[0];
+      } else {
+        ok = last_groups_ready();
       }
-      if (!ok) break;
-      if (merge_n > 0)
-        merge_chunks<D>(layer, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R, slot_rows, part_buf_o,
-                        part_buf_ml, part_o_stride, part_ml_stride);
-    }
-    // every chunk of every layer is merged (by whichever warp) before the exit count
-    if (ok && merge_n > 0 && n_layers > 0) {
-      if (lane == 0) ok = merged_upto(n_layers * merge_n);
-      ok = __shfl_sync(0xffffffffu, ok, 0) != 0;
+      if (ok)
+        merge_chunks<D>(layer, set, tasks, n_tasks, merge_n, merge_claimed, merge_done, K, Hq, Hkv, R,
+                        part_buf_o, part_buf_ml, part_o_stride, part_ml_stride);
     }
     if (!ok && lane == 0 && !misc[0]) {
       raise_status(status, LIBRASPEC_ST_TIMEOUT);
@@ -1390,14 +1373,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
 // ---------------------------------------------------------------------------
 int num_sms_current();
 
-// Q [B*(K+1), Hq, D] as 3-D; box = 64 columns x g heads x RU/g positions (one
-// unit of rows of one kv head), 128-byte swizzle.
-static bool make_q_map(CUtensorMap* map, const void* base, int D, int Hq, int BT, int g, int RU) {
+// Q [B*(K+1), Hq, D] as 3-D; box = 64 columns x g heads x R/g positions (one
+// row group of one kv head), 128-byte swizzle.
+static bool make_q_map(CUtensorMap* map, const void* base, int D, int Hq, int BT, int g, int R) {
   auto enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)BT};
   cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)Hq * D * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)g, (cuuint32_t)(RU / g)};
+  cuuint32_t box[3] = {64, (cuuint32_t)g, (cuuint32_t)(R / g)};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -1559,28 +1542,28 @@ struct LayerSetCache {
 };
 constexpr int kCachedChunks = 4;
 
-template <int D, int QS, bool PAGED>
+template <int D, bool PAGED>
 static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* const* Kc, const uint16_t* const* Vc,
                                    int n_layers, const int32_t* kv_len, const int32_t* L, const uint64_t* tree_vis,
                                    const int32_t* block_table,
                                    int max_pages, int page_size, int n_pages, int B, int K, int Hq, int Hkv, int S_cap,
                                    float scale, uint16_t* const* O, float* const* lse, char* ws, const WsLayout& lay,
                                    cudaStream_t stream) {
-  using SM = AttnSmem<D, QS>;
+  using SM = AttnSmem<D>;
   constexpr int kSmem = PAGED ? SM::kAllocPaged : SM::kAlloc;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(verify_attn_kernel<D, QS, PAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(verify_attn_kernel<D, PAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kSmem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
   int grid = num_sms_current();  // one CTA per SM (it holds all 512 tensor-memory columns)
   if (grid > kAttnMaxCtas) grid = kAttnMaxCtas;
-  auto kern = verify_attn_kernel<D, QS, PAGED>;
+  auto kern = verify_attn_kernel<D, PAGED>;
   const int item_tiles = attn_item_tiles();
   const int g = Hq / Hkv;
-  const int R = attn_unit_rows(g);
+  const int R = g * (kAttnRows / g);
   // layers beyond kMaxLayers go in further launches of the same kernel
   for (int l0 = 0; l0 < n_layers; l0 += kMaxLayers) {
     const int n = n_layers - l0 < kMaxLayers ? n_layers - l0 : kMaxLayers;
@@ -1646,7 +1629,7 @@ static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* con
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(
         &cfg, kern, set, kv_len, L, tree_vis, tree_words(K), block_table, max_pages, page_size, n_pages, attn_page_cache(SM::kPageCap), B, K,
-        Hq, Hkv, S_cap, scale * kLog2e, attn_min_tiles(), item_tiles, attn_slot_rows(g, K),
+        Hq, Hkv, S_cap, scale * kLog2e, attn_min_tiles(), item_tiles,
         reinterpret_cast<float*>(ws + lay.attn_o), reinterpret_cast<float*>(ws + lay.attn_ml), o_part / sizeof(float),
         ml_part / sizeof(float), reinterpret_cast<uint32_t*>(ws + lay.attn_cnt),
         reinterpret_cast<uint32_t*>(ws + lay.attn_grp), reinterpret_cast<int*>(ws + lay.status));
@@ -1665,9 +1648,7 @@ cudaError_t launch_verify_attn_layers(const uint16_t* const* Q, const uint16_t* 
   const uint64_t* vis = nullptr;
   cudaError_t e = tree_vis(parent, L, B, K, ws, lay, stream, &vis);
   if (e != cudaSuccess) return e;
-  const bool two = attn_slot_rows(Hq / Hkv, K) > kAttnRows;  // row groups of up to two units
-  auto* launch = D == 128 ? (two ? launch_layers_t<128, 2, false> : launch_layers_t<128, 1, false>)
-                          : (two ? launch_layers_t<64, 2, false> : launch_layers_t<64, 1, false>);
+  auto* launch = D == 128 ? launch_layers_t<128, false> : launch_layers_t<64, false>;
   return launch(Q, Kc, Vc, n_layers, kv_len, L, vis, nullptr, 0, 0, 0, B, K, Hq, Hkv, S_cap,
                                           scale, O, lse, ws, lay, stream);
 }
@@ -1683,9 +1664,7 @@ cudaError_t launch_verify_attn_paged_layers(const uint16_t* const* Q, const uint
   const uint64_t* vis = nullptr;
   cudaError_t e = tree_vis(parent, L, B, K, ws, lay, stream, &vis);
   if (e != cudaSuccess) return e;
-  const bool two = attn_slot_rows(Hq / Hkv, K) > kAttnRows;
-  auto* launch = D == 128 ? (two ? launch_layers_t<128, 2, true> : launch_layers_t<128, 1, true>)
-                          : (two ? launch_layers_t<64, 2, true> : launch_layers_t<64, 1, true>);
+  auto* launch = D == 128 ? launch_layers_t<128, true> : launch_layers_t<64, true>;
   return launch(Q, Kp, Vp, n_layers, kv_len, L, vis, block_table, max_pages, page_size,
                                          n_pages, B, K, Hq, Hkv, S_cap, scale, O, lse, ws, lay, stream);
 }

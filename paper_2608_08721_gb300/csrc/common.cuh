@@ -77,14 +77,6 @@ struct WsLayout {
   int max_items, max_groups;
 };
 
-// Attention rows: units of whole block positions, at most 128 rows. Where a
-// (sequence, kv head) may have more rows than a unit, a row group is two
-// units, and a partial's slot has room for both.
-__host__ __device__ constexpr int attn_unit_rows(int g) { return g * (kAttnRows / g); }
-__host__ __device__ constexpr int attn_slot_rows(int g, int K) {
-  return (K + 1) * g > attn_unit_rows(g) ? 2 * kAttnRows : kAttnRows;
-}
-
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 inline WsLayout ws_layout(int B, int K, int V, int Hq, int Hkv, int d, int S_cap) {
@@ -95,7 +87,7 @@ inline WsLayout ws_layout(int B, int K, int V, int Hq, int Hkv, int d, int S_cap
   const size_t rows_d = size_t(B) * K, rows_t = size_t(B) * (K + 1);
   const int g = Hkv > 0 ? Hq / Hkv : 1;
   const int m_max = (K + 1) * g;
-  const int rows = g >= 1 && g <= kAttnRows ? attn_unit_rows(g) : 1;
+  const int rows = g >= 1 && g <= kAttnRows ? g * (kAttnRows / g) : 1;
   const int n_mg = (m_max + rows - 1) / rows;
   w.max_groups = B * Hkv * n_mg;
   w.max_items = kAttnMaxCtas + w.max_groups;
@@ -118,9 +110,8 @@ inline WsLayout ws_layout(int B, int K, int V, int Hq, int Hkv, int d, int S_cap
   w.acc_plan = take(16 + 8 * std::max(size_t(kAccMaxGrid), rows_t));
   // two partial slots per attention CTA (its first and its last item), in
   // kAttnPartBufs buffers that rotate with the layer (layer % kAttnPartBufs)
-  const int slot_rows = g >= 1 && g <= kAttnRows ? attn_slot_rows(g, K) : kAttnRows;
-  w.attn_o = take(kAttnPartBufs * size_t(2 * kAttnMaxCtas) * slot_rows * d * sizeof(float));
-  w.attn_ml = take(kAttnPartBufs * size_t(2 * kAttnMaxCtas) * slot_rows * 2 * sizeof(float));
+  w.attn_o = take(kAttnPartBufs * size_t(2 * kAttnMaxCtas) * kAttnRows * d * sizeof(float));
+  w.attn_ml = take(kAttnPartBufs * size_t(2 * kAttnMaxCtas) * kAttnRows * 2 * sizeof(float));
   // grid-barrier counters, one per layer of a launch, then the exit counter
   w.attn_cnt = take((kAttnMaxLayers + 1) * sizeof(uint32_t));
   // per row group: parts of the last layer counted in, CTAs past its wait

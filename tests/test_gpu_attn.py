@@ -237,3 +237,18 @@ def test_attn_step_and_unit_edges(orc, d, Hq, Hkv, K):
     for _ in range(3):
         O, lse = _run(Q, Kc, Vc, kv, L, K)
         check_attn(O, lse, O_ref, lse_ref, L)
+
+
+@pytest.mark.parametrize("B,kv,L,Hq,Hkv,d", [(1, 4096, 5, 8, 8, 128), (1, 100, 0, 32, 8, 128), (3, 640, 9, 16, 4, 64),
+                                             (5, 63, 3, 8, 2, 128), (40, 200, 12, 16, 4, 64), (2, 9000, 12, 64, 64, 128)])
+def test_attn_equal_groups_get_whole_ctas(orc, B, kv, L, Hq, Hkv, d):
+    """Equal caches and lengths: each row group has its own CTAs (one that covers it, or several whose parts are
+    merged), or, with groups a few too many for that, the batch is cut by cost. Tolerances as in check_attn."""
+    K = 16
+    Q, Kc, Vc = _inputs(B, K, Hq, Hkv, d, None, kv + K + 1, seed=B * 100 + kv, scale_k=2.0)
+    kvs, Ls = [kv] * B, [L] * B
+    rows = np.array([(b, h, t) for b in range(B) for h in (0, Hq // 2, Hq - 1) for t in {0, L}], np.int32)
+    O_ref, lse_ref = orc.verify_attn(Q, Kc, Vc, np.array(kvs), np.array(Ls), rows=rows)
+    for _ in range(2):
+        O, lse = _run(Q, Kc, Vc, kvs, Ls, K)
+        check_attn(O, lse, O_ref, lse_ref, Ls, rows=[tuple(r) for r in rows])
