@@ -1160,7 +1160,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
                 b = fmaxf(fmaxf(b, __uint_as_float(x[c + 2])), __uint_as_float(x[c + 3]));
               }
               const float cmax = fmaxf(a, b) * scale_log2;
-              if (__any_sync(0xffffffffu, cmax > m_run + kRescaleLog2)) raise_to(cmax, c0);
+              if (i == 0 && c0 == 0) m_run = cmax;
+              else if (__any_sync(0xffffffffu, cmax > m_run + kRescaleLog2)) raise_to(cmax, c0);
               const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
               uint32_t pk[16];
 #pragma unroll
