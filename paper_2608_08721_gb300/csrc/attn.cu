@@ -11,7 +11,7 @@
 // head, row group, key tile); CTA c of the persistent grid (one CTA per SM)
 // takes a contiguous range of it: with equal groups its part of one group
 // (aligned_ctas), else a range cut by cost (each row group weighs its tiles
-// plus an item's fixed cost; tile_of_weighted), so that CTAs finish together
+// plus an item's fixed cost; find_tile), so that CTAs finish together
 // whatever the ragged lengths. The plan is derived on the device from L[] and
 // kv_len[] by every CTA, and it is the same for every layer (all layers share
 // L and kv_len).
@@ -205,50 +205,6 @@ __device__ long long total_tiles(int B, const int32_t* kv_len, const int32_t* Ls
   return tot;
 }
 
-// Where tile position `pos` of the batch's tile sequence lies (warp-wide).
-struct TileLoc {
-  int b;                  // sequence (-1: past the end)
-  long long seq_start;    // first tile of sequence b
-  int group0;             // global index of b's first row group
-  SeqPlan p;
-};
-
-__device__ TileLoc locate_tile(long long pos, int B, const int32_t* kv_len, const int32_t* Ls, int K, int g, int R,
-                               int Hkv, int S_cap) {
-  const int lane = threadIdx.x & 31;
-  TileLoc loc{-1, 0, 0, {}};
-  long long carry_t = 0;
-  int carry_g = 0;
-  for (int base = 0; base < B; base += 32) {
-    const int b = base + lane;
-    const SeqPlan p = seq_plan(b, B, kv_len, Ls, K, g, R, S_cap);
-    const long long nt = p.ok ? (long long)Hkv * p.n_mg * p.n_tiles : 0;
-    const int ng = p.ok ? Hkv * p.n_mg : 0;
-    long long inc_t = nt;
-    int inc_g = ng;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const long long a = __shfl_up_sync(0xffffffffu, inc_t, off);
-      const int c = __shfl_up_sync(0xffffffffu, inc_g, off);
-      if (lane >= off) { inc_t += a; inc_g += c; }
-    }
-    const long long st = carry_t + inc_t - nt;
-    const bool mine = nt > 0 && pos >= st && pos < st + nt;
-    const unsigned ball = __ballot_sync(0xffffffffu, mine);
-    if (ball) {
-      const int src = __ffs(ball) - 1;
-      loc.b = base + src;
-      loc.seq_start = __shfl_sync(0xffffffffu, st, src);
-      loc.group0 = __shfl_sync(0xffffffffu, carry_g + inc_g - ng, src);
-      loc.p = seq_plan(loc.b, B, kv_len, Ls, K, g, R, S_cap);
-      return loc;
-    }
-    carry_t += __shfl_sync(0xffffffffu, inc_t, 31);
-    carry_g += __shfl_sync(0xffffffffu, inc_g, 31);
-  }
-  return loc;
-}
-
 // a / b for a >= 0, b > 0: 32-bit when both fit (a 64-bit division is a
 // long software sequence, and the plan runs on one warp before any copy)
 __device__ __forceinline__ long long div_nn(long long a, long long b) {
@@ -273,41 +229,52 @@ __device__ __forceinline__ int cta_of(long long t, long long T, int G) {
 // with few tiles without any): 16 paged sequences 110 -> 102 us (2 layers), a
 // tree of 512 nodes 352 -> 339 (4 layers), ragged B = 64 312 -> 296; C = 8 and
 // 12 gave ragged 298 and 301, the tree 332.
-__device__ long long tile_of_weighted(long long x, long long W, long long T, int C, int B, const int32_t* kv_len,
-                                      const int32_t* Ls, int K, int g, int R, int Hkv, int S_cap) {
-  if (x >= W) return T;
+struct TileLoc {
+  long long tile;       // the tile (T: past the end)
+  int b;                // its sequence
+  long long seq_start;  // first tile of sequence b
+  int group0;           // global index of b's first row group
+  SeqPlan p;
+};
+
+// The tile at weighted position x (at C = 0: tile x), and where it lies (warp-wide).
+__device__ TileLoc find_tile(long long x, int C, long long T, int B, const int32_t* kv_len, const int32_t* Ls, int K,
+                             int g, int R, int Hkv, int S_cap) {
   const int lane = threadIdx.x & 31;
-  long long carry_w = 0, carry_t = 0;
+  TileLoc loc{T, 0, 0, 0, {}};
+  long long carry_t = 0;
+  int carry_g = 0;
   for (int base = 0; base < B; base += 32) {
-    const int b = base + lane;
-    const SeqPlan p = seq_plan(b, B, kv_len, Ls, K, g, R, S_cap);
-    const long long nt = p.ok ? (long long)Hkv * p.n_mg * p.n_tiles : 0;
-    const long long nw = p.ok ? nt + (long long)C * Hkv * p.n_mg : 0;
-    long long inc_w = nw, inc_t = nt;
+    const SeqPlan p = seq_plan(base + lane, B, kv_len, Ls, K, g, R, S_cap);
+    const int ng = p.ok ? Hkv * p.n_mg : 0;
+    const long long nt = (long long)ng * p.n_tiles;
+    long long inc_t = nt;
+    int inc_g = ng;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const long long a = __shfl_up_sync(0xffffffffu, inc_w, off);
-      const long long t = __shfl_up_sync(0xffffffffu, inc_t, off);
-      if (lane >= off) { inc_w += a; inc_t += t; }
+      const long long a = __shfl_up_sync(0xffffffffu, inc_t, off);
+      const int c = __shfl_up_sync(0xffffffffu, inc_g, off);
+      if (lane >= off) { inc_t += a; inc_g += c; }
     }
-    const long long sw = carry_w + inc_w - nw;
-    const bool mine = nw > 0 && x >= sw && x < sw + nw;
-    const unsigned ball = __ballot_sync(0xffffffffu, mine);
+    const long long st = carry_t + inc_t - nt;  // the sequence's first tile and row group
+    const int sg = carry_g + inc_g - ng;
+    const long long sw = st + (long long)C * sg;
+    const unsigned ball = __ballot_sync(0xffffffffu, nt > 0 && x >= sw && x < sw + nt + (long long)C * ng);
     if (ball) {
       const int src = __ffs(ball) - 1;
-      const long long wstart = __shfl_sync(0xffffffffu, sw, src);
-      const long long tstart = __shfl_sync(0xffffffffu, carry_t + inc_t - nt, src);
-      const SeqPlan q = seq_plan(base + src, B, kv_len, Ls, K, g, R, S_cap);
-      const long long per = q.n_tiles + C;
-      const long long o = x - wstart;
-      const long long gib = div_nn(o, per);
-      const long long r = o - gib * per;
-      return tstart + gib * q.n_tiles + (r > C ? r - C : 0);
+      loc.b = base + src;
+      loc.seq_start = __shfl_sync(0xffffffffu, st, src);
+      loc.group0 = __shfl_sync(0xffffffffu, sg, src);
+      loc.p = seq_plan(loc.b, B, kv_len, Ls, K, g, R, S_cap);
+      const long long o = x - (loc.seq_start + (long long)C * loc.group0);
+      const long long gib = div_nn(o, loc.p.n_tiles + C), r = o - gib * (loc.p.n_tiles + C);
+      loc.tile = loc.seq_start + gib * loc.p.n_tiles + (r > C ? r - C : 0);
+      return loc;
     }
-    carry_w += __shfl_sync(0xffffffffu, inc_w, 31);
     carry_t += __shfl_sync(0xffffffffu, inc_t, 31);
+    carry_g += __shfl_sync(0xffffffffu, inc_g, 31);
   }
-  return T;
+  return loc;
 }
 
 // Equal groups. Where every row group has the same number nt of tiles (one
@@ -350,7 +317,8 @@ struct ItemInfo {
   int partial;     // 1: write a partial, else write O
   int slot;        // partial slot
   int grp;         // global row group index
-  int pad[6];
+  int last;        // 1: the CTA's last item of the layer; 2: no item, in any layer
+  int pad[5];
 };
 static_assert(sizeof(ItemInfo) == 64, "items lie in 64-byte slots");
 
@@ -395,7 +363,7 @@ struct AttnSmem {
   static constexpr int kInfo = kBar + ((8 * kNumBars + 63) / 64) * 64;
   static constexpr int kTasks = kInfo + 2 * 64;
   static constexpr int kTmem = kTasks + 64;
-  // [0] abort, [1] merge tasks, [2] items per layer, [3] merge chunks per
+  // [0] abort, [1] merge tasks, [2] the tasks are set, [3] merge chunks per
   // layer, [4] chunks claimed, [5] chunks done, [6] the last layer's merges
   // may start
   static constexpr int kMisc = kTmem + 16;
@@ -404,14 +372,13 @@ struct AttnSmem {
   // kv_len and L of up to kPlanCap sequences, read once from global memory
   // for the CTA's tile plan (a larger batch plans from global memory)
   static constexpr int kPlanCap = 1024;
-  static constexpr int kRange = kStat + kStreams * 128 * 8;  // the CTA's tile range [lo, hi)
-  static constexpr int kPlan = kRange + 16;
+  static constexpr int kPlan = kStat + kStreams * 128 * 8;
   static constexpr int kBytes = kPlan + 2 * 4 * kPlanCap;
   static constexpr int kAlloc = kBytes + 1024;           // room to align the base to 1024
   // tensor-memory columns: per stream S of a tile (128 fp32, its P as 64
   // columns of bf16 pairs in the same place) and O (D fp32); lane = row
   static constexpr int kColS = 0, kColO = 256;
-  static_assert(kStat % 16 == 0 && kRange % 8 == 0 && kInfo % 16 == 0, "alignment");
+  static_assert(kStat % 16 == 0 && kInfo % 16 == 0, "alignment");
   static_assert(kAlloc <= 227 * 1024, "shared memory per CTA");
   // paged caches: the page of each of the CTA's tiles, after everything else
   static constexpr int kPageCap = 4096;
@@ -644,6 +611,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
   const int32_t* kvs = plan_cached ? plan_kv : kv_len;
   const int32_t* Lss = plan_cached ? plan_L : Ls;
 
+  if (plan_cached)
+    for (int b = tid; b < B; b += kAttnThreads) {
+      plan_kv[b] = kv_len[b];
+      plan_L[b] = Ls[b];
+    }
   if (tid == 0) {
     for (int s = 0; s < SM::kChunks; ++s) {
       mbar_init(bFull + 8 * s, 1);
@@ -661,6 +633,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     mbar_init(bOFree, kSoftmaxWarps);
     mbar_init(bDrain, 1);
     misc[0] = 0;
+    misc[2] = 0;
     misc[4] = 0;
     misc[5] = 0;
     misc[6] = 0;
@@ -674,103 +647,106 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // The plan (identical for every layer): this CTA's tile range, its item
-  // count and the split groups it helps merge.
-  if (warp == 0) {
-    if (plan_cached) {
-      // one round trip: four sequences per lane in flight
-      for (int b0 = 0; b0 < B; b0 += 128) {
-        int kv4[4], L4[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int b = b0 + u * 32 + lane;
-          kv4[u] = b < B ? kv_len[b] : 0;
-          L4[u] = b < B ? Ls[b] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int b = b0 + u * 32 + lane;
-          if (b < B) {
-            plan_kv[b] = kv4[u];
-            plan_L[b] = L4[u];
-          }
-        }
-      }
-      __syncwarp();
-    }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  int* merge_claimed = const_cast<int*>(misc) + 4;
+  int* merge_done = const_cast<int*>(misc) + 5;
+  // The plan (identical for every layer) is worked out by the warps that need
+  // it, in one copy of code that runs while the others already wait for their
+  // first item: the producer needs the CTA's first and last tile, the first
+  // merge warp the split groups the CTA contributes to. (One warp planning for
+  // all before a block barrier, and the producer locating every item again:
+  // 16 paged sequences, 2 layers, 98 us instead of 96.)
+  struct {
+    long long lo, hi;  // the CTA's tiles
+    TileLoc first;     // where tile lo lies
+  } plan{};
+  if (warp == kProducerWarp || warp == kMergeWarp) {
     long long NG = 0;
     int equal = 0;
-    const long long T = total_tiles(B, kvs, Lss, K, g, R, Hkv, S_cap, status, blockIdx.x == 0, &NG, &equal);
+    const long long T = total_tiles(B, kvs, Lss, K, g, R, Hkv, S_cap, status,
+                                    blockIdx.x == 0 && warp == kProducerWarp, &NG, &equal);
     int G = (int)n_ctas;
     if (T > 0) {
       const long long g_cap = div_nn(T + min_tiles - 1, min_tiles);
       if ((long long)G > g_cap) G = (int)g_cap;
     }
     const int c = blockIdx.x;
-    // an item's fixed cost in tiles, less where a CTA has few
-    const int C = T > 0 ? (int)min((long long)item_tiles, div_nn(T, 4 * (long long)G)) : 0;
-    const long long W = T + (long long)C * NG;  // weighted length
     const int p_cta = aligned_ctas(T, NG, equal, G);  // > 0: CTAs of each group
-    long long lo = 0, hi = 0;
+    // an item's fixed cost in tiles, less where a CTA has few
+    const int C = T > 0 && p_cta == 0 ? (int)min((long long)item_tiles, div_nn(T, 4 * (long long)G)) : 0;
+    const long long W = T + (long long)C * NG;  // weighted length
+    long long x0 = 0, x1 = 0;                   // the CTA's range in weighted positions
     if (p_cta > 0) {
       const int grp = c / p_cta, k = c - grp * p_cta;
       if (grp < NG) {
-        lo = (long long)grp * equal + equal * k / p_cta;
-        hi = (long long)grp * equal + equal * (k + 1) / p_cta;
+        x0 = (long long)grp * equal + equal * k / p_cta;
+        x1 = (long long)grp * equal + equal * (k + 1) / p_cta;
       }
     } else if (T > 0 && c < G) {
-      lo = range_lo(c, W, G);
-      hi = range_lo(c + 1, W, G);
-      if (C > 0) {
-        lo = tile_of_weighted(lo, W, T, C, B, kvs, Lss, K, g, R, Hkv, S_cap);
-        hi = tile_of_weighted(hi, W, T, C, B, kvs, Lss, K, g, R, Hkv, S_cap);
-      }
+      x0 = range_lo(c, W, G);
+      x1 = range_lo(c + 1, W, G);
     }
-    int n_items = 0, n_tasks = 0;
-    long long* range = reinterpret_cast<long long*>(smem + SM::kRange);
-    if (lane == 0) {
-      range[0] = lo;
-      range[1] = hi;
-    }
-    if (lo < hi) {
-      int group_lo = 0;
-      for (int e = 0; e < 2; ++e) {
-        const long long pos = e == 0 ? lo : hi - 1;
-        const TileLoc loc = locate_tile(pos, B, kvs, Lss, K, g, R, Hkv, S_cap);
+    if (x0 < x1) {
+      int n_tasks = 0, group_lo = 0;
+      // e = 0: the first tile; 1: the end; 2 (merges): the last tile
+#pragma unroll 1
+      for (int e = 0; e < (warp == kMergeWarp ? 3 : 2); ++e) {
+        if (e == 2 && plan.lo >= plan.hi) break;
+        const TileLoc loc = find_tile(e == 0 ? x0 : e == 1 ? x1 : plan.hi - 1, e == 2 ? 0 : C, T, B, kvs, Lss, K, g, R,
+                                      Hkv, S_cap);
+        if (e == 0) {
+          plan.lo = loc.tile;
+          plan.first = loc;
+        }
+        if (e == 1) plan.hi = loc.tile;
+        if (e == 1 || warp == kProducerWarp) continue;
+        // a group at either end of the range that other CTAs share
         const int nt = loc.p.n_tiles;
-        const int gib = (int)div_nn(pos - loc.seq_start, nt);
+        const int gib = (int)div_nn(loc.tile - loc.seq_start, nt), group = loc.group0 + gib;
         const long long gstart = loc.seq_start + (long long)gib * nt, gend = gstart + nt;
-        const int group = loc.group0 + gib;
-        if (e == 0) group_lo = group;
-        else n_items = group - group_lo + 1;
-        if ((gstart < lo || gend > hi) && !(e == 1 && group == group_lo)) {
-          if (lane == 0) {
-            MergeTask t;
-            t.b = loc.b;
-            t.kvh = gib / loc.p.n_mg;
-            t.mg = gib % loc.p.n_mg;
-            t.rows = min(R, loc.p.M - t.mg * R);
-            t.c0 = p_cta > 0 ? group * p_cta : cta_of(weighted_pos(gstart, group, C), W, G);
-            t.np = p_cta > 0 ? p_cta : cta_of(weighted_pos(gend - 1, group, C), W, G) - t.c0 + 1;
-            t.grp = group;
-            tasks[n_tasks] = t;
-          }
+        MergeTask t;
+        t.b = loc.b;
+        t.kvh = gib / loc.p.n_mg;
+        t.mg = gib % loc.p.n_mg;
+        t.rows = min(R, loc.p.M - t.mg * R);
+        t.c0 = p_cta > 0 ? group * p_cta : cta_of(weighted_pos(gstart, group, C), W, G);
+        t.np = p_cta > 0 ? p_cta : cta_of(weighted_pos(gend - 1, group, C), W, G) - t.c0 + 1;
+        t.grp = group;
+        if (t.np > 1 && !(e == 2 && group == group_lo)) {
+          if (lane == 0) tasks[n_tasks] = t;
           ++n_tasks;
         }
+        if (e == 0) group_lo = group;
       }
+      if (plan.lo >= plan.hi) n_tasks = 0;  // (the range lies in a group's fixed cost)
+      if (warp == kMergeWarp && lane == 0) {
+        misc[1] = n_tasks;
+        misc[3] = merge_chunk_count<D>(tasks, n_tasks);  // merge chunks per layer
+      }
+    } else if (warp == kMergeWarp && lane == 0) {
+      misc[1] = 0;
+      misc[3] = 0;
     }
-    if (lane == 0) {
-      misc[1] = n_tasks;
-      misc[2] = n_items;
-      misc[3] = merge_chunk_count<D>(tasks, n_tasks);  // merge chunks per layer
+    if (warp == kMergeWarp && lane == 0) {
+      __threadfence_block();
+      misc[2] = 1;  // the merge tasks may be read
     }
+    __syncwarp();
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const int n_tasks = misc[1], n_items = misc[2], merge_n = misc[3];
-  int* merge_claimed = const_cast<int*>(misc) + 4;
-  int* merge_done = const_cast<int*>(misc) + 5;
+  // bounded wait (one lane) for the merge tasks
+  auto tasks_ready = [&]() {
+    for (int i = 0; i < kMaxWaitIters; ++i) {
+      if (misc[2]) {
+        __threadfence_block();
+        return true;
+      }
+      if (misc[0]) return false;
+      __nanosleep(64);
+    }
+    return false;
+  };
   // bounded wait until every CTA has finished `layer` (lane 0 polls)
   auto layer_done = [&](int layer) {
     bool ok = false;
@@ -804,8 +780,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
   if (warp == kProducerWarp) {
     // ======================= producer =======================
     const int c = blockIdx.x;
-    const long long lo = reinterpret_cast<const long long*>(smem + SM::kRange)[0];
-    const long long hi = reinterpret_cast<const long long*>(smem + SM::kRange)[1];
+    const long long lo = plan.lo, hi = plan.hi;
     // lane 0 reads the abort flag for the whole warp (the loop body has warp-wide steps)
     auto aborted = [&]() { return __shfl_sync(0xffffffffu, misc[0], 0) != 0; };
     // paged: the page of every tile of the range, read once for all layers
@@ -821,20 +796,49 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       }
       return id;
     };
+    // the item at hand: row group gib of sequence loc.b, from its first tile gstart
+    TileLoc loc = plan.first;
+    int gib = 0;
+    long long gstart = 0;
+    auto first_item = [&]() {
+      loc = plan.first;
+      gib = lo < hi ? (int)div_nn(lo - loc.seq_start, loc.p.n_tiles) : 0;
+      gstart = loc.seq_start + (long long)gib * loc.p.n_tiles;
+    };
+    auto next_item = [&]() {  // (there is one: the range goes on)
+      gstart += loc.p.n_tiles;
+      if (++gib < Hkv * loc.p.n_mg) return;
+      loc.group0 += gib;
+      loc.seq_start = gstart;
+      gib = 0;
+      do {
+        loc.p = seq_plan(++loc.b, B, kvs, Lss, K, g, R, S_cap);
+      } while (!loc.p.ok && loc.b < B);
+    };
     if (pages_cached) {
+      first_item();
       for (long long pos = lo; pos < hi;) {
-        const TileLoc loc = locate_tile(pos, B, kvs, Lss, K, g, R, Hkv, S_cap);
-        const int nt = loc.p.n_tiles;
-        const long long gstart = loc.seq_start + div_nn(pos - loc.seq_start, nt) * nt;
-        const long long iend = gstart + nt < hi ? gstart + nt : hi;
+        const long long iend = gstart + loc.p.n_tiles < hi ? gstart + loc.p.n_tiles : hi;
         const int key0 = (int)(pos - gstart) * kAttnTileKeys;
         for (int i = lane; i < (int)(iend - pos); i += 32)
           tile_page[pos - lo + i] = page_of(loc.b, key0 + i * kAttnTileKeys);
         pos = iend;
+        if (pos < hi) next_item();
       }
       __syncwarp();
     }
+    if (lo >= hi && lane == 0) {  // nothing to do in any layer
+      info[0].last = 2;
+      mbar_arrive(bIFull);
+    }
     uint32_t item_ctr = 0, chunk_ctr = 0;           // items; chunks filled
+    // K and V are read once and pass through L2 first in, first out: a stream
+    // larger than L2 otherwise pushes out the kernel's own code, and a role's
+    // first instructions then wait behind the copies in flight (the first
+    // MMA of the ragged batch issued 4000 cycles after its operands had landed,
+    // with the hint 600): 16 paged sequences, 2 layers, 96 -> 88 us, 32 layers
+    // at B = 1 248 -> 240, ragged B = 64 295 -> 291.
+    const uint64_t policy = evict_first_policy();
     // the next chunk may be filled
     auto chunk_free = [&]() { return bEmpty + 8 * (chunk_ctr % SM::kChunks); };
     auto chunk_parity = [&]() { return ((chunk_ctr / SM::kChunks) & 1) ^ 1; };
@@ -842,13 +846,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       // layer's dependent data (Q, the block's keys) is readable once every
       // CTA has finished the previous layer
       bool ready = layer == 0;
+      first_item();
       for (long long pos = lo; pos < hi && !aborted();) {
         ItemInfo it{};
-        const TileLoc loc = locate_tile(pos, B, kvs, Lss, K, g, R, Hkv, S_cap);
-        const int nt = loc.p.n_tiles;
-        const int gib = (int)div_nn(pos - loc.seq_start, nt);
-        const long long gstart = loc.seq_start + (long long)gib * nt;
-        const long long gend = gstart + nt;
+        const long long gend = gstart + loc.p.n_tiles;
         const long long iend = gend < hi ? gend : hi;
         it.b = loc.b;
         it.kvh = gib / loc.p.n_mg;
@@ -860,6 +861,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         it.partial = ((pos == gstart) && (gend <= hi)) ? 0 : 1;
         it.slot = (pos == gstart) ? 2 * c + 1 : 2 * c;
         it.grp = loc.group0 + gib;
+        it.last = iend >= hi ? 1 : 0;
         const int n_half = (int)(iend - pos), n_tiles = (n_half + 1) >> 1;
         const int zc = loc.b * Hkv + it.kvh;
         const long long item_pos = pos;  // the item's first 64-key tile in the tile sequence
@@ -891,8 +893,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
               // K: per 64 dims 128 keys; V: per 64 keys all dims (boxes of 64 keys x 64 dims)
 #pragma unroll
               for (int hb = 0; hb < SM::kBoxes; ++hb) {
-                if (is_k) tma_load_3d(dst + hb * 16384 + h * 8192, &set.K[layer], bar, hb * 64, y, z);
-                else tma_load_3d(dst + (h * SM::kBoxes + hb) * 8192, &set.V[layer], bar, hb * 64, y, z);
+                if (is_k) tma_load_3d_hint(dst + hb * 16384 + h * 8192, &set.K[layer], bar, hb * 64, y, z, policy);
+                else tma_load_3d_hint(dst + (h * SM::kBoxes + hb) * 8192, &set.V[layer], bar, hb * 64, y, z, policy);
               }
             }
             ++chunk_ctr;
@@ -954,6 +956,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         }
         ready = true;
         ++item_ctr;
+        if (pos < hi) next_item();
         __syncwarp();
       }
     }
@@ -978,12 +981,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         ++chunk_ctr;
         return ch;
       };
-      for (int layer = 0; layer < n_layers && ok; ++layer) {
-        for (int item = 0; item < n_items && ok; ++item, ++item_ctr) {
+      bool none = false;  // the CTA has no item
+      for (int layer = 0; layer < n_layers && ok && !none; ++layer) {
+        for (int last = 0; !last && ok; ++item_ctr) {
           ok = mbar_spin(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
           if (!ok) break;
           const ItemInfo it = info[item_ctr & 1];
           mbar_arrive(bIEmpty + 8 * (item_ctr & 1));
+          last = it.last;
+          if (last == 2) {
+            none = true;
+            break;
+          }
           const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
           const uint32_t ob = item_ctr & 1;
           // Step j: tile j, stream j & 1. S of a step goes where P of the
@@ -1040,7 +1049,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     const uint32_t ts = tmem + lane_off + SM::kColS + st * 128;
     float2* stat = reinterpret_cast<float2*>(smem + SM::kStat);  // [stream][128]
     uint32_t item_ctr = 0, done0 = 0, done1 = 0;   // steps of streams 0 and 1 in the items before this one
-    bool ok = true;
+    bool ok = true, none = false;  // none: the CTA has no item
     // A wait that fails leaves `ok` false; the item is then finished without
     // further waits, so that every thread still reaches every named barrier.
     auto wait = [&](uint32_t bar, uint32_t parity) { ok = ok && warp_wait(bar, parity); };
@@ -1057,14 +1066,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       }
       __nv_bfloat16* O = set.p[layer].O;
       float* lse = set.p[layer].lse;
-      bool failed = false;
-      for (int item = 0; item < n_items; ++item) {
+      bool failed = false;  // (of a wait for an item)
+      for (int last = none ? 1 : 0; !last;) {
         wait(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
         if (softmax_any(!ok)) {
           failed = true;
           break;
         }
         const ItemInfo& it = info[item_ctr & 1];
+        last = it.last;
+        if (last == 2) {
+          none = true;
+          break;
+        }
         const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
         const int steps0 = (n_tiles + 1) >> 1, steps1 = n_tiles >> 1;
         const int my_steps = st ? steps1 : steps0;
@@ -1291,8 +1305,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       // This CTA is done with the layer's items. Once its grid barrier
       // passes, CTAs write layer + 1's partials into the buffer of layer - 2,
       // whose merge must be done first.
-      if (layer >= kAttnPartBufs - 1 && merge_n > 0 && tid == 0 &&
-          !merged_upto((layer - (kAttnPartBufs - 2)) * merge_n))
+      if (layer >= kAttnPartBufs - 1 && tid == 0 &&
+          !(tasks_ready() && merged_upto((layer - (kAttnPartBufs - 2)) * misc[3])))
         ok = false;
       if (softmax_any(!ok || misc[0])) {
         ok = false;
@@ -1315,7 +1329,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
   // instructions and their registers.
   __syncwarp();
   {
-    bool ok = true;
+    bool ok = lane != 0 || tasks_ready();
+    ok = __all_sync(0xffffffffu, ok);
+    const int n_tasks = misc[1], merge_n = misc[3];
     for (int layer = warp >= kMergeWarp ? 0 : n_layers - 1; layer < n_layers && ok && merge_n > 0; ++layer) {
       if (layer < n_layers - 1) {
         ok = layer_done(layer);
@@ -1419,7 +1435,7 @@ static int attn_min_tiles() {
 }
 
 // Tile-equivalents an item costs in the Stream-K split (see
-// tile_of_weighted); the LIBRASPEC_ATTN_ITEM_TILES environment variable
+// find_tile); the LIBRASPEC_ATTN_ITEM_TILES environment variable
 // overrides the default, read once per process.
 static int attn_item_tiles() {
   static int t = [] {
