@@ -3,15 +3,15 @@
 // bf16) are accumulated by the 5th-generation tensor cores in tensor memory
 // and reduced there to per-row (max, sum of exp, argmax, logit of one token)
 // partials, so the logits never reach HBM; a second kernel merges each row's
-// partials in binary64 (Assumption 1's confidence q = softmax(x / T)[token],
+// partials (Assumption 1's confidence q = softmax(x / T)[token],
 // and the max / argmax / Z of the acceptance rows, Sec. 3.1).
 //
 // Work: CTA pairs (cta_group::2), one pair per two SMs. The vocabulary lies
 // on the MMA's M side (256 head rows over the pair, 128 per CTA) and the rows
 // of H on its N side (up to 256, split between the two CTAs), so a k-slab of
 // 64 brings 16 KB of W and N x 64 bytes of H into each CTA. At N = 256 that
-// is 64 bytes per cycle and SM at the tensor peak, which L2 sustains (1269 us
-// for 2112 rows over V = 128256, Dm = 4096: 1.75 PFLOP/s); single-CTA tiles of
+// is 64 bytes per cycle and SM at the tensor peak, which L2 sustains (1180 us
+// for 2112 rows over V = 128256, Dm = 4096: 1.88 PFLOP/s, 1318 us back to back, at the power limit); single-CTA tiles of
 // 128 x 128 need twice the bytes and were bound by them (1920 us). The time
 // of a tile follows its operand bytes, 256 + N (N = 64: 96 us per row tile
 // of that head, 128: 103, 192: 119, 256: 141), so rows are cut into as few
@@ -33,6 +33,7 @@
 // row's 32 logits, reduce them, and combine the four warps' shares. Rows past
 // M and columns past V come from the TMA's zero fill (or are never loaded)
 // and are left out of the statistics.
+#include <cmath>
 #include <cstdio>
 
 #include "tc.cuh"
@@ -49,7 +50,8 @@ constexpr uint32_t kLmATile = kLmHalf * kLmBK * 2;     // 16 KB
 constexpr int kLmBarBytes = (2 * kLmMaxStages + 5) * 8 + 16;  // barriers and the tensor-memory slot
 constexpr int kLmTurn = kLmEpiWarps * 32 * 33 * 4;     // a padded 32 x 32 block per epilogue warp
 constexpr int kLmShares = kLmEpiWarps * kLmRows;       // the warps' (max, sum, argmax) per row
-constexpr int kLmFixed = 1024 + 1024 + kLmTurn + 3 * kLmShares * 4;  // shared memory besides the ring
+// shared memory besides the ring (with log2(e)/T and the token of each row of the item)
+constexpr int kLmFixed = 1024 + 1024 + kLmTurn + 3 * kLmShares * 4 + 2 * kLmRows * 4;
 constexpr int kLmSmemMax = 227 * 1024;
 static_assert(kLmBarBytes <= 1024, "barriers before the ring");
 
@@ -118,6 +120,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
   float* sh_m = turn + kLmEpiWarps * 32 * 33;
   float* sh_z = sh_m + kLmShares;
   int* sh_arg = reinterpret_cast<int*>(sh_z + kLmShares);
+  float* sh_c = reinterpret_cast<float*>(sh_arg + kLmShares);
+  int* sh_tok = reinterpret_cast<int*>(sh_c + kLmRows);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
@@ -126,8 +130,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
   const int nk = Dm / kLmBK / sub;
   auto item_at = [&](int it) { return lm_item(it, pair, pairs, (int)rank, cut); };
 
-  // the merge launch may start its CTAs (they wait for this grid's end)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
       mbar_init(bFull + 8 * s, 1);   // (the leader's) its expect_tx; both CTAs' bytes as transactions
@@ -156,6 +158,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
 
   if (warp == kLmProducer) {
     if (lane == 0) {
+      // One row tile: the head passes through L2 once, ahead of H and the code (64 rows over V = 32896, Dm = 2048:
+      // 39.8 -> 34.1 us). Several: its tiles are read again by the other row tiles, so they keep the usual priority
+      // (2112 rows: 1277 us, evict first 1597).
+      const uint64_t policy = cut.row_tiles == 1 ? evict_first_policy() : evict_normal_policy();
+      const uint64_t keep = cut.row_tiles == 1 ? evict_last_policy() : evict_normal_policy();
       uint32_t s = 0, ph = 0;
       for (int it = 0; it < n_items && ok; ++it) {
         const LmItem x = item_at(it);
@@ -170,8 +177,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
           if (rank == 0) mbar_expect_tx(bFull + 8 * s, 2 * bytes);
           for (int j = 0; j < sub; ++j) {
             const int kc = (k * sub + j) * kLmBK;
-            tma_load_2d_pair(a + j * slab_bytes, mw, bar, kc, x.v0);
-            tma_load_2d_pair(a + j * slab_bytes + kLmATile, mh, bar, kc, hrow);
+            tma_load_2d_pair(a + j * slab_bytes, mw, bar, kc, x.v0, policy);
+            tma_load_2d_pair(a + j * slab_bytes + kLmATile, mh, bar, kc, hrow, keep);
           }
           if (++s == (uint32_t)stages) {
             s = 0;
@@ -223,10 +230,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
     // ===== epilogue: accumulator lane = head row v0 + warp * 32 + lane, column = row of H =====
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
     float* tw = turn + warp * 32 * 33;
-    auto factor = [&](int grow) {  // log2(e) / T of row grow of H
-      float T = temperature ? temperature[grow / rows_per_seq] : 1.f;
-      return log2e_over(T > 0.f ? T : 1.f);
-    };
     // one row tile: the statistics so far of rows threadIdx.x and threadIdx.x + 128
     float run_m[2] = {-INFINITY, -INFINITY}, run_z[2] = {0.f, 0.f};
     int run_arg[2] = {0x7fffffff, 0x7fffffff};
@@ -236,14 +239,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
       const int vw = x.v0 + warp * 32;
       int nvalid = min(min(32, x.rows - warp * 32), V - vw);
       if (cut.row_tiles == 1) nvalid = min(nvalid, (pair + 1) * cut.range - vw);  // the next range's columns
+      // log2(e) / T and the token of the item's rows, read while its MMAs run (a load from global memory takes
+      // thousands of cycles beside the stream of the head: read block by block below, 128 rows over V = 32896, Dm =
+      // 2048 took 70 us)
+      if (it == 0 || cut.row_tiles > 1) {
+        for (int j = threadIdx.x; j < x.nrow; j += kLmEpiWarps * 32) {
+          const int grow = min(x.h0 + j, M - 1);
+          const float T = temperature ? temperature[grow / rows_per_seq] : 1.f;
+          sh_c[j] = log2e_over(T > 0.f ? T : 1.f);
+          sh_tok[j] = tokens && x.h0 + j < M ? tokens[grow] : -1;
+        }
+        epi_sync();
+      }
       if (!(ok = warp_wait(bAccFull + 8 * ab, aph))) break;
       tc_fence_after();
 #pragma unroll 1
       for (int ch = 0; ch < x.nrow / 32; ++ch) {
         const int grow = x.h0 + ch * 32 + lane;  // this thread's row of H
-        const bool valid = grow < M;
-        const int tok = (valid && tokens) ? tokens[grow] : -1;
-        const float c = factor(valid ? grow : 0);
+        const int tok = sh_tok[ch * 32 + lane];
+        const float c = sh_c[ch * 32 + lane];
         uint32_t r[32];
         tmem_ld32(tmem + lane_off + ab * kLmRows + ch * 32, r);
         tmem_wait_ld();
@@ -281,7 +295,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
       for (int h = 0; h < 2; ++h) {
         const int j = threadIdx.x + h * kLmEpiWarps * 32, grow = x.h0 + j;
         if (j >= x.nrow || grow >= M) continue;
-        const float c = factor(grow);
+        const float c = sh_c[j];
         float m = run_m[h];
         int arg = run_arg[h];
 #pragma unroll
@@ -317,58 +331,139 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * kLmRows) : "memory");
 }
 
-// One warp per row (a programmatic dependent launch): the row's partials in binary64. Z = sum_n z_n
-// 2^((m_n - m) c); the argmax is the first column of the largest max (the
-// partials are in column order); the token probability is
-// 2^((x_tok - m) c) / Z.
+// 2^(j / 32) as a sum of two floats.
+struct LmExpTable {
+  float2 t[32];
+};
+
+// (m - mx) c as a sum of two floats, its error at most 2^-46 of it.
+__device__ __forceinline__ void lm_exponent(float m, float mx, float c, float& xh, float& xl) {
+  const float d = __fsub_rn(m, mx), b = __fsub_rn(d, m);
+  const float dl = __fsub_rn(__fsub_rn(m, __fsub_rn(d, b)), __fadd_rn(mx, b));  // the difference's rounding error
+  xh = __fmul_rn(d, c);
+  xl = __fmaf_rn(dl, c, __fmaf_rn(d, c, -xh));
+}
+
+// (h + l) 2^n = 2^(xh + xl) for xh in [-1000, 0] (below, h = l = 0), within 2^-39 of it: the argument is cut at the
+// nearest multiple of 1/32, whose power comes from the table, and the rest g = f ln 2, |g| < 0.011, goes through
+// the Taylor series of e^g, whose first three terms are carried in two floats.
+__device__ __forceinline__ void lm_exp2(float xh, float xl, const float2* table, float& h, float& l, int& n) {
+  if (xh < -1000.f) {
+    h = l = 0.f;
+    n = 0;
+    return;
+  }
+  constexpr float kLn2 = 0x1.62e43p-1f, kLn2Lo = -0x1.05c61p-29f;  // ln 2 to 48 bits
+  const float kf = rintf(xh * 32.f);
+  const int k = (int)kf;
+  const float f0 = __fsub_rn(xh, kf * 0.03125f);  // exact
+  const float f = __fadd_rn(f0, xl), fb = __fsub_rn(f, f0);
+  const float fl = __fadd_rn(__fsub_rn(f0, __fsub_rn(f, fb)), __fsub_rn(xl, fb));
+  const float g = __fmul_rn(f, kLn2);
+  const float gl = __fadd_rn(__fmaf_rn(f, kLn2, -g), __fmaf_rn(f, kLn2Lo, __fmul_rn(fl, kLn2)));
+  const float q = __fmul_rn(g, g);  // g^2 = q + ql
+  const float ql = __fmaf_rn(2.f * g, gl, __fmaf_rn(g, g, -q));
+  const float rest = __fmul_rn(__fmul_rn(q, g), __fmaf_rn(__fmaf_rn(g, 1.f / 120.f, 1.f / 24.f), g, 1.f / 6.f));
+  const float a = __fadd_rn(1.f, g), al = __fsub_rn(g, __fsub_rn(a, 1.f));
+  const float e = __fadd_rn(a, 0.5f * q), el0 = __fsub_rn(0.5f * q, __fsub_rn(e, a));
+  const float el = __fadd_rn(__fadd_rn(al, el0), __fadd_rn(__fmaf_rn(0.5f, ql, gl), rest));
+  const float2 t = table[k & 31];
+  h = __fmul_rn(e, t.x);
+  l = __fadd_rn(__fmaf_rn(e, t.x, -h), __fmaf_rn(e, t.y, __fmul_rn(el, t.x)));
+  n = k >> 5;
+}
+
+// One CTA per row, a programmatic dependent launch: Z = sum_n z_n 2^((m_n - m) c); the argmax is the first column
+// of the largest max; the token probability is 2^((x_tok - m) c) / Z. What bounds it: the powers. In binary64 (a
+// sixty-fourth of the rate), a warp per row, this launch took 9 us of 37 (128 rows over V = 32896, Dm = 2048) and 100 of
+// 1320 (2112 rows over V = 128256, Dm = 4096), so terms and sum are carried in two floats each (2^-39, against the
+// 2^-22 of the z_n) and the last steps in binary64: 31 and 1270 us in all. The launch of the tiles gives no early
+// signal: a merge that may start beside the tiles puts all of its CTAs on the few SMs without one and took 66 us
+// for those 128 rows.
 // A token outside [-1, V) sets LIBRASPEC_ST_BAD_TOKEN (probability NaN).
-__global__ void __launch_bounds__(128) lm_head_merge_kernel(const LmPartial* __restrict__ part, int M, int V,
-                                                            int n_part, const float* __restrict__ temperature,
-                                                            int rows_per_seq, const int32_t* __restrict__ tokens,
-                                                            float* __restrict__ row_stat,
-                                                            int32_t* __restrict__ row_argmax,
-                                                            float* __restrict__ token_prob, int* __restrict__ status) {
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * 4 + (threadIdx.x >> 5);
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // every partial is written
-  if (r >= M) return;
+constexpr int kMergeThreads = 128;
+__global__ void __launch_bounds__(kMergeThreads) lm_head_merge_kernel(
+    const LmPartial* __restrict__ part, int V, int n_part, const float* __restrict__ temperature, int rows_per_seq,
+    const int32_t* __restrict__ tokens, const __grid_constant__ LmExpTable exp_table, float* __restrict__ row_stat,
+    int32_t* __restrict__ row_argmax, float* __restrict__ token_prob, int* __restrict__ status) {
+  __shared__ float2 table[32];
+  __shared__ float sh_m[kMergeThreads / 32];
+  __shared__ int sh_arg[kMergeThreads / 32];
+  __shared__ double sh_z[kMergeThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = blockIdx.x;
   const LmPartial* p = part + (size_t)r * n_part;
   float T = temperature ? temperature[r / rows_per_seq] : 1.f;
   if (!(T > 0.f)) T = 1.f;
-  const double c = (double)log2e_over(T);
+  const float c = log2e_over(T);
+  if (warp == 0) table[lane] = exp_table.t[lane];
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every partial is written
   float mx = -INFINITY;
   int arg = 0x7fffffff;
-  for (int n = lane; n < n_part; n += 32) argmax_combine(mx, arg, __ldcg(&p[n].m), __ldcg(&p[n].arg));
+#pragma unroll 4
+  for (int n = threadIdx.x; n < n_part; n += kMergeThreads) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p + n));
+    argmax_combine(mx, arg, v.x, __float_as_int(v.z));
+  }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const float m2 = __shfl_xor_sync(0xffffffffu, mx, off);
     const int a2 = __shfl_xor_sync(0xffffffffu, arg, off);
     argmax_combine(mx, arg, m2, a2);
   }
-  double Z = 0.0;
-  for (int n = lane; n < n_part; n += 32) {
-    const float mn = __ldcg(&p[n].m);
-    if (mn > -INFINITY) Z += (double)__ldcg(&p[n].z) * exp2(((double)mn - (double)mx) * c);
+  if (lane == 0) {
+    sh_m[warp] = mx;
+    sh_arg[warp] = arg;
   }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kMergeThreads / 32; ++w) argmax_combine(mx, arg, sh_m[w], sh_arg[w]);
+  float zh = 0.f, zl = 0.f;
+#pragma unroll 4
+  for (int n = threadIdx.x; n < n_part; n += kMergeThreads) {
+    const float2 v = __ldcg(reinterpret_cast<const float2*>(p + n));
+    if (!(v.x > -INFINITY)) continue;
+    float xh, xl, h, l;
+    int e;
+    lm_exponent(v.x, mx, c, xh, xl);
+    lm_exp2(xh, xl, table, h, l, e);
+    // z_n 2^x (below 2^-126 nothing: the sum has a term of at least 1)
+    const float s = e < -126 ? 0.f : __int_as_float((e + 127) << 23);
+    const float z = v.y * s, t = __fmul_rn(h, z), tl = __fmaf_rn(l, z, __fmaf_rn(h, z, -t));
+    const float sum = __fadd_rn(zh, t), b = __fsub_rn(sum, zh);
+    zl = __fadd_rn(zl, __fadd_rn(__fadd_rn(__fsub_rn(zh, __fsub_rn(sum, b)), __fsub_rn(t, b)), tl));
+    zh = sum;
+  }
+  double Z = (double)zh + (double)zl;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, off);
-  if (lane == 0) {
-    if (row_stat) {
-      row_stat[2 * (size_t)r] = mx;
-      row_stat[2 * (size_t)r + 1] = (float)Z;
-    }
-    if (row_argmax) row_argmax[r] = arg;
-    if (token_prob) {
-      const int tok = tokens ? tokens[r] : -1;
-      if (tok >= V || tok < -1) {
-        raise_status(status, LIBRASPEC_ST_BAD_TOKEN);
-        token_prob[r] = __int_as_float(0x7fc00000);
-      } else {
-        token_prob[r] = tok >= 0 ? (float)(exp2(((double)__ldcg(&p->xtok) - (double)mx) * c) / Z) : 0.f;
-      }
+  if (lane == 0) sh_z[warp] = Z;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  Z = (sh_z[0] + sh_z[1]) + (sh_z[2] + sh_z[3]);
+  if (row_stat) {
+    row_stat[2 * (size_t)r] = mx;
+    row_stat[2 * (size_t)r + 1] = (float)Z;
+  }
+  if (row_argmax) row_argmax[r] = arg;
+  if (token_prob) {
+    const int tok = tokens ? tokens[r] : -1;
+    if (tok >= V || tok < -1) {
+      raise_status(status, LIBRASPEC_ST_BAD_TOKEN);
+      token_prob[r] = __int_as_float(0x7fc00000);
+    } else if (tok < 0) {
+      token_prob[r] = 0.f;
+    } else {
+      float xh, xl, h, l;
+      int e;
+      lm_exponent(__ldcg(&p->xtok), mx, c, xh, xl);
+      lm_exp2(xh, xl, table, h, l, e);
+      const double scale = __hiloint2double((e + 1023) << 20, 0);  // 2^e, e >= -1000
+      token_prob[r] = (float)(((double)h + (double)l) * scale / Z);
     }
   }
 }
+static_assert(sizeof(LmPartial) == 16, "a partial is one float4");
+static_assert(kMergeThreads == 128, "four warps' sums");
 
 int num_sms_current();
 
@@ -389,6 +484,19 @@ static bool make_2d_map(CUtensorMap* map, const void* base, int cols, int rows, 
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+static const LmExpTable& exp_table() {
+  static const LmExpTable table = [] {
+    LmExpTable t;
+    for (int j = 0; j < 32; ++j) {
+      const double v = std::exp2(j / 32.0);
+      t.t[j].x = (float)v;
+      t.t[j].y = (float)(v - (double)t.t[j].x);
+    }
+    return t;
+  }();
+  return table;
 }
 
 // Workspace: the status word, then the partials [M, n_part].
@@ -441,18 +549,18 @@ cudaError_t launch_lm_head_stats(const uint16_t* H, const uint16_t* W, const flo
       n_part, part, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // the merge's CTAs start beside the last tiles and wait for them
+  // the merge launch is prepared while the tiles run (2.5 us less than a plain launch)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((M + 3) / 4);
-  cfg.blockDim = dim3(128);
+  cfg.gridDim = dim3(M);
+  cfg.blockDim = dim3(kMergeThreads);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const LmPartial*)part, M, V, n_part, temperature,
-                            rows_per_seq, tokens, row_stat, row_argmax, token_prob, status);
+  return cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const LmPartial*)part, V, n_part, temperature, rows_per_seq,
+                            tokens, exp_table(), row_stat, row_argmax, token_prob, status);
 }
 
 }  // namespace libraspec

@@ -124,3 +124,34 @@ def test_lm_head_tile_edges(orc, M, V, Dm):
     assert lr.libraspec_get_status(ws) == 0
     flag = _check(orc, H, W, T.cpu().numpy(), 1, tok, out)
     assert flag.sum() <= max(1, M // 20)
+
+
+@pytest.mark.parametrize("M,V", [(3, 20), (40, 40000), (300, 129 * 128 + 1)])
+def test_lm_head_merge_of_steep_and_flat_rows(M, V):
+    """Logits that are exact in fp32 (h_m s_v), tile maxima apart by 0 to 4000 in units of log2: Z and the token
+    probability against binary64. Tolerance: a term's argument |a| <= 32 (smaller terms are below 2^-32 of Z, at most
+    V of them) is rounded by 2^-24 |a| ln 2 = 1.3e-6, ex2.approx adds 2^-22, the sums of 128 terms 7 x 2^-24."""
+    g = np.random.default_rng(M + V)
+    s = (-g.integers(0, 256, size=V) / 4).astype(np.float32)
+    s[: V // 2] -= 64.0  # (whole tiles far below the others)
+    s = torch.from_numpy(s).to(torch.bfloat16)
+    h = torch.tensor([[0.0, 0.25, 1.0, 2.0, 16.0][i % 5] for i in range(M)])
+    T = torch.tensor([[1.0, 0.7, 0.0][i % 3] for i in range(M)])
+    tok = g.integers(0, V, size=M).astype(np.int32)
+    H, W = torch.zeros(M, 64), torch.zeros(V, 64)
+    H[:, 5], W[:, 5] = h, s.float()
+    ws = lr.LmHeadWorkspace(M, V)
+    stat, arg, tp = lr.libraspec_lm_head_stats(H.to(cuda(), torch.bfloat16), W.to(cuda(), torch.bfloat16), ws,
+                                               temperature=T.to(cuda()), tokens=torch.from_numpy(tok).to(cuda()))
+    torch.cuda.synchronize()
+    assert lr.libraspec_get_status(ws) == 0
+    x = np.outer(h.numpy().astype(np.float64), s.float().numpy().astype(np.float64))
+    c = np.where(T.numpy() > 0, 1 / np.maximum(T.numpy().astype(np.float64), 1e-9), 1.0)[:, None]
+    mx = x.max(1)
+    e = np.exp((x - mx[:, None]) * c)
+    Z = e.sum(1)
+    assert (arg.cpu().numpy() == x.argmax(1)).all()
+    assert (stat[:, 0].cpu().numpy() == mx).all()
+    np.testing.assert_allclose(stat[:, 1].cpu().numpy(), Z, rtol=2.5e-6)
+    p = e[np.arange(M), tok] / Z
+    np.testing.assert_allclose(tp.cpu().numpy(), p, rtol=3e-6, atol=1.5e-45)
