@@ -36,7 +36,7 @@ cudaError_t launch_accept_tree(const T*, const int32_t*, const int32_t*, const i
 template <typename T>
 cudaError_t launch_accept(const T*, const T*, const int32_t*, const float*, const float*, const int32_t*,
                           const float*, int, int, int, uint64_t, uint64_t, uint32_t, int32_t*, int32_t*, char*,
-                          const WsLayout&, cudaStream_t, const uint64_t*, bool);
+                          const WsLayout&, cudaStream_t, const uint64_t*, bool, bool);
 cudaError_t launch_selftest_wait(const uint32_t*, uint64_t, int32_t*, int*, cudaStream_t);
 template <typename T>
 cudaError_t launch_accept_plan(const T*, const T*, const float*, const float*, const int32_t*, const float*, int,
@@ -323,7 +323,7 @@ static int accept_t(const T* target_logits, const T* draft_logits, const int32_t
                     const float* dstat, const int32_t* L, const float* temperature, int B, int K, int V, uint64_t seed,
                     uint64_t round_offset, uint32_t seq_offset, int32_t* n_accepted, int32_t* bonus_token,
                     void* workspace, size_t ws_bytes, void* stream, const uint64_t* rng = nullptr,
-                    bool plan_ready = false) {
+                    bool plan_ready = false, bool after_own = false) {
   if (!shapes_ok(B, K, V)) return LIBRASPEC_EINVAL;
   if (B == 0) return LIBRASPEC_OK;
   if (!target_logits || (!draft_logits && K > 0) || (!draft_tokens && K > 0) || !L || !temperature ||
@@ -336,7 +336,7 @@ static int accept_t(const T* target_logits, const T* draft_logits, const int32_t
   return from_cuda(launch_accept<T>(target_logits, draft_logits, draft_tokens, conf, dstat, L, temperature, B, K, V,
                                     seed, round_offset, seq_offset, n_accepted, bonus_token,
                                     static_cast<char*>(workspace), lay, static_cast<cudaStream_t>(stream), rng,
-                                    plan_ready));
+                                    plan_ready, after_own));
 }
 }  // extern "C++"
 
@@ -567,7 +567,8 @@ static int verify_round_t(const T* draft_logits, const int32_t* draft_tokens, co
   if (rc != LIBRASPEC_OK) return rc;
   if ((rc = staged_wait(st, 2, s)) != LIBRASPEC_OK) return rc;
   rc = accept_t(target_logits, draft_logits, draft_tokens, conf, dstat, L, temperature, B, K, V, seed, round_offset,
-                seq_offset, n_accepted, bonus_token, workspace, ws_bytes, stream, st ? st->rng_dev : nullptr, plan);
+                seq_offset, n_accepted, bonus_token, workspace, ws_bytes, stream, st ? st->rng_dev : nullptr, plan,
+                st == nullptr);
   if (rc != LIBRASPEC_OK || !st) return rc;
   cudaError_t e = cudaMemcpyAsync(st->n_host, n_accepted, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(st->bonus_host, bonus_token, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, s);

@@ -91,17 +91,21 @@ __global__ void __launch_bounds__(kRowThreads) tree_argmax_kernel(
 // ---------------------------------------------------------------------------
 // Acceptance of a chain draft (Sec. 3.1: the target verifies every drafted
 // position; the rule is the rejection sampler of Leviathan et al. at T > 0
-// and the argmax match at T = 0), in three launches:
+// and the argmax match at T = 0), in two launches (three above 256
+// sequences):
 //
-// accept_plan_kernel (one CTA). From L[] and the temperatures, the rows the
-//   decisions read: j <= L_b of a greedy sequence (the argmax of row L_b is
-//   its bonus token), j < L_b of a sampling one; cut into S slices, S chosen
-//   so that the units fill the rows grid (one unit per CTA); one 8-byte
-//   descriptor per unit (sequence, row, slice, L_b, and log2(e)/T of a
-//   sampling sequence). A sampling sequence with L_b = 0 is decided here
-//   (its bonus draw). In a whole round this launch runs before the attention
-//   layers.
-// accept_rows_kernel. CTA u reads descriptor u: a greedy row's slice yields
+// The plan. From L[] and the temperatures, the rows the decisions read:
+//   j <= L_b of a greedy sequence (the argmax of row L_b is its bonus token),
+//   j < L_b of a sampling one; cut into S slices, S chosen so that the units
+//   fill the rows grid (one unit per CTA). A sampling sequence with L_b = 0
+//   is decided here (its bonus draw). Up to 256 sequences every rows CTA
+//   makes the plan by itself, a sequence per thread (a prefix sum over the
+//   CTA, less than a microsecond); above, accept_plan_kernel (one CTA) writes
+//   one 8-byte descriptor per unit (sequence, row, slice, L_b, and log2(e)/T
+//   of a sampling sequence), in a whole round before the attention layers.
+//   As a launch of its own for every batch the plan cost 4 us (64 ragged
+//   sequences: 49.4 us, now 45.1).
+// accept_rows_kernel. CTA u works on unit u: a greedy row's slice yields
 //   (max, argmax); a sampling row's slice (max, sum of exp((y - max) / T))
 //   and, from the slice that holds the drafted token x_j, y_{j, x_j}. The CTA
 //   completing a sequence's last slice merges its rows and takes the
@@ -141,7 +145,9 @@ struct AcceptArgs {
   const float* conf;        // [B, K] q_j(x_j)
   const float* dstat;       // [B, K, 2] drafter (max, Z)
   const float* temperature; // [B]
+  const int32_t* L;         // [B]
   int B, K, V;
+  int have_q;               // conf and dstat are given
   int chunkB, SB;           // race slices: length and count per row
   uint64_t seed, round_offset;
   uint32_t seq_offset;
@@ -358,8 +364,43 @@ __device__ bool wait_published(const uint32_t* flag, int* status, uint64_t limit
   }
 }
 
-// The plan of the rows grid (G CTAs). A sequence whose L_b lies outside
-// [0, K], or that samples without q, gets no rows and its result at once.
+// The rows that sequence b's decisions read. A sequence whose L_b lies
+// outside [0, K], or that samples without q, has none and gets its result at
+// once (written where `write` holds).
+__device__ __forceinline__ int planned_rows(int b, int Lb, bool sampling, int K, int have_q, bool write,
+                                            int32_t* __restrict__ n_accepted, int32_t* __restrict__ bonus,
+                                            ResEntry* __restrict__ res, uint32_t* __restrict__ ready,
+                                            int* __restrict__ status) {
+  const bool bad_len = Lb < 0 || Lb > K;
+  const bool bad = bad_len || (sampling && !have_q);
+  if (!bad && !sampling) return Lb + 1;
+  if (!bad && Lb > 0) return Lb;
+  if (!write) return 0;
+  ResEntry en;
+  en.n = bad ? -1 : 0;
+  en.mode = bad ? 0 : 1;  // (no draft to verify: the bonus draw from row 0)
+  en.mp = 0.f;
+  en.invZp = 0.f;
+  if (bad) {
+    n_accepted[b] = 0;
+    bonus[b] = 0;
+    raise_status(status, bad_len ? LIBRASPEC_ST_BAD_LENGTH : LIBRASPEC_ST_MISSING_INPUT);
+  }
+  if (sampling) publish_draw(res, ready, b, en);  // its draw CTAs wait for it
+  return 0;
+}
+
+// Slices per row: as many as the grid of G CTAs holds (one unit per CTA),
+// each of at least 2048 logits.
+__device__ __forceinline__ void plan_slices(int R, int G, int V, int& S, int& chunk) {
+  const int smax = max(1, min(kRowMaxSplits, (V + 2047) / 2048));
+  S = R > 0 ? G / R : 1;
+  S = max(1, min(S, smax));
+  chunk = (((V + S - 1) / S) + kRowAlign - 1) & ~(kRowAlign - 1);
+  S = (V + chunk - 1) / chunk;
+}
+
+// The plan of the rows grid (G CTAs) above kPlanInline sequences.
 __global__ void __launch_bounds__(kPlanThreads) accept_plan_kernel(const int32_t* __restrict__ Ls,
                                                                    const float* __restrict__ temperature,
                                                                    int have_q, int B, int K, int V, int G,
@@ -384,27 +425,7 @@ __global__ void __launch_bounds__(kPlanThreads) accept_plan_kernel(const int32_t
     const int Lb = Ls[b];
     const float tb = temperature[b];
     const bool sampling = tb > 0.f;
-    const bool bad_len = Lb < 0 || Lb > K;
-    int r = 0;
-    ResEntry en;
-    en.n = -1;
-    en.mode = 0;
-    en.mp = 0.f;
-    en.invZp = 0.f;
-    if (bad_len || (sampling && !have_q)) {
-      n_accepted[b] = 0;
-      bonus[b] = 0;
-      if (sampling) publish_draw(res, ready, b, en);  // its draw CTAs wait for a draw (none)
-      raise_status(status, bad_len ? LIBRASPEC_ST_BAD_LENGTH : LIBRASPEC_ST_MISSING_INPUT);
-    } else if (!sampling) {
-      r = Lb + 1;
-    } else if (Lb > 0) {
-      r = Lb;
-    } else {  // no draft to verify: the bonus draw from row 0
-      en.n = 0;
-      en.mode = 1;
-      publish_draw(res, ready, b, en);
-    }
+    const int r = planned_rows(b, Lb, sampling, K, have_q, true, n_accepted, bonus, res, ready, status);
     s_start[b] = r;  // rows for now, turned into the prefix below
     s_c[b] = sampling ? log2e_over(tb) : 0.f;
     s_L[b] = Lb;
@@ -441,13 +462,8 @@ __global__ void __launch_bounds__(kPlanThreads) accept_plan_kernel(const int32_t
     }
   }
   const int R = s_tot;
-  // slices per row: as many as the grid holds (one unit per CTA), each of at
-  // least 2048 logits
-  const int smax = max(1, min(kRowMaxSplits, (V + 2047) / 2048));
-  int S = R > 0 ? G / R : 1;
-  S = max(1, min(S, smax));
-  const int chunk = (((V + S - 1) / S) + kRowAlign - 1) & ~(kRowAlign - 1);
-  S = (V + chunk - 1) / chunk;
+  int S, chunk;
+  plan_slices(R, G, V, S, chunk);
   const int U = R * S;
   if (tid == 0) {
     s_start[B] = R;
@@ -466,7 +482,9 @@ __global__ void __launch_bounds__(kPlanThreads) accept_plan_kernel(const int32_t
   }
 }
 
-template <bool VEC, typename E>
+// PLAN: at most kPlanInline sequences, the plan made here.
+constexpr int kPlanInline = kRowThreads;
+template <bool VEC, typename E, bool PLAN>
 __global__ void __launch_bounds__(kRowThreads, 6) accept_rows_kernel(const AcceptArgs<E> a) {
   __shared__ float s_m[kAccMaxRows];
   __shared__ double s_Z[kAccMaxRows];
@@ -475,21 +493,72 @@ __global__ void __launch_bounds__(kRowThreads, 6) accept_rows_kernel(const Accep
   __shared__ int smi[32];
   __shared__ int sh[1];
   __shared__ float s_yx;
-  // the race launch may start its CTAs (they wait for this grid's end)
+  __shared__ int4 s_unit;  // this unit's sequence, row, L_b, log2(e)/T
+  // the race launch may start its CTAs (each waits for its own sequence)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // after the attention layers of a round: a programmatic dependent launch
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = gridDim.x;
   const int K = a.K, V = a.V;
-  const AccPlanHeader h = *a.hdr;
-  uint2 d = a.desc[blockIdx.x];  // read beside the header (stale beyond the plan's units)
-  if ((int)blockIdx.x >= h.U) return;
-  const int S = h.S, chunk = h.chunk;
+  int S, chunk, U;
+  uint2 d = make_uint2(0, 0);
+  int my_rows = 0, my_first = 0, my_L = 0;  // PLAN: of sequence tid
+  float my_c = 0.f;
+  if constexpr (PLAN) {
+    if (tid < a.B) {
+      my_L = a.L[tid];
+      const float tb = a.temperature[tid];
+      my_rows = planned_rows(tid, my_L, tb > 0.f, K, a.have_q, blockIdx.x == 0, a.n_accepted, a.bonus, a.res, a.ready,
+                             a.status);
+      my_c = tb > 0.f ? log2e_over(tb) : 0.f;
+    }
+    int incl = my_rows;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    if (lane == 31) smi[warp] = incl;
+    __syncthreads();
+    int R = 0;
+    my_first = incl - my_rows;
+#pragma unroll
+    for (int w = 0; w < kRowThreads / 32; ++w) {
+      if (w < warp) my_first += smi[w];
+      R += smi[w];
+    }
+    plan_slices(R, G, V, S, chunk);
+    U = R * S;
+  } else {
+    const AccPlanHeader h = *a.hdr;
+    d = a.desc[blockIdx.x];  // read beside the header (stale beyond the plan's units)
+    S = h.S;
+    chunk = h.chunk;
+    U = h.U;
+  }
 
-  for (int u = blockIdx.x; u < h.U; u += G) {
-    if (u != (int)blockIdx.x) d = a.desc[u];
-    const int b = (int)(d.x & 0xfffu), j = (int)((d.x >> 12) & 0x7fu), s = (int)((d.x >> 19) & 0x3fu);
-    const int Lb = (int)(d.x >> 25);
-    const float c = __uint_as_float(d.y);
+  for (int u = blockIdx.x; u < U; u += G) {
+    int b, j, s, Lb;
+    float c;
+    if constexpr (PLAN) {
+      const int r = u / S;
+      s = u - r * S;
+      if (r >= my_first && r < my_first + my_rows)
+        s_unit = make_int4(tid, r - my_first, my_L, __float_as_int(my_c));
+      __syncthreads();  // (and smi has been read)
+      b = s_unit.x;
+      j = s_unit.y;
+      Lb = s_unit.z;
+      c = __int_as_float(s_unit.w);
+    } else {
+      if (u != (int)blockIdx.x) d = a.desc[u];
+      b = (int)(d.x & 0xfffu);
+      j = (int)((d.x >> 12) & 0x7fu);
+      s = (int)((d.x >> 19) & 0x3fu);
+      Lb = (int)(d.x >> 25);
+      c = __uint_as_float(d.y);
+    }
     const bool sampling = c > 0.f;
     const int rows_b = sampling ? Lb : Lb + 1;
     const size_t row = (size_t)b * (K + 1) + j;
@@ -882,6 +951,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) tree_walk_kernel(
     int32_t* __restrict__ last_node, int32_t* __restrict__ bonus, int* __restrict__ status) {
   __shared__ int arg_s[kWalkWarps][kWalkNodes];
   __shared__ int next_s[kWalkWarps][kWalkNodes];
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every node's draw is written
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * kWalkWarps + w;
   if (b >= B) return;
@@ -967,9 +1037,18 @@ cudaError_t launch_accept_tree(const T* target, const int32_t* tokens, const int
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  tree_walk_kernel<<<(B + kWalkWarps - 1) / kWalkWarps, kWalkWarps * 32, 0, stream>>>(
-      tokens, parent, L, B, K, V, rstat, n_accepted, last_node, bonus, st);
-  return cudaGetLastError();
+  // the walk's launch is prepared while the rows run (2 trees of 257 nodes: 88.7 -> 86.7 us)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((B + kWalkWarps - 1) / kWalkWarps);
+  cfg.blockDim = dim3(kWalkWarps * 32);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, tree_walk_kernel, tokens, parent, L, B, K, V, (const RowStat*)rstat, n_accepted,
+                            last_node, bonus, st);
 }
 template cudaError_t launch_accept_tree<float>(const float*, const int32_t*, const int32_t*, const int32_t*,
                                                const float*, int, int, int, uint64_t, uint64_t, uint32_t, int32_t*,
@@ -989,7 +1068,7 @@ int accept_grid() {
   int g = cached[dev];
   if (g == 0) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accept_rows_kernel<VEC, T>, kRowThreads, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, accept_rows_kernel<VEC, T, true>, kRowThreads, 0) !=
             cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
@@ -1006,12 +1085,13 @@ bool accept_vec(const T* target, const T* draft, int V) {
 }
 
 // The acceptance plan for the rows grid of launch_accept<T> with the same
-// pointers' alignment (one CTA; needs only L and the temperatures).
+// pointers' alignment (one CTA; needs only L and the temperatures); nothing
+// up to kPlanInline sequences, whose rows CTAs make it.
 template <typename T>
 cudaError_t launch_accept_plan(const T* target, const T* draft, const float* conf, const float* dstat,
                                const int32_t* L, const float* temperature, int B, int K, int V, int32_t* n_accepted,
                                int32_t* bonus, char* ws, const WsLayout& lay, cudaStream_t stream) {
-  if (B == 0) return cudaSuccess;
+  if (B <= kPlanInline) return cudaSuccess;
   const int G = accept_vec(target, draft, V) ? accept_grid<true, T>() : accept_grid<false, T>();
   if (G <= 0) return cudaErrorInvalidConfiguration;
   accept_plan_kernel<<<1, kPlanThreads, 0, stream>>>(
@@ -1024,13 +1104,17 @@ cudaError_t launch_accept_plan(const T* target, const T* draft, const float* con
 
 // rng (optional, device): {seed, round_offset, seq_offset} read by the
 // kernels in place of the three arguments. plan_ready: launch_accept_plan
-// already ran for these inputs on this stream.
+// already ran for these inputs on this stream. after_own: the launch before
+// this one on the stream is one of this call's, without a programmatic
+// trigger, so that the rows may be launched dependent on it (the rows after a
+// round's layers: with the plan 91.5 -> 84.8 us, 16 sampling sequences). A launch behind a draw never is: the draws
+// may end before their rows.
 template <typename T>
 cudaError_t launch_accept(const T* target, const T* draft, const int32_t* tokens, const float* conf,
                           const float* dstat, const int32_t* L, const float* temperature, int B, int K, int V,
                           uint64_t seed, uint64_t round_offset, uint32_t seq_offset, int32_t* n_accepted,
                           int32_t* bonus, char* ws, const WsLayout& lay, cudaStream_t stream,
-                          const uint64_t* rng, bool plan_ready) {
+                          const uint64_t* rng, bool plan_ready, bool after_own) {
   if (B == 0) return cudaSuccess;
   if (!plan_ready) {
     const cudaError_t e = launch_accept_plan<T>(target, draft, conf, dstat, L, temperature, B, K, V, n_accepted,
@@ -1045,6 +1129,8 @@ cudaError_t launch_accept(const T* target, const T* draft, const int32_t* tokens
   a.conf = conf;
   a.dstat = dstat;
   a.temperature = temperature;
+  a.L = L;
+  a.have_q = conf != nullptr && dstat != nullptr;
   a.B = B;
   a.K = K;
   a.V = V;
@@ -1072,22 +1158,21 @@ cudaError_t launch_accept(const T* target, const T* draft, const int32_t* tokens
   a.status = reinterpret_cast<int*>(ws + lay.status);
   const int G = vec ? accept_grid<true, T>() : accept_grid<false, T>();
   if (G <= 0) return cudaErrorInvalidConfiguration;
-  if (vec)
-    accept_rows_kernel<true, T><<<G, kRowThreads, 0, stream>>>(a);
-  else
-    accept_rows_kernel<false, T><<<G, kRowThreads, 0, stream>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // the draws: launched once every rows CTA has started (each waits for its sequence)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.SB, B);
+  cfg.gridDim = dim3(G);
   cfg.blockDim = dim3(kRowThreads);
-  cfg.dynamicSmemBytes = 0;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
+  cfg.numAttrs = after_own || (!plan_ready && B > kPlanInline) ? 1 : 0;
+  auto* rows = vec ? (B <= kPlanInline ? accept_rows_kernel<true, T, true> : accept_rows_kernel<true, T, false>)
+                   : (B <= kPlanInline ? accept_rows_kernel<false, T, true> : accept_rows_kernel<false, T, false>);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, rows, a);
+  if (e != cudaSuccess) return e;
+  // the draws: launched once every rows CTA has started (each waits for its sequence)
+  cfg.gridDim = dim3(a.SB, B);
   cfg.numAttrs = 1;
   if (vec) return cudaLaunchKernelEx(&cfg, accept_race_kernel<true, T>, a);
   return cudaLaunchKernelEx(&cfg, accept_race_kernel<false, T>, a);
@@ -1095,7 +1180,7 @@ cudaError_t launch_accept(const T* target, const T* draft, const int32_t* tokens
 template cudaError_t launch_accept<float>(const float*, const float*, const int32_t*, const float*, const float*,
                                           const int32_t*, const float*, int, int, int, uint64_t, uint64_t, uint32_t,
                                           int32_t*, int32_t*, char*, const WsLayout&, cudaStream_t,
-                                          const uint64_t*, bool);
+                                          const uint64_t*, bool, bool);
 template cudaError_t launch_accept_plan<float>(const float*, const float*, const float*, const float*,
                                                const int32_t*, const float*, int, int, int, int32_t*, int32_t*,
                                                char*, const WsLayout&, cudaStream_t);
@@ -1111,6 +1196,6 @@ cudaError_t launch_selftest_wait(const uint32_t* flag, uint64_t limit_ns, int32_
 template cudaError_t launch_accept<uint16_t>(const uint16_t*, const uint16_t*, const int32_t*, const float*,
                                              const float*, const int32_t*, const float*, int, int, int, uint64_t,
                                              uint64_t, uint32_t, int32_t*, int32_t*, char*, const WsLayout&,
-                                             cudaStream_t, const uint64_t*, bool);
+                                             cudaStream_t, const uint64_t*, bool, bool);
 
 }  // namespace libraspec

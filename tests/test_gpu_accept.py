@@ -206,3 +206,33 @@ def test_races_on_flat_steep_and_short_rows(orc, dtype, V, scale, T):
                                  L_t.cpu().numpy(), temp.cpu().numpy(), 78, 3)
     for a, r, what in zip(out, ref, ("n_accepted", "last_node", "bonus_token")):
         assert_exact_unless_flagged(a.cpu().numpy(), r, flag, what)
+
+
+@pytest.mark.parametrize("B,K,V", [(1, 1, 300), (31, 4, 2049), (255, 2, 2048), (256, 64, 130), (257, 3, 2051)])
+def test_accept_plan_edges(orc, B, K, V):
+    """The plan made by every rows CTA (up to 256 sequences, from one unit to more units than CTAs) and by a launch of
+    its own (257): lengths 0 to K, greedy and sampling, and two sequences of a bad length, which get (0, 0)."""
+    g = torch.Generator(device="cuda").manual_seed(B + V)
+    rng = np.random.default_rng(B)
+    T = torch.tensor([[0.0, 0.8, 1.0][i % 3] for i in range(B)], device=cuda())
+    draft = torch.randn((B, K, V), generator=g, device=cuda()) * 2
+    inp = {"draft_logits": draft, "draft_tokens": draft.argmax(2).to(torch.int32), "temperature": T,
+           "target_logits": torch.cat([draft, draft[:, :1]], 1)
+           + torch.randn((B, K + 1, V), generator=g, device=cuda()) * 0.3}
+    L = rng.integers(0, K + 1, size=B).astype(np.int32)
+    bad = rng.permutation(B)[:2] if B > 2 else np.zeros(0, np.int64)
+    ws = lr.Workspace(B, K, V, device=cuda())
+    conf, dstat = lr.libraspec_confidence(draft, inp["draft_tokens"], T, ws)
+    for _ in range(2):  # the counters and flags are left as they were found
+        Lb = L.copy()
+        Lb[bad] = [-1, K + 1][: len(bad)]
+        n, bonus = lr.libraspec_accept(inp["target_logits"], draft, inp["draft_tokens"], conf, dstat,
+                                       torch.from_numpy(Lb).to(cuda()), T, 77, ws, round_offset=3)
+        torch.cuda.synchronize()
+        assert lr.libraspec_get_status(ws) == (lr.ST_BAD_LENGTH if len(bad) else 0)
+    n, bonus = n.cpu().numpy(), bonus.cpu().numpy()
+    assert (n[bad] == 0).all() and (bonus[bad] == 0).all()
+    n_ref, b_ref, flag = _oracle_accept(orc, inp, L, 77, 3)
+    good = np.setdiff1d(np.arange(B), bad)
+    assert_exact_unless_flagged(n[good], n_ref[good], flag[good], "n_accepted")
+    assert_exact_unless_flagged(bonus[good], b_ref[good], flag[good], "bonus_token")
