@@ -1332,7 +1332,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     bool ok = lane != 0 || tasks_ready();
     ok = __all_sync(0xffffffffu, ok);
     const int n_tasks = misc[1], merge_n = misc[3];
-    for (int layer = warp >= kMergeWarp ? 0 : n_layers - 1; layer < n_layers && ok && merge_n > 0; ++layer) {
+    // (with more parts than rows some CTAs have a share of no rows: their first merge warp still passes the groups'
+    // counters, which the last of the np CTAs resets)
+    const bool merging = warp == kMergeWarp ? n_tasks > 0 : merge_n > 0;
+    for (int layer = warp >= kMergeWarp && merge_n > 0 ? 0 : n_layers - 1; layer < n_layers && ok && merging; ++layer) {
       if (layer < n_layers - 1) {
         ok = layer_done(layer);
       } else if (warp == kMergeWarp) {

@@ -252,3 +252,24 @@ def test_attn_equal_groups_get_whole_ctas(orc, B, kv, L, Hq, Hkv, d):
     for _ in range(2):
         O, lse = _run(Q, Kc, Vc, kvs, Ls, K)
         check_attn(O, lse, O_ref, lse_ref, Ls, rows=[tuple(r) for r in rows])
+
+
+@pytest.mark.parametrize("n_layers", [1, 2])
+@pytest.mark.parametrize("L,Hq,Hkv,kv", [(0, 2, 2, 1900), (1, 8, 2, 1101)])
+def test_attn_more_parts_than_rows_on_one_workspace(orc, n_layers, L, Hq, Hkv, kv):
+    """Row groups of 1 and 8 rows spread over 30 and 18 CTAs, most of which have no row to merge: the groups' counters
+    are left at zero for the next call all the same (new inputs every call). Tolerances as in check_attn."""
+    K, d = 4, 64
+    S_cap = kv + K + 1
+    ws = lr.Workspace(1, K, 1, Hq, Hkv, d, S_cap, device=cuda())
+    kv_t = torch.tensor([kv], dtype=torch.int32, device=cuda())
+    L_t = torch.tensor([L], dtype=torch.int32, device=cuda())
+    for call in range(6):
+        layers = [dict(zip(("Q", "Kc", "Vc"), _inputs(1, K, Hq, Hkv, d, None, S_cap, seed=10 * call + l, scale_k=2.0)))
+                  for l in range(n_layers)]
+        Os, lses = lr.libraspec_verify_attn_layers(layers, kv_t, L_t, ws, want_lse=True)
+        torch.cuda.synchronize()
+        assert lr.libraspec_get_status(ws) == 0
+        for lay, O, lse in zip(layers, Os, lses):
+            O_ref, lse_ref = orc.verify_attn(lay["Q"], lay["Kc"], lay["Vc"], np.array([kv]), np.array([L]))
+            check_attn(O, lse, O_ref, lse_ref, [L])
