@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2608_08721_gb300 import binding as lr
 
@@ -120,3 +121,15 @@ def test_newer_entry_points_reject_bad_arguments_before_any_launch(lib):
     assert lib.libraspec_selftest_wait(fake, 3_000_000_000, fake, fake256, 256, None) == lr.EINVAL
     assert lib.libraspec_selftest_wait(None, 1000, fake, fake256, 256, None) == lr.EINVAL
     assert lib.libraspec_selftest_wait(fake, 1000, fake, fake256, 16, None) == lr.EINVAL
+
+
+@pytest.mark.parametrize("t,dtype,shape,error", [
+    (3, torch.float32, None, TypeError),
+    (torch.zeros(2), torch.int32, None, TypeError),
+    (torch.zeros(2), torch.float32, (2,), ValueError),  # not on a CUDA device
+])
+def test_argument_checks_name_what_is_wrong(t, dtype, shape, error):
+    with pytest.raises(error, match="^x "):
+        lr._req(t, dtype, "x", shape)
+    with pytest.raises((TypeError, ValueError), match=r"^Q\[0\] "):
+        lr._check_layers([{"Q": t, "K": t, "V": t}], "K", "V", (2,), (2,))
