@@ -749,9 +749,10 @@ def measure_workload(args, w, dev, rank, world, local_rank, steps, primary):
                             "frac_of_measured_hbm": round(nbytes / sec / 1e9 / hbm_peak, 4)}
     # kernels launched per round: confidence + selection (one fused launch for the Thm. 4 selector, the LM
     # head's GEMM + merge + selection, or confidence + selection), the attention launches (+ the tree-mask
-    # kernel per launch), and the acceptance: plan + rows + draws (the tree: statistics + walk)
+    # kernel per launch), and the acceptance: rows + draws, above 256 sequences the
+    # plan before them (the tree: statistics + walk)
     conf_launches = 3 if args.lm_head else (1 if args.selector == "gain" else 2)
-    accept_launches = 2 if N else 3
+    accept_launches = 2 if N or w.B <= 256 else 3
     launches_per_round = attn_launches * (2 if N else 1) + conf_launches + accept_launches
     return {
         "w": w, "steps": steps, "elapsed_max_ms": elapsed_max, "us_per_round": us_per_round, "by": by,

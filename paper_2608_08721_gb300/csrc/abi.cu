@@ -550,8 +550,8 @@ static int verify_round_t(const T* draft_logits, const int32_t* draft_tokens, co
     rc = from_cuda(launch_select(conf, cost_table, B, K, L, ws, lay, s));
   }
   if (rc != LIBRASPEC_OK) return rc;
-  // the acceptance plan needs only L and the temperatures: it runs here, off
-  // the acceptance's critical path
+  // the acceptance plan needs only L and the temperatures: where it is a launch
+  // of its own (above 256 sequences) it runs here, off the acceptance's critical path
   const bool plan = target_logits != nullptr && (draft_logits != nullptr || K == 0) && aligned(target_logits, sizeof(T));
   if (plan && (rc = from_cuda(launch_accept_plan<T>(target_logits, draft_logits, conf, dstat, L, temperature, B, K,
                                                     V, n_accepted, bonus_token, ws, lay, s))) != LIBRASPEC_OK)

@@ -1107,8 +1107,8 @@ cudaError_t launch_accept_plan(const T* target, const T* draft, const float* con
 // already ran for these inputs on this stream. after_own: the launch before
 // this one on the stream is one of this call's, without a programmatic
 // trigger, so that the rows may be launched dependent on it (the rows after a
-// round's layers: with the plan 91.5 -> 84.8 us, 16 sampling sequences). A launch behind a draw never is: the draws
-// may end before their rows.
+// round's layers: with the plan 91.5 -> 84.8 us, 16 sampling sequences). A
+// launch behind a draw never is: draws may end before their rows.
 template <typename T>
 cudaError_t launch_accept(const T* target, const T* draft, const int32_t* tokens, const float* conf,
                           const float* dstat, const int32_t* L, const float* temperature, int B, int K, int V,

@@ -24,8 +24,8 @@
 // warp holds them all, and its 1150 cycles per 64-key tile did not keep up
 // with HBM, and large trees left the tensor cores idle three quarters of the
 // time. 8 sequences of 131072 keys (64/8 heads): 771 -> 606 us (104% of the
-// copy rate); B = 64 ragged: 326 -> 292; 32 layers at B = 1: 302 -> 254; a
-// 512-node tree, 4 layers: 367 -> 227.
+// copy rate); B = 64 ragged: 326 -> 285; 32 layers at B = 1: 302 -> 230; a
+// 512-node tree, 4 layers: 367 -> 221 (with what is said below).
 //
 // Roles in a CTA (384 threads):
 //  * producer warp: walks the CTA's range layer after layer in items; loads
@@ -390,9 +390,9 @@ struct AttnSmem {
 // [rows*k/np, rows*(k+1)/np) of each group it contributed to (k = its index
 // among the group's np CTAs): O = sum_p w_p O_p / sum_p w_p l_p with
 // w_p = 2^(m_p - M), M = max m_p, parts in CTA order. The share is cut into
-// chunks of (row, 4-column) items that any warp may claim once the layer's
-// grid barrier has passed: the merge warp right away (beside the next
-// layer's items), the softmax warps once their own items are done. A lane
+// chunks of (row, 4-column) items that a warp claims once the layer's grid
+// barrier has passed: the two merge warps, beside the next layer's items; the
+// last layer's any warp whose role is done. A lane
 // loads (m_p, l_p) and its 4 columns of O_p for a batch of parts at once and
 // folds the batch in with a running maximum, so a chunk costs one memory
 // round trip per batch and no weights are staged in shared memory.
@@ -404,7 +404,7 @@ __device__ __forceinline__ int merge_share(const MergeTask& t, int& u0) {
   return (int)((long long)t.rows * (k_me + 1) / t.np) - u0;
 }
 
-constexpr int kMergeLoads = 12;  // of a lane in flight (16 spill registers in the callers)
+constexpr int kMergeLoads = 12;  // of a lane in flight (16 spill registers)
 
 // Items per lane in a chunk of a group of np parts: J items x 12/J parts are
 // in flight per batch, and a share of `items` items costs ceil(items / 32J)
@@ -977,14 +977,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       bool ok = true;
       auto take = [&]() {  // the next chunk, once it is filled
         const uint32_t ch = chunk_ctr % SM::kChunks;
-        ok = ok && mbar_spin(bFull + 8 * ch, (chunk_ctr / SM::kChunks) & 1);
+        ok = ok && mbar_wait(bFull + 8 * ch, (chunk_ctr / SM::kChunks) & 1);
         ++chunk_ctr;
         return ch;
       };
       bool none = false;  // the CTA has no item
       for (int layer = 0; layer < n_layers && ok && !none; ++layer) {
         for (int last = 0; !last && ok; ++item_ctr) {
-          ok = mbar_spin(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
+          ok = mbar_wait(bIFull + 8 * (item_ctr & 1), (item_ctr >> 1) & 1);
           if (!ok) break;
           const ItemInfo it = info[item_ctr & 1];
           mbar_arrive(bIEmpty + 8 * (item_ctr & 1));
@@ -994,7 +994,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             break;
           }
           const int n_half = (it.key1 - it.key0 + kAttnTileKeys - 1) / kAttnTileKeys, n_tiles = (n_half + 1) >> 1;
-          const uint32_t ob = item_ctr & 1;
           // Step j: tile j, stream j & 1. S of a step goes where P of the
           // stream's last step lies, so its PV is issued first.
           for (int j = 0; j < n_tiles + 2 && ok; ++j) {
@@ -1002,9 +1001,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             const uint32_t ts = tmem + SM::kColS + st * 128;
             if (j >= 2) {  // O += P V of step j - 2
               const uint32_t ch = take();
-              ok = ok && mbar_spin(bPFull + 8 * st, (p_par >> st) & 1u);
+              ok = ok && mbar_wait(bPFull + 8 * st, (p_par >> st) & 1u);
               p_par ^= 1u << st;
-              if (j == 2) ok = ok && mbar_spin(bOFree, (item_ctr & 1) ^ 1);
+              if (j == 2) ok = ok && mbar_wait(bOFree, (item_ctr & 1) ^ 1);
               if (!ok) break;
               tc_fence_after();
               constexpr uint32_t idesc = mma_idesc(128, D, 1);
@@ -1017,7 +1016,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
             }
             if (j < n_tiles) {  // S = Q K^T of step j: the group's rows x up to 128 keys
               const uint32_t ch = take();
-              if (j == 0) ok = ok && mbar_spin(bQFull, item_ctr & 1);
+              if (j == 0) ok = ok && mbar_wait(bQFull, item_ctr & 1);
               if (!ok) break;
               tc_fence_after();
               const uint32_t idesc = mma_idesc(128, n_half - 2 * j >= 2 ? 128 : 64, 0);
@@ -1194,7 +1193,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
               }
               tmem_st16(ts + c0 / 2, pk);
             };
-            // 64 keys a trip, the next 32 loaded while these are worked on
+            // (one rolled copy of the code: two, with the next 32 keys loaded ahead, were slower)
             const int n_cols = two ? 128 : 64;
 #pragma unroll 1
             for (int c0 = 0; c0 < n_cols; c0 += 32) {
@@ -1423,8 +1422,8 @@ static bool make_kv_map(CUtensorMap* map, const void* base, int D, int S_cap, in
 
 // Smallest tile range per CTA (1: as many CTAs as there are tiles; at 2, half
 // the CTAs work on 3 sequences of 900 keys and 32 layers take 319 us instead
-// of 235); the LIBRASPEC_ATTN_MIN_TILES environment
-// variable overrides the default, read once per process.
+// of 235); the LIBRASPEC_ATTN_MIN_TILES environment variable overrides the
+// default, read once per process.
 static int attn_min_tiles() {
   static int t = [] {
     int v = 1;
@@ -1437,9 +1436,10 @@ static int attn_min_tiles() {
   return t;
 }
 
-// Tile-equivalents an item costs in the Stream-K split (see
-// find_tile); the LIBRASPEC_ATTN_ITEM_TILES environment variable
-// overrides the default, read once per process.
+// Tile-equivalents an item costs at most in the split by cost (see find_tile);
+// the LIBRASPEC_ATTN_ITEM_TILES environment variable overrides the default,
+// read once per process. 0 / 4 / 6 / 8 / 12: 16 paged sequences, 2 layers 110 /
+// 102 / 102 / 102 / 102 us, ragged B = 64 312 / 296 / 299 / 298 / 301.
 static int attn_item_tiles() {
   static int t = [] {
     int v = 4;
@@ -1581,7 +1581,6 @@ static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* con
   int grid = num_sms_current();  // one CTA per SM (it holds all 512 tensor-memory columns)
   if (grid > kAttnMaxCtas) grid = kAttnMaxCtas;
   auto kern = verify_attn_kernel<D, PAGED>;
-  const int item_tiles = attn_item_tiles();
   const int g = Hq / Hkv;
   const int R = g * (kAttnRows / g);
   // layers beyond kMaxLayers go in further launches of the same kernel
@@ -1648,8 +1647,8 @@ static cudaError_t launch_layers_t(const uint16_t* const* Q, const uint16_t* con
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(
-        &cfg, kern, set, kv_len, L, tree_vis, tree_words(K), block_table, max_pages, page_size, n_pages, attn_page_cache(SM::kPageCap), B, K,
-        Hq, Hkv, S_cap, scale * kLog2e, attn_min_tiles(), item_tiles,
+        &cfg, kern, set, kv_len, L, tree_vis, tree_words(K), block_table, max_pages, page_size, n_pages,
+        attn_page_cache(SM::kPageCap), B, K, Hq, Hkv, S_cap, scale * kLog2e, attn_min_tiles(), attn_item_tiles(),
         reinterpret_cast<float*>(ws + lay.attn_o), reinterpret_cast<float*>(ws + lay.attn_ml), o_part / sizeof(float),
         ml_part / sizeof(float), reinterpret_cast<uint32_t*>(ws + lay.attn_cnt),
         reinterpret_cast<uint32_t*>(ws + lay.attn_grp), reinterpret_cast<int*>(ws + lay.status));
@@ -1669,8 +1668,8 @@ cudaError_t launch_verify_attn_layers(const uint16_t* const* Q, const uint16_t* 
   cudaError_t e = tree_vis(parent, L, B, K, ws, lay, stream, &vis);
   if (e != cudaSuccess) return e;
   auto* launch = D == 128 ? launch_layers_t<128, false> : launch_layers_t<64, false>;
-  return launch(Q, Kc, Vc, n_layers, kv_len, L, vis, nullptr, 0, 0, 0, B, K, Hq, Hkv, S_cap,
-                                          scale, O, lse, ws, lay, stream);
+  return launch(Q, Kc, Vc, n_layers, kv_len, L, vis, nullptr, 0, 0, 0, B, K, Hq, Hkv, S_cap, scale, O, lse, ws, lay,
+                stream);
 }
 
 cudaError_t launch_verify_attn_paged_layers(const uint16_t* const* Q, const uint16_t* const* Kp,
@@ -1685,8 +1684,8 @@ cudaError_t launch_verify_attn_paged_layers(const uint16_t* const* Q, const uint
   cudaError_t e = tree_vis(parent, L, B, K, ws, lay, stream, &vis);
   if (e != cudaSuccess) return e;
   auto* launch = D == 128 ? launch_layers_t<128, true> : launch_layers_t<64, true>;
-  return launch(Q, Kp, Vp, n_layers, kv_len, L, vis, block_table, max_pages, page_size,
-                                         n_pages, B, K, Hq, Hkv, S_cap, scale, O, lse, ws, lay, stream);
+  return launch(Q, Kp, Vp, n_layers, kv_len, L, vis, block_table, max_pages, page_size, n_pages, B, K, Hq, Hkv, S_cap,
+                scale, O, lse, ws, lay, stream);
 }
 
 cudaError_t launch_verify_attn(const uint16_t* Q, const uint16_t* Kc, const uint16_t* Vc, const int32_t* kv_len,

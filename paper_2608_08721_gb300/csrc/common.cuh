@@ -270,18 +270,6 @@ struct Logit<uint16_t> {
   }
 };
 
-// Combine two (m, s) pairs (binary64 sums); c = log2(e) / T.
-__device__ __forceinline__ void combine_ms(float& m, double& s, float m2, double s2, float c) {
-  if (m2 == -INFINITY) return;
-  if (m == -INFINITY) { m = m2; s = s2; return; }
-  if (m2 > m) {
-    s = s * (double)exp2f((m - m2) * c) + s2;
-    m = m2;
-  } else {
-    s = s + s2 * (double)exp2f((m2 - m) * c);
-  }
-}
-
 // (value, index) max with the lowest index winning ties.
 __device__ __forceinline__ void argmax_combine(float& v, int& i, float v2, int i2) {
   if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }

@@ -3,16 +3,17 @@
 // bf16) are accumulated by the 5th-generation tensor cores in tensor memory
 // and reduced there to per-row (max, sum of exp, argmax, logit of one token)
 // partials, so the logits never reach HBM; a second kernel merges each row's
-// partials (Assumption 1's confidence q = softmax(x / T)[token],
-// and the max / argmax / Z of the acceptance rows, Sec. 3.1).
+// partials (Assumption 1's confidence q = softmax(x / T)[token], and the max /
+// argmax / Z of the acceptance rows, Sec. 3.1).
 //
 // Work: CTA pairs (cta_group::2), one pair per two SMs. The vocabulary lies
 // on the MMA's M side (256 head rows over the pair, 128 per CTA) and the rows
 // of H on its N side (up to 256, split between the two CTAs), so a k-slab of
 // 64 brings 16 KB of W and N x 64 bytes of H into each CTA. At N = 256 that
 // is 64 bytes per cycle and SM at the tensor peak, which L2 sustains (1180 us
-// for 2112 rows over V = 128256, Dm = 4096: 1.88 PFLOP/s, 1318 us back to back, at the power limit); single-CTA tiles of
-// 128 x 128 need twice the bytes and were bound by them (1920 us). The time
+// for 2112 rows over V = 128256, Dm = 4096: 1.88 PFLOP/s; 1320 back to back,
+// at the power limit); single-CTA tiles of 128 x 128 need twice the bytes and
+// were bound by them (1920 us). The time
 // of a tile follows its operand bytes, 256 + N (N = 64: 96 us per row tile
 // of that head, 128: 103, 192: 119, 256: 141), so rows are cut into as few
 // tiles as 256 allows, of sizes that differ by 32 at most.

@@ -228,7 +228,7 @@ def test_attn_layer_chain_matches_per_layer_oracle(orc, name, n_layers, L_max):
 @pytest.mark.parametrize("Hq,Hkv,K", [(16, 2, 16), (32, 8, 32), (14, 2, 17), (8, 8, 8)])
 def test_attn_step_and_unit_edges(orc, d, Hq, Hkv, K):
     """Items of one to several 128-key steps whose last is half or full (one stream idle, both, an odd count), and
-    row groups that end inside, at and just past their first unit of 128 rows. Tolerances as in check_attn."""
+    row groups of fewer than 128 rows, of exactly 128, and a second group behind them. Tolerances as in check_attn."""
     kv = [0, 62, 63, 64, 127, 128, 129, 191, 255, 256, 257, 320, 500, 1100]
     L = [K, 0, K, K - 1, K - 2, K, 1, K, K // 2, K, 0, K - 1, K, K]
     S_cap = max(kv) + K + 1
