@@ -1128,6 +1128,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
               la[1] *= f;
               lb[0] *= f;
               lb[1] *= f;
+              // the P read back here was stored by this thread, chunk by chunk; a load is ordered behind a store of the
+              // same thread by the wait alone
+              tmem_wait_st();
 #pragma unroll 1
               for (int c = 0; c < c0 / 2; c += 16) {
                 uint32_t q[16];

@@ -273,3 +273,28 @@ def test_attn_more_parts_than_rows_on_one_workspace(orc, n_layers, L, Hq, Hkv, k
         for lay, O, lse in zip(layers, Os, lses):
             O_ref, lse_ref = orc.verify_attn(lay["Q"], lay["Kc"], lay["Vc"], np.array([kv]), np.array([L]))
             check_attn(O, lse, O_ref, lse_ref, [L])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_attn_late_rise_of_the_reference_max(orc, d):
+    """One key raises a row's max by 2^9 to 2^12 above that of the item's first 32 keys: in each 32-key chunk of a
+    128-key step, in the first step of either stream and in later ones, in some rows of a warp and not in others. The
+    earlier keys keep a good part of the weight (2^6 each, or large values), so that P, l and O rescaled wrongly show.
+    Each of the 128 row groups is one item. Tolerances as in check_attn."""
+    K, Hq, Hkv, kv = 16, 16, 4, 520
+    at = [33, 47, 63, 64, 65, 95, 96, 100, 127, 160, 163, 191, 192, 222, 224, 255,
+          256, 257, 288, 300, 320, 352, 383, 384, 416, 450, 480, 511, 512, 513, 517, 519]
+    B, S_cap = len(at), kv + K + 1
+    L = [[0, 3, 7, 16][b % 4] for b in range(B)]
+    Q, Kc, Vc = _inputs(B, K, Hq, Hkv, d, None, S_cap, seed=d, scale_k=0.1)
+    key = torch.arange(S_cap, device=cuda())
+    level = torch.where((key < 256) & (key % 128 < 32), 0.0, 6.0).repeat(B, 1)  # in log2 of the weight
+    for b, k in enumerate(at):
+        level[b, k] = 9.0 + b % 4
+    Kc[..., 0] = (level * (d ** 0.5 * np.log(2.0))).to(torch.bfloat16)[:, None, :]
+    Q[..., 0] = torch.tensor([1.0, -1.0, 0.9375, 1.0], device=cuda()).repeat(Hq // 4)
+    Vc[:, :, :32] += 4.0
+    O_ref, lse_ref = orc.verify_attn(Q, Kc, Vc, np.array([kv] * B), np.array(L))
+    for _ in range(3):
+        O, lse = _run(Q, Kc, Vc, [kv] * B, L, K)
+        check_attn(O, lse, O_ref, lse_ref, L)
