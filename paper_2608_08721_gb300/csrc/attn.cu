@@ -364,8 +364,8 @@ struct AttnSmem {
   static constexpr int kTasks = kInfo + 2 * 64;
   static constexpr int kTmem = kTasks + 64;
   // [0] abort, [1] merge tasks, [2] the tasks are set, [3] merge chunks per
-  // layer, [4] chunks claimed, [5] chunks done, [6] the last layer's merges
-  // may start
+  // layer, [4] chunks claimed, [5] the last layer's merges may start, [6..8]
+  // chunks done of the layers in each buffer of partials
   static constexpr int kMisc = kTmem + 16;
   // (m, l) of each stream's rows, for the epilogue of an item whose streams are combined
   static constexpr int kStat = kMisc + 48;
@@ -509,7 +509,8 @@ __device__ __forceinline__ void merge_chunk(const MergeTask& t, int u0, int nr, 
 
 // Claims and merges chunks of layers up to `last_layer` until none is left,
 // oldest first. Chunks are numbered [l * C, (l + 1) * C) for layer l on the
-// CTA's monotonic counters; ctr_done counts the chunks merged (stores done).
+// CTA's monotonic counter; ctr_done counts the chunks merged (stores done) of
+// the layers in each buffer of partials.
 template <int D>
 __device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set, const MergeTask* tasks, int n_tasks, int C,
                              int* ctr_claim, int* ctr_done, int K, int Hq, int Hkv, int R,
@@ -550,7 +551,10 @@ __device__ __forceinline__ void merge_chunks(int last_layer, const LayerSet& set
       else merge_chunk<4, D>(t, u0, nr, lc, part_o, part_ml, K, Hq, g, R, O, lse);
     }
     __syncwarp();
-    if (lane == 0) atomicAdd(ctr_done, 1);
+    if (lane == 0) {
+      __threadfence_block();  // (the warp's reads lie before the count)
+      atomicAdd(ctr_done + layer % kAttnPartBufs, 1);
+    }
   }
 }
 
@@ -636,7 +640,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     misc[2] = 0;
     misc[4] = 0;
     misc[5] = 0;
-    misc[6] = 0;
+    for (int i = 0; i < kAttnPartBufs; ++i) misc[6 + i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == kMmaWarp) {
@@ -651,7 +655,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
   __syncthreads();
   tc_fence_after();
   int* merge_claimed = const_cast<int*>(misc) + 4;
-  int* merge_done = const_cast<int*>(misc) + 5;
+  int* merge_done = const_cast<int*>(misc) + 6;
   // The plan (identical for every layer) is worked out by the warps that need
   // it, in one copy of code that runs while the others already wait for their
   // first item: the producer needs the CTA's first and last tile, the first
@@ -759,17 +763,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     bool ok = false;
     if ((threadIdx.x & 31) == 0) {
       for (int i = 0; i < kMaxWaitIters; ++i) {
-        if (misc[6]) { ok = true; break; }
+        if (misc[5]) { ok = true; break; }
         if (misc[0]) break;
         __nanosleep(64);
       }
     }
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
   };
-  // bounded wait (one lane) until the CTA has merged n chunks
-  auto merged_upto = [&](int n) {
+  // bounded wait (one lane) until the next layer may write its partials
+  auto next_buf_free = [&](int layer) {
     for (int i = 0; i < kMaxWaitIters; ++i) {
-      if (*reinterpret_cast<volatile int*>(merge_done) >= n) return true;
+      if (part_buf_free(merge_done, layer, misc[3])) {
+        __threadfence_block();  // (the merges' reads lie before what this thread releases)
+        return true;
+      }
       if (misc[0]) return false;
       __nanosleep(64);
     }
@@ -1307,9 +1314,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
       // This CTA is done with the layer's items. Once its grid barrier
       // passes, CTAs write layer + 1's partials into the buffer of layer - 2,
       // whose merge must be done first.
-      if (layer >= kAttnPartBufs - 1 && tid == 0 &&
-          !(tasks_ready() && merged_upto((layer - (kAttnPartBufs - 2)) * misc[3])))
-        ok = false;
+      if (layer >= kAttnPartBufs - 1 && tid == 0 && !(tasks_ready() && next_buf_free(layer))) ok = false;
       if (softmax_any(!ok || misc[0])) {
         ok = false;
         break;
@@ -1347,7 +1352,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         if (lane == 0) {
           for (int ti = 0; ti < n_tasks && ok; ++ti) ok = wait_counter(grp_cnt + 2 * tasks[ti].grp, tasks[ti].np);
           if (ok) {
-            misc[6] = 1;  // the other warps may start
+            misc[5] = 1;  // the other warps may start
             for (int ti = 0; ti < n_tasks; ++ti) {
               uint32_t* gc = grp_cnt + 2 * tasks[ti].grp;
               if (atomicAdd(gc + 1, 1u) == (uint32_t)tasks[ti].np - 1) {

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 
+#include "attn_rules.h"
 #include "libraspec.h"
 
 namespace libraspec {
@@ -22,9 +23,6 @@ constexpr int kConfMaxSplits = 64;    // CTAs per drafter row
 constexpr int kRowMaxSplits = 64;     // CTAs per target row (acceptance)
 constexpr int kRaceMaxSplits = 128;   // CTAs per sequence for a vocabulary draw
 constexpr int kAttnMaxCtas = 192;     // persistent attention grid cap (one CTA per SM)
-// Buffers of split-group partials: layer l writes buffer l % 3, so layer l's
-// merge may run until layer l + 2 starts, a layer after the one it overlaps.
-constexpr int kAttnPartBufs = 3;
 constexpr int kAttnRows = 128;        // query rows per attention row group (at most)
 constexpr int kAttnTileKeys = 64;     // keys per KV tile
 constexpr int kAttnMaxLayers = LIBRASPEC_ATTN_LAYERS_PER_LAUNCH;  // layers per attention launch
