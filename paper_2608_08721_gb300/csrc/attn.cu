@@ -100,16 +100,7 @@ __device__ __forceinline__ void softmax_sync() {
   asm volatile("bar.sync %0, %1;" ::"n"(kSoftmaxBar), "n"(kSoftmaxWarps * 32) : "memory");
 }
 // Barrier of the softmax warpgroups that also tells whether any of their threads holds `pred`.
-__device__ __forceinline__ bool softmax_any(bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-      "barrier.cta.red.or.aligned.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)pred), "n"(kSoftmaxBar), "n"(kSoftmaxWarps * 32)
-      : "memory");
-  return r != 0;
-}
+__device__ __forceinline__ bool softmax_any(bool pred) { return bar_any<kSoftmaxBar, kSoftmaxWarps * 32>(pred); }
 
 // (d0, d1) = (a0, a1) * b + c, and (d0, d1) += (a0, a1): one instruction for two elements
 __device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c) {

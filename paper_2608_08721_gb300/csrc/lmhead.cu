@@ -252,7 +252,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
         }
         epi_sync();
       }
-      if (!(ok = warp_wait(bAccFull + 8 * ab, aph))) break;
+      // (one verdict of the four warps: they meet at the barriers below)
+      if (!(ok = group_wait<kEpiBar, kLmEpiWarps * 32>(bAccFull + 8 * ab, aph))) break;
       tc_fence_after();
 #pragma unroll 1
       for (int ch = 0; ch < x.nrow / 32; ++ch) {

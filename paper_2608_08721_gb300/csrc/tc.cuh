@@ -64,19 +64,39 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: false once kWaitLimitNs have passed.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// Bounded wait: false once the limit has passed.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_ns();
   for (;;) {
     if (mbar_try_wait(bar, parity)) return true;
-    if (global_ns() - t0 > kWaitLimitNs) return false;
+    if (global_ns() - t0 > limit_ns) return false;
   }
 }
 
 // Bounded wait of a whole (converged) warp, with one verdict for all lanes.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
+}
+
+// Named barrier of THREADS threads (whole warps) that also tells whether any of them holds `pred`.
+template <int BAR, int THREADS>
+__device__ __forceinline__ bool bar_any(bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.aligned.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)pred), "n"(BAR), "n"(THREADS)
+      : "memory");
+  return r != 0;
+}
+
+// Bounded wait of THREADS threads that meet at named barriers: one verdict for all of them. (A warp that gave up by
+// itself, and left, would be missing at the barriers of those whose wait ended in time.)
+template <int BAR, int THREADS>
+__device__ __forceinline__ bool group_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns = kWaitLimitNs) {
+  return !bar_any<BAR, THREADS>(!warp_wait(bar, parity, limit_ns));
 }
 
 // L2 policies of a copy. Evict first: data that is read once; a stream larger

@@ -7,6 +7,9 @@ is pointed at a flag that nothing sets, with a short limit: the status must
 report the timeout, the launch must return, and the same context and a
 re-initialised workspace must then run a verify round that matches the
 oracle."""
+import ctypes
+import os
+import subprocess
 import time
 
 import numpy as np
@@ -15,7 +18,7 @@ import torch
 
 from helpers import check_attn, cuda
 from paper_2608_08721_gb300 import binding as lr
-from paper_2608_08721_gb300 import workloads
+from paper_2608_08721_gb300 import build, workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -74,3 +77,43 @@ def test_selftest_wait_rejects_bad_arguments():
     for limit in (0, 3_000_000_000):
         with pytest.raises(lr.LibraspecError):
             lr.libraspec_selftest_wait(flag, limit, ws)
+
+
+def test_one_warps_wait_that_runs_out_is_the_verdict_of_its_group(tmp_path):
+    """group_wait, the form of the LM head's epilogue: four warps that meet at named barriers, one of them on an
+    mbarrier that nothing completes (limit 5 ms). All four must give up together; then none is missing at the next
+    barrier."""
+    src, so = tmp_path / "group_wait.cu", tmp_path / "group_wait.so"
+    src.write_text(r"""
+#include "tc.cuh"
+using namespace libraspec;
+__global__ void probe(int* verdict) {
+  __shared__ alignas(8) uint64_t bar[2];
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bar[0]), 1);
+    mbar_init(smem_u32(&bar[1]), 1);
+    mbar_arrive(smem_u32(&bar[1]));
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5;
+  for (int late = 0; late < 5; ++late) {  // warp `late` waits for what does not come (4: none does)
+    const bool ok = group_wait<1, 128>(smem_u32(&bar[warp != late]), 0, 5000000);
+    verdict[late * 128 + threadIdx.x] = ok;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+  }
+}
+extern "C" int run(int* verdict, void* stream) {
+  probe<<<1, 128, 0, (cudaStream_t)stream>>>(verdict);
+  return (int)cudaGetLastError();
+}
+""")
+    nvcc = build._nvcc()
+    subprocess.run([nvcc] + build.ARCH + ["-std=c++17", "--expt-relaxed-constexpr", "-shared", "-cudart", "shared",
+                                          "-Xcompiler", "-fPIC", "-I", build.CSRC, "-I",
+                                          os.path.join(build.ROOT, "include"), str(src), "-o", str(so), "-Xlinker",
+                                          "-rpath," + build._cuda_lib_dir(nvcc)], check=True)
+    out = torch.full((5, 128), -1, dtype=torch.int32, device=cuda())
+    stream = torch.cuda.current_stream().cuda_stream
+    assert ctypes.CDLL(str(so)).run(ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(stream)) == 0
+    torch.cuda.synchronize()
+    assert (out[:4] == 0).all() and (out[4] == 1).all()
