@@ -676,8 +676,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
     if (p_cta > 0) {
       const int grp = c / p_cta, k = c - grp * p_cta;
       if (grp < NG) {
-        x0 = (long long)grp * equal + equal * k / p_cta;
-        x1 = (long long)grp * equal + equal * (k + 1) / p_cta;
+        x0 = (long long)grp * equal + group_part(equal, k, p_cta);
+        x1 = (long long)grp * equal + group_part(equal, k + 1, p_cta);
       }
     } else if (T > 0 && c < G) {
       x0 = range_lo(c, W, G);

@@ -10,6 +10,11 @@
 
 namespace libraspec {
 
+// First tile of part k of a row group of `tiles` tiles that p CTAs share
+// (k = p: the end): floor(tiles k / p), whose product would pass 2^31 from 15
+// million tiles on (a billion keys, which pages may repeat).
+LIBRASPEC_HD int group_part(int tiles, int k, int p) { return tiles / p * k + tiles % p * k / p; }
+
 // Buffers of split-group partials: layer l writes buffer l % 3, so layer l's
 // merge may run until layer l + 2 starts, a layer after the one it overlaps.
 constexpr int kAttnPartBufs = 3;

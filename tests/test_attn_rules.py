@@ -15,7 +15,8 @@ def rules(tmp_path_factory):
     src.write_text('#include "attn_rules.h"\n'
                    'extern "C" int part_bufs() { return libraspec::kAttnPartBufs; }\n'
                    'extern "C" int buf_free(const int* done, int layer, int chunks) {\n'
-                   '  return libraspec::part_buf_free(done, layer, chunks);\n}\n')
+                   '  return libraspec::part_buf_free(done, layer, chunks);\n}\n'
+                   'extern "C" int part(int tiles, int k, int p) { return libraspec::group_part(tiles, k, p); }\n')
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     return ctypes.CDLL(str(lib))
 
@@ -61,3 +62,10 @@ def test_partials_are_not_overwritten_before_they_are_merged(rules, chunks):
 
 def test_a_cta_without_merge_chunks_never_waits(rules):
     assert all(rules.buf_free((ctypes.c_int * 3)(0, 0, 0), layer, 0) for layer in range(64))
+
+
+@pytest.mark.parametrize("tiles", [1, 151, 152, 2049, 15_000_000, (1 << 31) // 64])
+@pytest.mark.parametrize("p", [1, 2, 7, 152, 192])
+def test_the_parts_of_a_row_group_cover_it_evenly(rules, tiles, p):
+    p = min(p, tiles)
+    assert [rules.part(tiles, k, p) for k in range(p + 1)] == [tiles * k // p for k in range(p + 1)]
