@@ -395,9 +395,13 @@ int libraspec_accept_tree_bf16(const uint16_t* target_logits, const int32_t* dra
  *   NULL (needs tokens).
  * With H the drafter rows (rows_per_seq = K) and tokens the drafted tokens,
  * token_prob and row_stat are libraspec_confidence's conf and dstat. Logits
- * are binary32 accumulations of exact bf16 products; partials merge in
- * binary64. A token outside [-1, V) sets LIBRASPEC_ST_BAD_TOKEN (its
- * probability NaN). Reads W once per 256-row tile of H.
+ * are binary32 accumulations of exact bf16 products; the terms of Z are
+ * binary32, summed over 32 columns in binary32 and from there on in pairs of
+ * binary32 (48 bits, powers to 2^-39), the last steps in binary64; rms error of
+ * Z 6e-8 for exact logits, that of partials merged in binary64. token_prob
+ * holds the tokens' logits in between. A token outside [-1, V) sets
+ * LIBRASPEC_ST_BAD_TOKEN (its probability NaN). Reads W once per 256-row tile
+ * of H.
  * Workspace: libraspec_lm_head_workspace_size(M, V) bytes (status word and
  * the per-tile partials).
  */

@@ -51,16 +51,81 @@ constexpr uint32_t kLmATile = kLmHalf * kLmBK * 2;     // 16 KB
 constexpr int kLmBarBytes = (2 * kLmMaxStages + 5) * 8 + 16;  // barriers and the tensor-memory slot
 constexpr int kLmTurn = kLmEpiWarps * 32 * 33 * 4;     // a padded 32 x 32 block per epilogue warp
 constexpr int kLmShares = kLmEpiWarps * kLmRows;       // the warps' (max, sum, argmax) per row
-// shared memory besides the ring (with log2(e)/T and the token of each row of the item)
-constexpr int kLmFixed = 1024 + 1024 + kLmTurn + 3 * kLmShares * 4 + 2 * kLmRows * 4;
+// shared memory besides the ring (with log2(e)/T and the token of each row of the item, and the table of powers)
+constexpr int kLmFixed = 1024 + 1024 + kLmTurn + 3 * kLmShares * 4 + 2 * kLmRows * 4 + 32 * 8;
 constexpr int kLmSmemMax = 227 * 1024;
 static_assert(kLmBarBytes <= 1024, "barriers before the ring");
 
 struct LmPartial {
-  float m, z;  // max of the logits, sum of 2^((x - m) c)
-  int arg;     // first column of the max
-  float xtok;  // in a row's first partial: the logit of the row's token
+  float m, zh, zl;  // max of the logits, sum of 2^((x - m) c) as two floats
+  int arg;          // first column of the max
 };
+
+// 2^(j / 32) as a sum of two floats.
+struct LmExpTable {
+  float2 t[32];
+};
+
+// (m - mx) c as a sum of two floats, its error at most 2^-46 of it.
+__device__ __forceinline__ void lm_exponent(float m, float mx, float c, float& xh, float& xl) {
+  const float d = __fsub_rn(m, mx), b = __fsub_rn(d, m);
+  const float dl = __fsub_rn(__fsub_rn(m, __fsub_rn(d, b)), __fadd_rn(mx, b));  // the difference's rounding error
+  xh = __fmul_rn(d, c);
+  xl = __fmaf_rn(dl, c, __fmaf_rn(d, c, -xh));
+}
+
+// (h + l) 2^n = 2^(xh + xl) for xh in [-1000, 0] (below, h = l = 0), within 2^-39 of it: the argument is cut at the
+// nearest multiple of 1/32, whose power comes from the table, and the rest g = f ln 2, |g| < 0.011, goes through
+// the Taylor series of e^g, whose first three terms are carried in two floats.
+__device__ __forceinline__ void lm_exp2(float xh, float xl, const float2* table, float& h, float& l, int& n) {
+  if (xh < -1000.f) {
+    h = l = 0.f;
+    n = 0;
+    return;
+  }
+  constexpr float kLn2 = 0x1.62e43p-1f, kLn2Lo = -0x1.05c61p-29f;  // ln 2 to 48 bits
+  const float kf = rintf(xh * 32.f);
+  const int k = (int)kf;
+  const float f0 = __fsub_rn(xh, kf * 0.03125f);  // exact
+  const float f = __fadd_rn(f0, xl), fb = __fsub_rn(f, f0);
+  const float fl = __fadd_rn(__fsub_rn(f0, __fsub_rn(f, fb)), __fsub_rn(xl, fb));
+  const float g = __fmul_rn(f, kLn2);
+  const float gl = __fadd_rn(__fmaf_rn(f, kLn2, -g), __fmaf_rn(f, kLn2Lo, __fmul_rn(fl, kLn2)));
+  const float q = __fmul_rn(g, g);  // g^2 = q + ql
+  const float ql = __fmaf_rn(2.f * g, gl, __fmaf_rn(g, g, -q));
+  const float rest = __fmul_rn(__fmul_rn(q, g), __fmaf_rn(__fmaf_rn(g, 1.f / 120.f, 1.f / 24.f), g, 1.f / 6.f));
+  const float a = __fadd_rn(1.f, g), al = __fsub_rn(g, __fsub_rn(a, 1.f));
+  const float e = __fadd_rn(a, 0.5f * q), el0 = __fsub_rn(0.5f * q, __fsub_rn(e, a));
+  const float el = __fadd_rn(__fadd_rn(al, el0), __fadd_rn(__fmaf_rn(0.5f, ql, gl), rest));
+  const float2 t = table[k & 31];
+  h = __fmul_rn(e, t.x);
+  l = __fadd_rn(__fmaf_rn(e, t.x, -h), __fmaf_rn(e, t.y, __fmul_rn(el, t.x)));
+  n = k >> 5;
+}
+
+// (zh + zl) += t + tl, |t| >= |tl|
+__device__ __forceinline__ void two_add(float& zh, float& zl, float t, float tl) {
+  const float sum = __fadd_rn(zh, t), b = __fsub_rn(sum, zh);
+  zl = __fadd_rn(zl, __fadd_rn(__fadd_rn(__fsub_rn(zh, __fsub_rn(sum, b)), __fsub_rn(t, b)), tl));
+  zh = sum;
+}
+
+// (zh + zl) += (vh + vl) 2^((m - mx) c), in two floats; a sum whose maximum is -inf is 0, or NaN.
+__device__ __forceinline__ void lm_add(float& zh, float& zl, float vh, float vl, float m, float mx, float c,
+                                       const float2* table) {
+  if (!(m > -INFINITY)) {
+    zh += vh;
+    return;
+  }
+  float xh, xl, h, l;
+  int e;
+  lm_exponent(m, mx, c, xh, xl);
+  lm_exp2(xh, xl, table, h, l, e);
+  // (below 2^-126 nothing: the sum has a term of at least 1)
+  const float s = e < -126 ? 0.f : __int_as_float((e + 127) << 23);
+  const float z = vh * s, t = __fmul_rn(h, z);
+  two_add(zh, zl, t, __fmaf_rn(l, z, __fmaf_rn(h, vl * s, __fmaf_rn(h, z, -t))));
+}
 
 // How the work is cut. The vocabulary: ranges of `range` columns, each in
 // `tiles` tiles of which the last gives each CTA `tail` head rows (a multiple
@@ -105,8 +170,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
     const __grid_constant__ CUtensorMap mapH, const __grid_constant__ CUtensorMap mapHs,
     const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapWt,
     const float* __restrict__ temperature, int rows_per_seq, const int32_t* __restrict__ tokens, int M, int V, int Dm,
-    LmCut cut, int stages, int sub, int n_part, LmPartial* __restrict__ part,
-    int* __restrict__ status) {
+    LmCut cut, int stages, int sub, int n_part, const __grid_constant__ LmExpTable exp_table,
+    LmPartial* __restrict__ part, float* __restrict__ token_logit, int* __restrict__ status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // a stage holds `sub` consecutive k-slabs (W slab, then H slab), so every row is read `sub` * 128 contiguous
@@ -123,6 +188,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
   int* sh_arg = reinterpret_cast<int*>(sh_z + kLmShares);
   float* sh_c = reinterpret_cast<float*>(sh_arg + kLmShares);
   int* sh_tok = reinterpret_cast<int*>(sh_c + kLmRows);
+  float2* table = reinterpret_cast<float2*>(sh_tok + kLmRows);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
@@ -131,6 +197,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
   const int nk = Dm / kLmBK / sub;
   auto item_at = [&](int it) { return lm_item(it, pair, pairs, (int)rank, cut); };
 
+  if (threadIdx.x < 32) table[threadIdx.x] = exp_table.t[threadIdx.x];
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
       mbar_init(bFull + 8 * s, 1);   // (the leader's) its expect_tx; both CTAs' bytes as transactions
@@ -232,7 +299,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
     float* tw = turn + warp * 32 * 33;
     // one row tile: the statistics so far of rows threadIdx.x and threadIdx.x + 128
-    float run_m[2] = {-INFINITY, -INFINITY}, run_z[2] = {0.f, 0.f};
+    float run_m[2] = {-INFINITY, -INFINITY}, run_zh[2] = {0.f, 0.f}, run_zl[2] = {0.f, 0.f};
     int run_arg[2] = {0x7fffffff, 0x7fffffff};
     for (int it = 0; it < n_items; ++it) {
       const LmItem x = item_at(it);
@@ -287,7 +354,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
         sh_m[at] = cm;
         sh_z[at] = (zs[0] + zs[1]) + (zs[2] + zs[3]);
         sh_arg[at] = ca;
-        if (tok >= vw && tok - vw < nvalid) part[(size_t)grow * n_part].xtok = tw[(tok - vw) * 33 + lane];
+        if (tok >= vw && tok - vw < nvalid && token_logit) token_logit[grow] = tw[(tok - vw) * 33 + lane];
       }
       tc_fence_before();
       __syncwarp();
@@ -306,20 +373,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
             m = sh_m[w * kLmRows + j];
             arg = sh_arg[w * kLmRows + j];
           }
-        float z = run_m[h] == -INFINITY ? 0.f : run_z[h] * ex2_approx((run_m[h] - m) * c);
+        // the tile's sum, then the pair's range so far, in two floats (a sum over the range in one, rescaled by
+        // ex2.approx: rms error of Z against 64 bits 9.5e-8 for 33 rows over V = 128256, with exact logits; so 5.6e-8,
+        // and 6.4e-8 for 128-column partials in one float merged in binary64)
+        const float mt = fmaxf(fmaxf(sh_m[j], sh_m[kLmRows + j]), fmaxf(sh_m[2 * kLmRows + j], sh_m[3 * kLmRows + j]));
+        float zh = 0.f, zl = 0.f;
 #pragma unroll
-        for (int w = 0; w < kLmEpiWarps; ++w)
-          z += sh_z[w * kLmRows + j] * ex2_approx((sh_m[w * kLmRows + j] - m) * c);
+        for (int w = 0; w < kLmEpiWarps; ++w) {
+          const float v = sh_z[w * kLmRows + j], mw = sh_m[w * kLmRows + j];
+          const float f = mw > -INFINITY ? ex2_approx((mw - mt) * c) : 0.f;
+          const float t = __fmul_rn(v, f);
+          two_add(zh, zl, t, __fmaf_rn(v, f, -t));
+        }
+        if (cut.row_tiles == 1 && it > 0) {
+          const bool up = mt > run_m[h];
+          float ah = up ? zh : run_zh[h], al = up ? zl : run_zl[h];
+          lm_add(ah, al, up ? run_zh[h] : zh, up ? run_zl[h] : zl, up ? run_m[h] : mt, m, c, table);
+          zh = ah;
+          zl = al;
+        }
         if (cut.row_tiles == 1) {
           run_m[h] = m;
-          run_z[h] = z;
+          run_zh[h] = zh;
+          run_zl[h] = zl;
           run_arg[h] = arg;
         }
-        if ((cut.row_tiles > 1 || it == n_items - 1) && x.slot < n_part) {
-          LmPartial* p = part + (size_t)grow * n_part + x.slot;
-          *reinterpret_cast<float2*>(p) = make_float2(m, z);
-          p->arg = arg;
-        }
+        if ((cut.row_tiles > 1 || it == n_items - 1) && x.slot < n_part)
+          *reinterpret_cast<float4*>(part + (size_t)grow * n_part + x.slot) =
+              make_float4(m, zh, zl, __int_as_float(arg));
       }
       epi_sync();  // the shares are read before the next item's are written
     }
@@ -333,53 +414,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(2 * kLmRows) : "memory");
 }
 
-// 2^(j / 32) as a sum of two floats.
-struct LmExpTable {
-  float2 t[32];
-};
-
-// (m - mx) c as a sum of two floats, its error at most 2^-46 of it.
-__device__ __forceinline__ void lm_exponent(float m, float mx, float c, float& xh, float& xl) {
-  const float d = __fsub_rn(m, mx), b = __fsub_rn(d, m);
-  const float dl = __fsub_rn(__fsub_rn(m, __fsub_rn(d, b)), __fadd_rn(mx, b));  // the difference's rounding error
-  xh = __fmul_rn(d, c);
-  xl = __fmaf_rn(dl, c, __fmaf_rn(d, c, -xh));
-}
-
-// (h + l) 2^n = 2^(xh + xl) for xh in [-1000, 0] (below, h = l = 0), within 2^-39 of it: the argument is cut at the
-// nearest multiple of 1/32, whose power comes from the table, and the rest g = f ln 2, |g| < 0.011, goes through
-// the Taylor series of e^g, whose first three terms are carried in two floats.
-__device__ __forceinline__ void lm_exp2(float xh, float xl, const float2* table, float& h, float& l, int& n) {
-  if (xh < -1000.f) {
-    h = l = 0.f;
-    n = 0;
-    return;
-  }
-  constexpr float kLn2 = 0x1.62e43p-1f, kLn2Lo = -0x1.05c61p-29f;  // ln 2 to 48 bits
-  const float kf = rintf(xh * 32.f);
-  const int k = (int)kf;
-  const float f0 = __fsub_rn(xh, kf * 0.03125f);  // exact
-  const float f = __fadd_rn(f0, xl), fb = __fsub_rn(f, f0);
-  const float fl = __fadd_rn(__fsub_rn(f0, __fsub_rn(f, fb)), __fsub_rn(xl, fb));
-  const float g = __fmul_rn(f, kLn2);
-  const float gl = __fadd_rn(__fmaf_rn(f, kLn2, -g), __fmaf_rn(f, kLn2Lo, __fmul_rn(fl, kLn2)));
-  const float q = __fmul_rn(g, g);  // g^2 = q + ql
-  const float ql = __fmaf_rn(2.f * g, gl, __fmaf_rn(g, g, -q));
-  const float rest = __fmul_rn(__fmul_rn(q, g), __fmaf_rn(__fmaf_rn(g, 1.f / 120.f, 1.f / 24.f), g, 1.f / 6.f));
-  const float a = __fadd_rn(1.f, g), al = __fsub_rn(g, __fsub_rn(a, 1.f));
-  const float e = __fadd_rn(a, 0.5f * q), el0 = __fsub_rn(0.5f * q, __fsub_rn(e, a));
-  const float el = __fadd_rn(__fadd_rn(al, el0), __fadd_rn(__fmaf_rn(0.5f, ql, gl), rest));
-  const float2 t = table[k & 31];
-  h = __fmul_rn(e, t.x);
-  l = __fadd_rn(__fmaf_rn(e, t.x, -h), __fmaf_rn(e, t.y, __fmul_rn(el, t.x)));
-  n = k >> 5;
-}
-
 // One CTA per row, a programmatic dependent launch: Z = sum_n z_n 2^((m_n - m) c); the argmax is the first column
 // of the largest max; the token probability is 2^((x_tok - m) c) / Z. What bounds it: the powers. In binary64 (a
 // sixty-fourth of the rate), a warp per row, this launch took 9 us of 37 (128 rows over V = 32896, Dm = 2048) and 100 of
 // 1320 (2112 rows over V = 128256, Dm = 4096), so terms and sum are carried in two floats each (2^-39, against the
-// 2^-22 of the z_n) and the last steps in binary64: 31 and 1270 us in all. The launch of the tiles gives no early
+// 2^-22 of the terms of z_n) and the last steps in binary64: 31 and 1270 us in all. The launch of the tiles gives no early
 // signal: a merge that may start beside the tiles puts all of its CTAs on the few SMs without one and took 66 us
 // for those 128 rows.
 // A token outside [-1, V) sets LIBRASPEC_ST_BAD_TOKEN (probability NaN).
@@ -404,7 +443,7 @@ __global__ void __launch_bounds__(kMergeThreads) lm_head_merge_kernel(
 #pragma unroll 4
   for (int n = threadIdx.x; n < n_part; n += kMergeThreads) {
     const float4 v = __ldcg(reinterpret_cast<const float4*>(p + n));
-    argmax_combine(mx, arg, v.x, __float_as_int(v.z));
+    argmax_combine(mx, arg, v.x, __float_as_int(v.w));
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -422,18 +461,8 @@ __global__ void __launch_bounds__(kMergeThreads) lm_head_merge_kernel(
   float zh = 0.f, zl = 0.f;
 #pragma unroll 4
   for (int n = threadIdx.x; n < n_part; n += kMergeThreads) {
-    const float2 v = __ldcg(reinterpret_cast<const float2*>(p + n));
-    if (!(v.x > -INFINITY)) continue;
-    float xh, xl, h, l;
-    int e;
-    lm_exponent(v.x, mx, c, xh, xl);
-    lm_exp2(xh, xl, table, h, l, e);
-    // z_n 2^x (below 2^-126 nothing: the sum has a term of at least 1)
-    const float s = e < -126 ? 0.f : __int_as_float((e + 127) << 23);
-    const float z = v.y * s, t = __fmul_rn(h, z), tl = __fmaf_rn(l, z, __fmaf_rn(h, z, -t));
-    const float sum = __fadd_rn(zh, t), b = __fsub_rn(sum, zh);
-    zl = __fadd_rn(zl, __fadd_rn(__fadd_rn(__fsub_rn(zh, __fsub_rn(sum, b)), __fsub_rn(t, b)), tl));
-    zh = sum;
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p + n));
+    if (v.x > -INFINITY) lm_add(zh, zl, v.y, v.z, v.x, mx, c, table);
   }
   double Z = (double)zh + (double)zl;
 #pragma unroll
@@ -457,7 +486,7 @@ __global__ void __launch_bounds__(kMergeThreads) lm_head_merge_kernel(
     } else {
       float xh, xl, h, l;
       int e;
-      lm_exponent(__ldcg(&p->xtok), mx, c, xh, xl);
+      lm_exponent(__ldcg(token_prob + r), mx, c, xh, xl);  // (the token's logit, left there by the tiles)
       lm_exp2(xh, xl, table, h, l, e);
       const double scale = __hiloint2double((e + 1023) << 20, 0);  // 2^e, e >= -1000
       token_prob[r] = (float)(((double)h + (double)l) * scale / Z);
@@ -548,7 +577,7 @@ cudaError_t launch_lm_head_stats(const uint16_t* H, const uint16_t* W, const flo
   auto* status = reinterpret_cast<int*>(ws);
   lm_head_stats_kernel<<<2 * pairs, kLmThreads, kLmFixed + stages * stage_bytes, stream>>>(
       mapH, mapHs, mapW, mapWt, temperature, rows_per_seq, tokens, M, V, Dm, cut, stages, sub,
-      n_part, part, status);
+      n_part, exp_table(), part, token_prob, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // the merge launch is prepared while the tiles run (2.5 us less than a plain launch)

@@ -130,7 +130,8 @@ def test_lm_head_tile_edges(orc, M, V, Dm):
 def test_lm_head_merge_of_steep_and_flat_rows(M, V):
     """Logits that are exact in fp32 (h_m s_v), tile maxima apart by 0 to 4000 in units of log2: Z and the token
     probability against binary64. Tolerance: a term's argument |a| <= 32 (smaller terms are below 2^-32 of Z, at most
-    V of them) is rounded by 2^-24 |a| ln 2 = 1.3e-6, ex2.approx adds 2^-22, the sums of 128 terms 7 x 2^-24."""
+    V of them) is rounded by 2^-24 |a| ln 2 = 1.3e-6, ex2.approx adds 2^-22, the sum of 32 terms 9 x 2^-24; those sums
+    are added in two floats (2^-39)."""
     g = np.random.default_rng(M + V)
     s = (-g.integers(0, 256, size=V) / 4).astype(np.float32)
     s[: V // 2] -= 64.0  # (whole tiles far below the others)
@@ -155,3 +156,27 @@ def test_lm_head_merge_of_steep_and_flat_rows(M, V):
     np.testing.assert_allclose(stat[:, 1].cpu().numpy(), Z, rtol=2.5e-6)
     p = e[np.arange(M), tok] / Z
     np.testing.assert_allclose(tp.cpu().numpy(), p, rtol=3e-6, atol=1.5e-45)
+
+
+@pytest.mark.parametrize("M", [1, 33, 200, 300])
+def test_lm_head_sum_keeps_small_terms_beside_a_large_one(M):
+    """One column of each row weighs 1 and every other 2^-32 (T = log2(e): logits in units of log2): every power and
+    every product is exact, so Z has its last rounding alone, 2^-24. A CTA's 128 columns add 2^-25 to the 1, which a
+    sum in 32 bits over its six or seven tiles would drop each time."""
+    V = 128256
+    s = torch.full((V, M), -32.0)
+    at = torch.arange(M) * 379 % V  # (in every tile of a CTA's columns)
+    s[at, torch.arange(M)] = 0.0
+    D = (M + 63) // 64 * 64
+    H, W = torch.eye(M, D), torch.zeros(V, D)
+    W[:, :M] = s
+    T = torch.full((M,), float(np.float32(np.log2(np.e))))
+    ws = lr.LmHeadWorkspace(M, V)
+    stat, arg, tp = lr.libraspec_lm_head_stats(H.to(cuda(), torch.bfloat16), W.to(cuda(), torch.bfloat16), ws,
+                                               temperature=T.to(cuda()), tokens=at.int().to(cuda()))
+    torch.cuda.synchronize()
+    assert lr.libraspec_get_status(ws) == 0
+    Z = 1.0 + (V - 1) * 2.0 ** -32
+    assert (arg.cpu() == at).all() and (stat[:, 0] == 0).all()
+    assert np.abs(stat[:, 1].cpu().numpy().astype(np.float64) / Z - 1).max() <= 2.0 ** -24
+    assert np.abs(tp.cpu().numpy().astype(np.float64) * Z - 1).max() <= 2.0 ** -24
