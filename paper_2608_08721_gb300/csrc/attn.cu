@@ -345,7 +345,7 @@ struct AttnSmem {
   static constexpr int kBoxes = D / 64;
   static constexpr int kChunkBytes = kBoxes * 16384;     // K or V of one 128-key tile
   static constexpr int kChunks = D == 128 ? 5 : 10;      // in the ring
-    static constexpr int kQ = 0;
+  static constexpr int kQ = 0;
   static constexpr int kRing = kQ + kBoxes * 16384;      // (Q: per 64 columns 128 rows)
   // mbarriers: full[chunks], empty[chunks], ifull[2], iempty[2], sfull[2], pfull[2], pvdone[2], qfull, qempty,
   // ofree, drain
@@ -1086,6 +1086,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
         const int rr = it.mg * R + row;  // row of the (sequence, kv head)
         const int t_row = rr / g;
         float m_run = -INFINITY, l_run = 0.f;
+        // (a lane past the group's rows holds scores of whatever its Q row is: at 0 they ask for no raise)
+        const float scale_row = valid ? scale_log2 : 0.f;
         {
           // Keys seen by this row: the cache prefix and the root (keys <= kv),
           // then chain: the block positions up to t_row (keys <= kv + t_row);
@@ -1173,7 +1175,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
                 a = fmaxf(fmaxf(a, __uint_as_float(x[c])), __uint_as_float(x[c + 1]));
                 b = fmaxf(fmaxf(b, __uint_as_float(x[c + 2])), __uint_as_float(x[c + 3]));
               }
-              const float cmax = fmaxf(a, b) * scale_log2;
+              const float cmax = fmaxf(a, b) * scale_row;
               if (i == 0 && c0 == 0) m_run = cmax;
               else if (__any_sync(0xffffffffu, cmax > m_run + kRescaleLog2)) raise_to(cmax, c0);
               const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
@@ -1181,8 +1183,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) verify_attn_kernel(
 #pragma unroll
               for (int c = 0; c < 32; c += 4) {
                 float y0, y1, y2, y3;
-                fma2(y0, y1, __uint_as_float(x[c]), __uint_as_float(x[c + 1]), scale_log2, neg_m);
-                fma2(y2, y3, __uint_as_float(x[c + 2]), __uint_as_float(x[c + 3]), scale_log2, neg_m);
+                fma2(y0, y1, __uint_as_float(x[c]), __uint_as_float(x[c + 1]), scale_row, neg_m);
+                fma2(y2, y3, __uint_as_float(x[c + 2]), __uint_as_float(x[c + 3]), scale_row, neg_m);
                 y0 = ex2_approx(y0);
                 y1 = ex2_approx(y1);
                 y2 = ex2_approx(y2);
