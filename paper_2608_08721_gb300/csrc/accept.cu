@@ -4,68 +4,27 @@
 namespace libraspec {
 
 // ---------------------------------------------------------------------------
-// Row statistics of the node rows of a draft tree (the greedy walk reads
-// their argmaxes). Grid (nsplit, K+1, B); rows j > L_b exit at once. Greedy
-// sequences need only max / argmax; sampling sequences need (m, Z) at their
-// temperature. Partials of a row are merged by the last CTA to finish
-// (atomic ticket) into row_stat[b, j].
+// Node rows of a draft tree: grid (nsplit, K+1, B), rows j > L_b exit at once.
+// A row's slices each leave (value, token), and the CTA that completes the row
+// (atomic ticket) takes the token of the largest value (the lowest on ties)
+// into node_arg[b, j], which the walk reads.
 // ---------------------------------------------------------------------------
-template <bool VEC, typename E>
-__global__ void __launch_bounds__(kRowThreads) tree_argmax_kernel(
-    const E* __restrict__ target, const int32_t* __restrict__ Ls, const float* __restrict__ temperature,
-    int K, int V, int nsplit, int chunk, RowPartial* __restrict__ part, uint32_t* __restrict__ cnt,
-    RowStat* __restrict__ stat, int* __restrict__ status) {
-  __shared__ float smf[64];
+__device__ __forceinline__ void tree_row_finish(float m, int arg, int row, int split, int nsplit,
+                                                RowPartial* __restrict__ part, uint32_t* __restrict__ cnt,
+                                                int32_t* __restrict__ node_arg) {
+  __shared__ float smf[32];
   __shared__ int smi[32];
   __shared__ int last;
-  const int split = blockIdx.x, j = blockIdx.y, b = blockIdx.z;
-  const int Lb = Ls[b];
-  if (Lb < 0 || Lb > K) {
-    if (split == 0 && j == 0 && threadIdx.x == 0) raise_status(status, LIBRASPEC_ST_BAD_LENGTH);
-    return;
-  }
-  if (j > Lb) return;
-  const int row = b * (K + 1) + j;
-  const float tb = temperature ? temperature[b] : 0.f;  // none: every sequence greedy
-  const bool sampling = tb > 0.f;
-  const float T = sampling ? tb : 1.f;
-  const float c = log2e_over(T);
-  const E* xr = target + (size_t)row * V;
-  const int c0 = split * chunk, c1 = min(V, c0 + chunk);
-
-  SumAcc sa;
-  ArgAcc aa;
-  sa.init();
-  aa.init();
-  float m;
-  int arg = 0;
-  float s = 0.f;
-  if (sampling) {
-    row_slice_pass<true, false, VEC, E>(xr, c0, c1, c, sa, aa);
-    m = sa.m;
-    s = sa.value();
-    cta_reduce_sum(m, s, c, smf);
-  } else {
-    row_slice_pass<false, true, VEC, E>(xr, c0, c1, c, sa, aa);
-    m = aa.m;
-    arg = aa.arg;
-    cta_reduce_arg(m, arg, smf, smi);
-  }
+  cta_reduce_arg(m, arg, smf, smi);
   if (nsplit == 1) {
-    if (threadIdx.x == 0) {
-      RowStat st;
-      st.m = m;
-      st.arg = arg;
-      st.Z = (double)s;
-      stat[row] = st;
-    }
+    if (threadIdx.x == 0) node_arg[row] = arg;
     return;
   }
   if (threadIdx.x == 0) {
     RowPartial p;
     p.m = m;
     p.arg = arg;
-    p.s = (double)s;
+    p.s = 0.0;
     part[(size_t)row * kRowMaxSplits + split] = p;
     __threadfence();
     const uint32_t ticket = atomicAdd(&cnt[row], 1u);
@@ -77,15 +36,34 @@ __global__ void __launch_bounds__(kRowThreads) tree_argmax_kernel(
   float M;
   int A;
   double Z;
-  warp_merge_partials(part + (size_t)row * kRowMaxSplits, nsplit, sampling ? c : 0.f, !sampling, M, A, Z);
+  warp_merge_partials(part + (size_t)row * kRowMaxSplits, nsplit, 0.f, true, M, A, Z);
   if (threadIdx.x == 0) {
-    RowStat st;
-    st.m = M;
-    st.arg = sampling ? 0 : A;
-    st.Z = Z;
-    stat[row] = st;
+    node_arg[row] = A;
     cnt[row] = 0u;
   }
+}
+
+// Every sequence greedy: the rows' argmaxes.
+template <bool VEC, typename E>
+__global__ void __launch_bounds__(kRowThreads) tree_argmax_kernel(
+    const E* __restrict__ target, const int32_t* __restrict__ Ls, int K, int V, int nsplit, int chunk,
+    RowPartial* __restrict__ part, uint32_t* __restrict__ cnt, int32_t* __restrict__ node_arg,
+    int* __restrict__ status) {
+  const int split = blockIdx.x, j = blockIdx.y, b = blockIdx.z;
+  const int Lb = Ls[b];
+  if (Lb < 0 || Lb > K) {
+    if (split == 0 && j == 0 && threadIdx.x == 0) raise_status(status, LIBRASPEC_ST_BAD_LENGTH);
+    return;
+  }
+  if (j > Lb) return;
+  const int row = b * (K + 1) + j;
+  const int c0 = split * chunk, c1 = min(V, c0 + chunk);
+  SumAcc sa;
+  ArgAcc aa;
+  sa.init();
+  aa.init();
+  row_slice_pass<false, true, VEC, E>(target + (size_t)row * V, c0, c1, 1.f, sa, aa);
+  tree_row_finish(aa.m, aa.arg, row, split, nsplit, part, cnt, node_arg);
 }
 
 // ---------------------------------------------------------------------------
@@ -842,24 +820,21 @@ __global__ void selftest_wait_kernel(const uint32_t* __restrict__ flag, uint64_t
 }
 
 // ---------------------------------------------------------------------------
-// Per-node draws of a draft tree. Grid (nsplit, N+1, B); nodes t > L_b exit
-// at once. A greedy sequence (temperature 0) takes the argmax of the node's
-// target row; a sampling one draws from softmax(row / T) by the exponential
-// race x = argmin_v key_v, key_v = log2(E_v) - y_v log2(e) / T, E_v = -ln u_v,
-// u_v from Philox at (v >> 2, node t, sequence, purpose 2), word v & 3
-// (race_slice). The race is carried as an argmax of -key so the partials
-// merge like argmaxes (lowest index on ties).
-// The draw of node t lands in stat[b, t].arg for the walk.
+// Per-node draws of a draft tree (the same grid). A greedy sequence
+// (temperature 0) takes the argmax of the node's target row; a sampling one
+// draws from softmax(row / T) by the exponential race x = argmin_v key_v,
+// key_v = log2(E_v) - y_v log2(e) / T, E_v = -ln u_v, u_v from Philox at
+// (v >> 2, node t, sequence, purpose 2), word v & 3 (race_slice). The race is
+// carried as an argmax of -key so the partials merge like argmaxes (lowest
+// index on ties).
 // ---------------------------------------------------------------------------
 template <bool VEC, typename E>
 __global__ void __launch_bounds__(kRowThreads, 4) tree_rows_kernel(
     const E* __restrict__ target, const int32_t* __restrict__ Ls, const float* __restrict__ temperature, int K,
     int V, int nsplit, int chunk, uint64_t seed, uint64_t round_offset, uint32_t seq_offset,
-    RowPartial* __restrict__ part, uint32_t* __restrict__ cnt, RowStat* __restrict__ stat, int* __restrict__ status) {
-  __shared__ float smf[64];
-  __shared__ int smi[32];
+    RowPartial* __restrict__ part, uint32_t* __restrict__ cnt, int32_t* __restrict__ node_arg,
+    int* __restrict__ status) {
   __shared__ int s_thr;
-  __shared__ int last;
   const int split = blockIdx.x, j = blockIdx.y, b = blockIdx.z;
   const int Lb = Ls[b];
   if (Lb < 0 || Lb > K) {
@@ -894,51 +869,16 @@ __global__ void __launch_bounds__(kRowThreads, 4) tree_rows_kernel(
     m = -best;
     arg = besti;
   }
-  cta_reduce_arg(m, arg, smf, smi);
-  if (nsplit == 1) {
-    if (threadIdx.x == 0) {
-      RowStat st;
-      st.m = m;
-      st.arg = arg;
-      st.Z = 0.0;
-      stat[row] = st;
-    }
-    return;
-  }
-  if (threadIdx.x == 0) {
-    RowPartial p;
-    p.m = m;
-    p.arg = arg;
-    p.s = 0.0;
-    part[(size_t)row * kRowMaxSplits + split] = p;
-    __threadfence();
-    const uint32_t ticket = atomicAdd(&cnt[row], 1u);
-    last = (ticket == (uint32_t)(nsplit - 1));
-  }
-  __syncthreads();
-  if (!last || threadIdx.x >= 32) return;
-  __threadfence();
-  float M;
-  int A;
-  double Z;
-  warp_merge_partials(part + (size_t)row * kRowMaxSplits, nsplit, 0.f, true, M, A, Z);
-  if (threadIdx.x == 0) {
-    RowStat st;
-    st.m = M;
-    st.arg = A;
-    st.Z = 0.0;
-    stat[row] = st;
-    cnt[row] = 0u;
-  }
+  tree_row_finish(m, arg, row, split, nsplit, part, cnt, node_arg);
 }
 
 // ---------------------------------------------------------------------------
-// Greedy walk of a draft tree, one warp per sequence. Node t in [1, L_b] has
-// parent parent[b, t] < t and token tokens[b, t-1]. The warp first finds, for
-// every node p, its matching child next[p]: the lowest-numbered child whose
-// token is the argmax of p's target row (argmaxes from tree_argmax_kernel),
+// Walk of a draft tree, one warp per sequence. Node t in [1, L_b] has parent
+// parent[b, t] < t and token tokens[b, t-1]. The warp first finds, for every
+// node p, its matching child next[p]: the lowest-numbered child whose token is
+// p's (node_arg: its target row's argmax, or the draw of a sampling sequence),
 // by shared-memory atomicMin over the nodes; then it follows next[] from the
-// root. n = nodes walked, last = the final node, bonus = its argmax. A parent
+// root. n = nodes walked, last = the final node, bonus = its token. A parent
 // outside [0, t) or a token outside [0, V) never matches and raises its
 // status bit.
 // ---------------------------------------------------------------------------
@@ -947,16 +887,16 @@ constexpr int kWalkNodes = LIBRASPEC_MAX_TREE_NODES + 1;
 
 __global__ void __launch_bounds__(kWalkWarps * 32) tree_walk_kernel(
     const int32_t* __restrict__ tokens, const int32_t* __restrict__ parent, const int32_t* __restrict__ Ls, int B,
-    int K, int V, const RowStat* __restrict__ stat, int32_t* __restrict__ n_accepted,
+    int K, int V, const int32_t* __restrict__ node_arg, int32_t* __restrict__ n_accepted,
     int32_t* __restrict__ last_node, int32_t* __restrict__ bonus, int* __restrict__ status) {
   __shared__ int arg_s[kWalkWarps][kWalkNodes];
   __shared__ int next_s[kWalkWarps][kWalkNodes];
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // every node's draw is written
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every node's token is written
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * kWalkWarps + w;
   if (b >= B) return;
   const int Lb = Ls[b];
-  if (Lb < 0 || Lb > K) {  // tree_argmax_kernel raised the status
+  if (Lb < 0 || Lb > K) {  // the rows' kernel raised the status
     if (lane == 0) {
       n_accepted[b] = 0;
       if (last_node) last_node[b] = 0;
@@ -968,7 +908,7 @@ __global__ void __launch_bounds__(kWalkWarps * 32) tree_walk_kernel(
   int* next = next_s[w];
   constexpr int kNone = 0x7fffffff;
   for (int t = lane; t <= Lb; t += 32) {
-    const int a = __ldcg(&stat[(size_t)b * (K + 1) + t].arg);
+    const int a = __ldcg(node_arg + (size_t)b * (K + 1) + t);
     arg[t] = a == 0x7fffffff ? 0 : a;  // a row without a finite logit
     next[t] = kNone;
   }
@@ -1008,7 +948,7 @@ cudaError_t launch_accept_tree(const T* target, const int32_t* tokens, const int
   if (B == 0) return cudaSuccess;
   const int sms = num_sms_current();
   auto* st = reinterpret_cast<int*>(ws + lay.status);
-  auto* rstat = reinterpret_cast<RowStat*>(ws + lay.row_stat);
+  auto* node_arg = reinterpret_cast<int32_t*>(ws + lay.node_arg);
   const long rows = (long)B * (K + 1);
   // The draws' rows: as few slices as make one wave of resident CTAs (4 per SM), since a race settles its threshold
   // anew in each (2 trees of 257 nodes: 100 us at 16 CTAs per SM, 94 at 8, 90 at 4, 99 at 2); the argmax rows: more,
@@ -1023,17 +963,17 @@ cudaError_t launch_accept_tree(const T* target, const int32_t* tokens, const int
   const bool vec = rows_vectorizable(target, V);
   if (temperature == nullptr) {
     if (vec)
-      tree_argmax_kernel<true, T><<<grid, kRowThreads, 0, stream>>>(target, L, nullptr, K, V, nsplit, chunk, part,
-                                                                     cnt, rstat, st);
+      tree_argmax_kernel<true, T><<<grid, kRowThreads, 0, stream>>>(target, L, K, V, nsplit, chunk, part, cnt,
+                                                                     node_arg, st);
     else
-      tree_argmax_kernel<false, T><<<grid, kRowThreads, 0, stream>>>(target, L, nullptr, K, V, nsplit, chunk, part,
-                                                                      cnt, rstat, st);
+      tree_argmax_kernel<false, T><<<grid, kRowThreads, 0, stream>>>(target, L, K, V, nsplit, chunk, part, cnt,
+                                                                      node_arg, st);
   } else if (vec) {
     tree_rows_kernel<true, T><<<grid, kRowThreads, 0, stream>>>(target, L, temperature, K, V, nsplit, chunk, seed,
-                                                                 round_offset, seq_offset, part, cnt, rstat, st);
+                                                                 round_offset, seq_offset, part, cnt, node_arg, st);
   } else {
     tree_rows_kernel<false, T><<<grid, kRowThreads, 0, stream>>>(target, L, temperature, K, V, nsplit, chunk, seed,
-                                                                  round_offset, seq_offset, part, cnt, rstat, st);
+                                                                  round_offset, seq_offset, part, cnt, node_arg, st);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -1047,7 +987,7 @@ cudaError_t launch_accept_tree(const T* target, const int32_t* tokens, const int
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tree_walk_kernel, tokens, parent, L, B, K, V, (const RowStat*)rstat, n_accepted,
+  return cudaLaunchKernelEx(&cfg, tree_walk_kernel, tokens, parent, L, B, K, V, (const int32_t*)node_arg, n_accepted,
                             last_node, bonus, st);
 }
 template cudaError_t launch_accept_tree<float>(const float*, const int32_t*, const int32_t*, const int32_t*,

@@ -35,17 +35,6 @@ struct RowPartial {      // one CTA's share of a logit row
 };
 static_assert(sizeof(RowPartial) == 16, "a partial is read as one 16-byte load");
 
-struct RowStat {         // merged statistics of a target row
-  float m;
-  int arg;
-  double Z;
-};
-
-struct RacePartial {
-  float key;
-  int idx;
-};
-
 // A race candidate carried without the row's normaliser: the key of token v
 // is E_v * 2^(-y_v c) (E_v = -ln u_v, c = log2(e) / T), compared between two
 // candidates as E_a < E_b * 2^((y_a - y_b) c).
@@ -69,7 +58,7 @@ struct ResEntry {
 };
 
 struct WsLayout {
-  size_t status, conf_part, conf_cnt, seq_cnt, row_part, row_cnt, row_stat, race_part, race_cnt;
+  size_t status, conf_part, conf_cnt, seq_cnt, row_part, row_cnt, node_arg, race_part, race_cnt;
   size_t acc_seq, acc_yx, acc_res, acc_ready, acc_plan;
   size_t attn_o, attn_ml, attn_cnt, attn_grp, tree_vis, total;
   int max_items, max_groups;
@@ -95,7 +84,7 @@ inline WsLayout ws_layout(int B, int K, int V, int Hq, int Hkv, int d, int S_cap
   w.seq_cnt = take(size_t(B) * sizeof(uint32_t));  // rows of a sequence done (fused selection)
   w.row_part = take(rows_t * kRowMaxSplits * sizeof(RowPartial));
   w.row_cnt = take(rows_t * sizeof(uint32_t));
-  w.row_stat = take(rows_t * sizeof(RowStat));
+  w.node_arg = take(rows_t * sizeof(int32_t));  // (trees) each node row's argmax or draw
   w.race_part = take(size_t(B) * kRaceMaxSplits * sizeof(RaceCand));
   w.race_cnt = take(size_t(B) * sizeof(uint32_t));
   // acceptance: slices done per sequence, the target logit at each drafted
