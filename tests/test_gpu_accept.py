@@ -196,6 +196,7 @@ def test_races_on_flat_steep_and_short_rows(orc, dtype, V, scale, T):
     n_ref, b_ref, flag = _oracle_accept(orc, wide, L, 77, round_offset=2)
     assert_exact_unless_flagged(n, n_ref, flag, "n_accepted")
     assert_exact_unless_flagged(bonus, b_ref, flag, "bonus_token")
+    assert_flag_budget(int((flag != 0).sum()), B, "chain")
     par = torch.from_numpy(workloads.draft_tree(B, K, K, 5, "random")).to(cuda())
     L_t = torch.full((B,), K, dtype=torch.int32, device=cuda())
     ws = lr.Workspace(B, K, V, device=cuda())
@@ -206,6 +207,7 @@ def test_races_on_flat_steep_and_short_rows(orc, dtype, V, scale, T):
                                  L_t.cpu().numpy(), temp.cpu().numpy(), 78, 3)
     for a, r, what in zip(out, ref, ("n_accepted", "last_node", "bonus_token")):
         assert_exact_unless_flagged(a.cpu().numpy(), r, flag, what)
+    assert_flag_budget(int((flag != 0).sum()), B, "tree")
 
 
 @pytest.mark.parametrize("B,K,V", [(1, 1, 300), (31, 4, 2049), (255, 2, 2048), (256, 64, 130), (257, 3, 2051)])
@@ -236,3 +238,4 @@ def test_accept_plan_edges(orc, B, K, V):
     good = np.setdiff1d(np.arange(B), bad)
     assert_exact_unless_flagged(n[good], n_ref[good], flag[good], "n_accepted")
     assert_exact_unless_flagged(bonus[good], b_ref[good], flag[good], "bonus_token")
+    assert_flag_budget(int((flag[good] != 0).sum()), len(good), "plan")

@@ -95,3 +95,61 @@ def test_host_buffer_api_round_trip(orc, in_place):
     np.testing.assert_array_equal(bonus, b_ref)
     O_ref, lse_ref = orc.verify_attn(lay["Q"], lay["Kc"], lay["Vc"], kv, L)
     check_attn(runner.out.O[0], None, O_ref, lse_ref, L)
+
+
+@pytest.mark.parametrize("B,K,V,n_layers,temps", [(16, 8, 128256, 2, (0.0,)), (16, 8, 32003, 2, (0.0, 0.8, 1.0)),
+                                                  (3, 4, 4104, 0, (1.0, 0.0)), (257, 2, 2050, 1, (0.0, 0.7))])
+def test_captured_round_equals_the_eager_one(B, K, V, n_layers, temps):
+    """The round's launches (cooperative attention, rows and draws as dependent launches; above 256 sequences the
+    plan as a launch) captured into a graph and replayed on new inputs: what a copy behind the draws sees, and every
+    output, is bit for bit that of the eager call. With greedy sequences alone the draws end before their rows."""
+    Hq, Hkv, d, kv_hi = 8, 2, 64, 300
+    S = kv_hi + K + 1
+    kv = torch.from_numpy(np.random.default_rng(B).integers(1, kv_hi + 1, B).astype(np.int32)).to(cuda())
+    temp = torch.tensor([temps[i % len(temps)] for i in range(B)], device=cuda())
+    cost = torch.tensor([1.0 + 0.01 * t for t in range(K + 1)], device=cuda())
+
+    def inputs(seed):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        target = torch.randn((B, K + 1, V), generator=g, device=cuda()) * 4
+        draft = target[:, :K] + torch.randn((B, K, V), generator=g, device=cuda()) * 0.5
+        bufs = [draft, draft.argmax(-1).int(), target]
+        for _ in range(n_layers):
+            bufs += [torch.randn(s, generator=g, device=cuda()).to(torch.bfloat16)
+                     for s in ((B, K + 1, Hq, d), (B, Hkv, S, d), (B, Hkv, S, d))]
+        return bufs
+
+    def run(bufs, ws, outputs=None):
+        layers = [dict(zip(("Q", "Kc", "Vc"), bufs[3 + 3 * l:6 + 3 * l])) for l in range(n_layers)]
+        return lr.libraspec_verify_round(bufs[0], bufs[1], temp, cost, bufs[2], layers, kv, 5, ws, round_offset=3,
+                                         outputs=outputs, want_lse=n_layers > 0)
+
+    shape = (B, K, V) + ((Hq, Hkv, d, S) if n_layers else ())
+    ws, ws_ref = lr.Workspace(*shape, device=cuda()), lr.Workspace(*shape, device=cuda())
+    bufs = inputs(0)
+    out = run(bufs, ws)
+    seen = torch.empty((2, B), dtype=torch.int32, device=cuda())
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run(bufs, ws, outputs=out)
+        seen[0].copy_(out.n_accepted)
+        seen[1].copy_(out.bonus_token)
+    for seed in range(1, 5):
+        new = inputs(seed)
+        for a, b in zip(bufs, new):
+            a.copy_(b)
+        for t in [out.conf, out.dstat, out.L, out.n_accepted, out.bonus_token, seen] + out.O + (out.lse or []):
+            t.fill_(7)
+        graph.replay()
+        graph.replay()  # (the workspace is left as it was found)
+        ref = run(new, ws_ref)
+        torch.cuda.synchronize()
+        assert lr.libraspec_get_status(ws) == 0 and lr.libraspec_get_status(ws_ref) == 0
+        for name in ("conf", "dstat", "L", "n_accepted", "bonus_token"):
+            assert torch.equal(getattr(out, name), getattr(ref, name)), name
+        assert torch.equal(seen[0], ref.n_accepted) and torch.equal(seen[1], ref.bonus_token)
+        for l in range(n_layers):
+            for b, n in enumerate((ref.L + 1).tolist()):
+                assert torch.equal(out.O[l][b, :n], ref.O[l][b, :n])
+                assert torch.equal(out.lse[l][b, :n], ref.lse[l][b, :n])
