@@ -104,11 +104,17 @@ def _check(rc: int, what: str) -> None:
         raise LibraspecError(what, rc)
 
 
+# The current stream's handle without making a Stream object (3.0 us -> 0.5); not a public function of torch.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
-    """The handle of the stream, or of the current one (read without making a Stream object: 3.0 us -> 0.5)."""
-    if stream is not None:
-        return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    """The handle of the stream, or of the current one."""
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
+    return stream.cuda_stream
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

@@ -133,3 +133,13 @@ def test_argument_checks_name_what_is_wrong(t, dtype, shape, error):
         lr._req(t, dtype, "x", shape)
     with pytest.raises((TypeError, ValueError), match=r"^Q\[0\] "):
         lr._check_layers([{"Q": t, "K": t, "V": t}], "K", "V", (2,), (2,))
+
+
+def test_current_stream_without_the_raw_handle(monkeypatch):
+    """A torch without the private handle function: the current stream is asked in the public way."""
+    class Stream:
+        cuda_stream = 7
+
+    monkeypatch.setattr(lr, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    assert lr._stream(None) == 7 and lr._stream(Stream()) == 7
