@@ -190,8 +190,8 @@ __device__ __forceinline__ float warp_fmin(float x) {
 // rounding of the test, so every possible winner passes.
 // Before (each token tested with two exponentials, exact steps whenever a
 // lane of the warp passed): 70 instructions per token; 2 trees of 257 nodes,
-// V = 152064, bf16: 148 us; now 23 instructions, 90 us (the integer
-// multiplies alone: 36 us).
+// V = 152064, bf16: 148 us; now 23 instructions, 87 us (the Philox blocks by
+// themselves: 50 us).
 // Loads run two trips ahead of the eight logits in use (two Philox blocks and
 // one copy of the exact step per trip: short code, and two chains to
 // interleave); the trip counts are the warp's, so that every lane joins the

@@ -23,9 +23,9 @@
 // softmax warpgroup over 64-key tiles was the limit before: with few rows one
 // warp holds them all, and its 1150 cycles per 64-key tile did not keep up
 // with HBM, and large trees left the tensor cores idle three quarters of the
-// time. 8 sequences of 131072 keys (64/8 heads): 771 -> 606 us (104% of the
-// copy rate); B = 64 ragged: 326 -> 285; 32 layers at B = 1: 302 -> 230; a
-// 512-node tree, 4 layers: 367 -> 221 (with what is said below).
+// time. 8 sequences of 131072 keys (64/8 heads): 771 -> 602 us (105% of the
+// copy rate); B = 64 ragged: 326 -> 286; 32 layers at B = 1: 302 -> 234; a
+// 512-node tree, 4 layers: 367 -> 220 (with what is said below).
 //
 // Roles in a CTA (384 threads):
 //  * producer warp: walks the CTA's range layer after layer in items; loads
@@ -272,10 +272,17 @@ __device__ TileLoc find_tile(long long x, int C, long long T, int B, const int32
 // sequence, or equal caches) and the NG groups fit the grid, each group may
 // get p = G / NG CTAs of its own: no CTA has two items, and a group of p = 1
 // is never split nor merged. Taken when the longest range, nt / p tiles, is
-// at most kAlignTiles above the even split's T / G (an extra item and its
-// merge cost a CTA about that much). 512 nodes (136 groups of 128 rows, 4
-// layers): 227 us; cut by cost, 353; with row groups of 256 rows, which read
-// each tile once for both halves but are split and merged, 320.
+// at most kAlignTiles above the even split's T / G: what a group cut at any
+// tile costs is an extra item per CTA and a merge of parts of unequal length,
+// the more the more rows it has. Over 56 shapes of equal groups (trees of 64
+// to 512 nodes, 1 to 36 sequences of 500 to 32000 keys, graphs of 2 to 8
+// layers) the rule gains 1 to 48% where it applies against the cut by cost
+// and loses nowhere: 512 nodes (136 groups of 128 rows, 4 layers) 213 us
+// against 245, 100 nodes 89 against 121, 16 sequences of 1500 keys 46 against
+// 56, 8 of 4096 (5.6 tiles above) 61 against 63. Between 10 and 20 tiles above
+// it would still gain mostly (500 nodes 209 against 241, 20 sequences of 28/4
+// heads 61.7 against 60.6), from 24 on it loses (10 sequences of 4096: 84
+// against 72).
 constexpr int kAlignTiles = 10;
 __device__ __forceinline__ int aligned_ctas(long long T, long long NG, int nt, int G) {
   if (nt <= 0 || NG > G) return 0;
@@ -395,7 +402,7 @@ __device__ __forceinline__ int merge_share(const MergeTask& t, int& u0) {
   return (int)((long long)t.rows * (k_me + 1) / t.np) - u0;
 }
 
-constexpr int kMergeLoads = 12;  // of a lane in flight (16 spill registers)
+constexpr int kMergeLoads = 12;  // of a lane in flight (with 16, registers spill)
 
 // Items per lane in a chunk of a group of np parts: J items x 12/J parts are
 // in flight per batch, and a share of `items` items costs ceil(items / 32J)

@@ -10,10 +10,10 @@
 // on the MMA's M side (256 head rows over the pair, 128 per CTA) and the rows
 // of H on its N side (up to 256, split between the two CTAs), so a k-slab of
 // 64 brings 16 KB of W and N x 64 bytes of H into each CTA. At N = 256 that
-// is 64 bytes per cycle and SM at the tensor peak, which L2 sustains (1180 us
-// for 2112 rows over V = 128256, Dm = 4096: 1.88 PFLOP/s; 1320 back to back,
-// at the power limit); single-CTA tiles of 128 x 128 need twice the bytes and
-// were bound by them (1920 us). The time
+// is 64 bytes per cycle and SM at the tensor peak, which L2 sustains (2112 rows
+// over V = 128256, Dm = 4096: 1160 us in 20 calls, 1.91 PFLOP/s; 1335 to 1385
+// over seconds of calls, at the power limit); single-CTA tiles of 128 x 128
+// need twice the bytes and were bound by them (1920 us over seconds). The time
 // of a tile follows its operand bytes, 256 + N (N = 64: 96 us per row tile
 // of that head, 128: 103, 192: 119, 256: 141), so rows are cut into as few
 // tiles as 256 allows, of sizes that differ by 32 at most.
@@ -24,14 +24,16 @@
 //    walks its own contiguous V / pairs columns, whose last tile is cut short,
 //    so no pair streams more than its share (whole tiles of 256 leave 6.6
 //    tiles per pair, a loss of 6%); its rows' statistics stay in registers
-//    from tile to tile and leave one partial per (row, CTA).
+//    from tile to tile, the sum as two floats, and leave one partial per
+//    (row, CTA).
 //
 // Roles (192 threads): warp 4 streams W and H k-slabs (128-byte swizzle) by
 // TMA into a ring of stages, each CTA its half, counted on the leader's
 // barrier; warp 5 of the leader issues tcgen05.mma into one of two
 // accumulators (lane = head column, column = row of H); warps 0-3 turn 32 x 32
 // blocks of an accumulator through shared memory, so that a thread holds one
-// row's 32 logits, reduce them, and combine the four warps' shares. Rows past
+// row's 32 logits, reduce them, and combine the four warps' shares (a wait
+// that runs out is the verdict of all four: they meet at named barriers). Rows past
 // M and columns past V come from the TMA's zero fill (or are never loaded)
 // and are left out of the statistics.
 #include <cmath>
@@ -74,9 +76,10 @@ __device__ __forceinline__ void lm_exponent(float m, float mx, float c, float& x
   xl = __fmaf_rn(dl, c, __fmaf_rn(d, c, -xh));
 }
 
-// (h + l) 2^n = 2^(xh + xl) for xh in [-1000, 0] (below, h = l = 0), within 2^-39 of it: the argument is cut at the
-// nearest multiple of 1/32, whose power comes from the table, and the rest g = f ln 2, |g| < 0.011, goes through
-// the Taylor series of e^g, whose first three terms are carried in two floats.
+// (h + l) 2^n = 2^(xh + xl) for xh in [-1000, 0] (below, h = l = 0), within 2^-39 of it, by Tang's table-driven method
+// (ACM Trans. Math. Softw. 15, 1989): the argument is cut at the nearest multiple of 1/32, whose power comes from the
+// table, and the rest g = f ln 2, |g| < 0.011, goes through the Taylor series of e^g, whose first three terms are
+// carried in two floats.
 __device__ __forceinline__ void lm_exp2(float xh, float xl, const float2* table, float& h, float& l, int& n) {
   if (xh < -1000.f) {
     h = l = 0.f;
@@ -228,7 +231,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
     if (lane == 0) {
       // One row tile: the head passes through L2 once, ahead of H and the code (64 rows over V = 32896, Dm = 2048:
       // 39.8 -> 34.1 us). Several: its tiles are read again by the other row tiles, so they keep the usual priority
-      // (2112 rows: 1277 us, evict first 1597).
+      // (2112 rows, over seconds of calls: 1277 us, evict first 1597).
       const uint64_t policy = cut.row_tiles == 1 ? evict_first_policy() : evict_normal_policy();
       const uint64_t keep = cut.row_tiles == 1 ? evict_last_policy() : evict_normal_policy();
       uint32_t s = 0, ph = 0;
@@ -415,12 +418,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kLmThreads, 1) lm_he
 }
 
 // One CTA per row, a programmatic dependent launch: Z = sum_n z_n 2^((m_n - m) c); the argmax is the first column
-// of the largest max; the token probability is 2^((x_tok - m) c) / Z. What bounds it: the powers. In binary64 (a
-// sixty-fourth of the rate), a warp per row, this launch took 9 us of 37 (128 rows over V = 32896, Dm = 2048) and 100 of
-// 1320 (2112 rows over V = 128256, Dm = 4096), so terms and sum are carried in two floats each (2^-39, against the
-// 2^-22 of the terms of z_n) and the last steps in binary64: 31 and 1270 us in all. The launch of the tiles gives no early
-// signal: a merge that may start beside the tiles puts all of its CTAs on the few SMs without one and took 66 us
-// for those 128 rows.
+// of the largest max; the token probability is 2^((x_tok - m) c) / Z, x_tok left in its place by the tiles. What
+// bounds it: the powers. In binary64 (a sixty-fourth of the rate), a warp per row, this launch took 9 us of 37 (128
+// rows over V = 32896, Dm = 2048) and 100 of 1320 (2112 rows over V = 128256, Dm = 4096), so terms and sum are carried
+// in two floats each (2^-39, against the 2^-22 of the terms within z_n) and the last steps in binary64: both launches
+// then took 31 and 1270 us. The launch of the tiles gives no early signal: a merge that may start beside the tiles
+// puts all of its CTAs on the few SMs without one and took 66 us for those 128 rows.
 // A token outside [-1, V) sets LIBRASPEC_ST_BAD_TOKEN (probability NaN).
 constexpr int kMergeThreads = 128;
 __global__ void __launch_bounds__(kMergeThreads) lm_head_merge_kernel(
